@@ -83,7 +83,9 @@ __device__ __forceinline__ void rand4(uint32_t k0, uint32_t k1, uint32_t pix, ui
 }
 
 // ---------------------------------------------------------------------------
-// FP32 vectors
+// FP32 vectors.  Wherever a product feeds a sum the code says whether the two
+// are fused: left to the compiler, that choice moves with register pressure,
+// and the kernels would no longer agree with one another bit for bit.
 // ---------------------------------------------------------------------------
 struct f3 {
     float x, y, z;
@@ -93,15 +95,27 @@ __device__ __forceinline__ f3 operator+(f3 a, f3 b) { return mk3(a.x + b.x, a.y 
 __device__ __forceinline__ f3 operator-(f3 a, f3 b) { return mk3(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ __forceinline__ f3 operator*(f3 a, float s) { return mk3(a.x * s, a.y * s, a.z * s); }
 __device__ __forceinline__ f3 operator*(f3 a, f3 b) { return mk3(a.x * b.x, a.y * b.y, a.z * b.z); }
-__device__ __forceinline__ float dot(f3 a, f3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+// a0 b0 + a1 b1 and a0 b0 - a1 b1 with one product rounded on its own
+__device__ __forceinline__ float sum2(float a0, float b0, float a1, float b1) { return fmaf(a0, b0, __fmul_rn(a1, b1)); }
+__device__ __forceinline__ float diff2(float a0, float b0, float a1, float b1) {
+    return fmaf(a0, b0, -__fmul_rn(a1, b1));
+}
+__device__ __forceinline__ float dot(f3 a, f3 b) { return fmaf(a.z, b.z, sum2(a.x, b.x, a.y, b.y)); }
 __device__ __forceinline__ f3 cross(f3 a, f3 b) {
-    return mk3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
+    return mk3(diff2(a.y, b.z, a.z, b.y), diff2(a.z, b.x, a.x, b.z), diff2(a.x, b.y, a.y, b.x));
+}
+// the same product sum with y rounded into x's place
+__device__ __forceinline__ float dot_yx(f3 a, f3 b) { return fmaf(a.z, b.z, sum2(a.y, b.y, a.x, b.x)); }
+// a + b s
+__device__ __forceinline__ f3 madd(f3 a, f3 b, float s) { return mk3(fmaf(b.x, s, a.x), fmaf(b.y, s, a.y), fmaf(b.z, s, a.z)); }
+// a x + b y + c z
+__device__ __forceinline__ f3 combine(f3 a, float x, f3 b, float y, f3 c, float z) {
+    return mk3(fmaf(c.x, z, sum2(a.x, x, b.x, y)), fmaf(c.y, z, sum2(a.y, x, b.y, y)), fmaf(c.z, z, sum2(a.z, x, b.z, y)));
 }
 __device__ __forceinline__ f3 normalize(f3 a) { return a * (1.0f / sqrtf(dot(a, a))); }
 __device__ __forceinline__ f3 xyz(float4 v) { return mk3(v.x, v.y, v.z); }
 __device__ __forceinline__ f3 mat3v(const float *M, f3 v) {
-    return mk3(M[0] * v.x + M[1] * v.y + M[2] * v.z, M[3] * v.x + M[4] * v.y + M[5] * v.z,
-               M[6] * v.x + M[7] * v.y + M[8] * v.z);
+    return mk3(dot(mk3(M[0], M[1], M[2]), v), dot(mk3(M[3], M[4], M[5]), v), dot(mk3(M[6], M[7], M[8]), v));
 }
 
 // ---------------------------------------------------------------------------
@@ -120,8 +134,8 @@ __device__ __forceinline__ float alpha_of(float r, float &dadr) {
 // cos^2 (a^2 - 1) + 1 is formed as s2 + a^2 cos^2 with s2 = |n x h|^2: the
 // textbook form cancels catastrophically in FP32 near the peak of sharp lobes.
 __device__ __forceinline__ float ggx_D(float ch, float s2, float a) {
-    const float a2 = a * a;
-    const float t = s2 + a2 * ch * ch;
+    const float a2 = __fmul_rn(a, a);
+    const float t = fmaf(a2 * ch, ch, s2);
     return a2 / (DPCS_PI_F * t * t);
 }
 __device__ __forceinline__ float sin2(f3 n, f3 h) {
@@ -130,27 +144,27 @@ __device__ __forceinline__ float sin2(f3 n, f3 h) {
 }
 
 __device__ __forceinline__ float ggx_G1(float c, float a) {
-    const float a2 = a * a;
-    return 2.0f * c / (c + sqrtf(a2 + (1.0f - a2) * c * c));
+    const float a2 = __fmul_rn(a, a);
+    return 2.0f * c / (c + sqrtf(fmaf((1.0f - a2) * c, c, a2)));
 }
 
 // ks * D G F / (4 ci co) and its derivative in roughness r (0 if ks == 0)
 __device__ __forceinline__ float spec_eval(f3 n, f3 wo, f3 wi, float r, float ks, float f0, float &dspec_dr) {
     dspec_dr = 0.0f;
-    const float co = dot(n, wo), ci = dot(n, wi);
+    const float co = dot_yx(n, wo), ci = dot(n, wi);
     if (ks <= 0.0f || co <= 0.0f || ci <= 0.0f) return 0.0f;
     float dadr;
     const float a = alpha_of(r, dadr);
     const f3 h = normalize(wo + wi);
     const float ch = dot(n, h);
-    const float a2 = a * a;
-    const float t = sin2(n, h) + a2 * ch * ch;
+    const float a2 = __fmul_rn(a, a), b2 = (1.0f - a2);
+    const float t = fmaf(a2 * ch, ch, sin2(n, h));
     const float D = a2 / (DPCS_PI_F * t * t);
-    const float si = sqrtf(a2 + (1.0f - a2) * ci * ci), so = sqrtf(a2 + (1.0f - a2) * co * co);
+    const float si = sqrtf(fmaf(b2 * ci, ci, a2)), so = sqrtf(fmaf(b2 * co, co, a2));
     const float G = (2.0f * ci / (ci + si)) * (2.0f * co / (co + so));
-    float m = fmaxf(0.0f, 1.0f - dot(wo, h));
+    float m = fmaxf(0.0f, 1.0f - dot_yx(wo, h));
     const float m2 = m * m;
-    const float F = f0 + (1.0f - f0) * (m2 * m2 * m);
+    const float F = fmaf(1.0f - f0, m2 * m2 * m, f0);
     const float spec = ks * D * G * F / (4.0f * ci * co);
     const float dlnD = 2.0f / a - 4.0f * a * ch * ch / t;
     const float dlnG = -(a * (1.0f - ci * ci) / si) / (ci + si) - (a * (1.0f - co * co) / so) / (co + so);
@@ -165,14 +179,19 @@ __device__ __forceinline__ void onb(f3 n, f3 &t, f3 &b) {
     const float sg = n.z >= -DPCS_INV_PI_F ? 1.0f : -1.0f;
     const float a = -1.0f / (sg + n.z);
     const float bb = n.x * n.y * a;
-    t = mk3(1.0f + sg * n.x * n.x * a, sg * bb, -sg * n.x);
-    b = mk3(bb, sg + n.y * n.y * a, -n.y);
+    t = mk3(fmaf(sg * n.x * n.x, a, 1.0f), sg * bb, -sg * n.x);
+    b = mk3(bb, fmaf(n.y * n.y, a, sg), -n.y);
+}
+
+// rho / pi + spec per channel
+__device__ __forceinline__ f3 lambert_plus(f3 rho, float spec) {
+    return mk3(fmaf(rho.x, DPCS_INV_PI_F, spec), fmaf(rho.y, DPCS_INV_PI_F, spec), fmaf(rho.z, DPCS_INV_PI_F, spec));
 }
 
 __device__ __forceinline__ float spec_prob(float ks) { return ks > 0.0f ? 0.5f : 0.0f; }
 
 __device__ __forceinline__ float bsdf_pdf(f3 n, f3 wo, f3 wi, float r, float ks) {
-    const float ci = dot(n, wi), co = dot(n, wo);
+    const float ci = dot(n, wi), co = dot_yx(n, wo);
     if (ci <= 0.0f || co <= 0.0f) return 0.0f;
     const float ps = spec_prob(ks);
     float p = (1.0f - ps) * ci * DPCS_INV_PI_F;
@@ -180,7 +199,8 @@ __device__ __forceinline__ float bsdf_pdf(f3 n, f3 wo, f3 wi, float r, float ks)
         float dadr;
         const float a = alpha_of(r, dadr);
         const f3 h = normalize(wo + wi);
-        p += ps * ggx_G1(co, a) * ggx_D(dot(n, h), sin2(n, h), a) / (4.0f * co);
+        const float q = ps * ggx_G1(co, a) * ggx_D(dot(n, h), sin2(n, h), a) / (4.0f * co);
+        p = fmaf((1.0f - ps) * ci, DPCS_INV_PI_F, q);
     }
     return p;
 }
@@ -199,21 +219,21 @@ __device__ __forceinline__ bool bsdf_sample(f3 n, f3 wo, float r, float ks, floa
     } else {
         float dadr;
         const float a = alpha_of(r, dadr);
-        const f3 wl = mk3(dot(wo, T), dot(wo, B), dot(wo, n));
+        const f3 wl = mk3(dot_yx(wo, T), dot_yx(wo, B), dot_yx(wo, n));
         const f3 Vh = normalize(mk3(a * wl.x, a * wl.y, wl.z));
-        const float lsq = Vh.x * Vh.x + Vh.y * Vh.y;
+        const float lsq = sum2(Vh.x, Vh.x, Vh.y, Vh.y);
         const f3 T1 = lsq > 0.0f ? mk3(-Vh.y, Vh.x, 0.0f) * (1.0f / sqrtf(lsq)) : mk3(1.0f, 0.0f, 0.0f);
         const f3 T2 = cross(Vh, T1);
         const float rr = sqrtf(u1);
-        const float t1 = rr * cp;
-        float t2 = rr * sp;
-        const float s = 0.5f * (1.0f + Vh.z);
-        t2 = (1.0f - s) * sqrtf(fmaxf(0.0f, 1.0f - t1 * t1)) + s * t2;
-        const f3 Nh = T1 * t1 + T2 * t2 + Vh * sqrtf(fmaxf(0.0f, 1.0f - t1 * t1 - t2 * t2));
+        const float t1 = __fmul_rn(rr, cp);
+        float t2 = __fmul_rn(rr, sp);
+        const float s = 0.5f * (1.0f + Vh.z), w1 = fmaf(-t1, t1, 1.0f);
+        t2 = sum2(1.0f - s, sqrtf(fmaxf(0.0f, w1)), s, t2);
+        const f3 Nh = combine(T1, t1, T2, t2, Vh, sqrtf(fmaxf(0.0f, fmaf(-t2, t2, w1))));
         const f3 Ne = normalize(mk3(a * Nh.x, a * Nh.y, fmaxf(0.0f, Nh.z)));
-        l = Ne * (2.0f * dot(wl, Ne)) - wl;
+        l = madd(wl * -1.0f, Ne, 2.0f * dot(wl, Ne));
     }
-    wi = T * l.x + B * l.y + n * l.z;
+    wi = combine(T, l.x, B, l.y, n, l.z);
     return dot(n, wi) > 0.0f;
 }
 
@@ -224,8 +244,8 @@ struct Bilin {
     int x0, y0;
     float fx, fy;
 };
-__device__ __forceinline__ Bilin bilin_setup(float xp, float yp, int W, int H) {
-    float x = xp - 0.5f, y = yp - 0.5f;
+// (x, y): the position less (1/2, 1/2)
+__device__ __forceinline__ Bilin bilin_setup(float x, float y, int W, int H) {
     x = fminf(fmaxf(x, -1.0f), (float)W);
     y = fminf(fmaxf(y, -1.0f), (float)H);
     const float fx0 = floorf(x), fy0 = floorf(y);
@@ -256,10 +276,10 @@ __device__ __forceinline__ float4 bilin_fetch(const float4 *__restrict__ img, co
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float4 v = __ldg(img + idx[k]);
-        r.x += w[k] * v.x;
-        r.y += w[k] * v.y;
-        r.z += w[k] * v.z;
-        r.w += w[k] * v.w;
+        r.x = fmaf(w[k], v.x, r.x);
+        r.y = fmaf(w[k], v.y, r.y);
+        r.z = fmaf(w[k], v.z, r.z);
+        r.w = fmaf(w[k], v.w, r.w);
     }
     return r;
 }
@@ -642,15 +662,15 @@ __device__ __forceinline__ Surf surface_at(const RenderArgs &a, const Hit &h, f3
     const float4 V1 = __ldg(a.tris + 3 * h.pos + 1);
     const float4 V2 = __ldg(a.tris + 3 * h.pos + 2);
     const f3 e1 = xyz(V1) - xyz(A), e2 = xyz(V2) - xyz(A);
-    S.x = xyz(A) + e1 * h.u + e2 * h.v;
+    S.x = madd(madd(xyz(A), e1, h.u), e2, h.v);
     S.n = normalize(cross(e1, e2));
     if (dot(S.n, d) > 0.0f) S.n = S.n * -1.0f;
     const float2 t0 = __ldg(a.tuv + 3 * h.pos + 0), t1 = __ldg(a.tuv + 3 * h.pos + 1),
                  t2 = __ldg(a.tuv + 3 * h.pos + 2);
     const float w0 = 1.0f - h.u - h.v;
-    const float su = w0 * t0.x + h.u * t1.x + h.v * t2.x;
-    const float sv = w0 * t0.y + h.u * t1.y + h.v * t2.y;
-    S.tb = bilin_setup(su * (float)a.Wt, sv * (float)a.Ht, a.Wt, a.Ht);
+    const float su = fmaf(h.v, t2.x, sum2(w0, t0.x, h.u, t1.x));
+    const float sv = fmaf(h.v, t2.y, sum2(w0, t0.y, h.u, t1.y));
+    S.tb = bilin_setup(fmaf(su, (float)a.Wt, -0.5f), fmaf(sv, (float)a.Ht, -0.5f), a.Wt, a.Ht);
     const float4 tex = bilin_fetch(a.tex, S.tb, a.Wt, a.Ht);
     S.rho = mk3(tex.x, tex.y, tex.z);
     S.rough = tex.w;
@@ -682,16 +702,16 @@ __device__ __forceinline__ bool nee_prepare(const RenderArgs &a, const Surf &S, 
     const float cs = dot(S.n, wp);
     if (!(cs > 0.0f)) return false;
     const float cpz = X.z / sqrtf(dot(X, X));
-    N.so = S.x + S.n * kRayEps;
+    N.so = madd(S.x, S.n, kRayEps);
     const f3 sv = cp - N.so;
     const float sd = sqrtf(dot(sv, sv));
     N.sdir = sv * (1.0f / sd);
     N.smax = sd - kRayEps;
-    N.pb = bilin_setup(up, vp, a.Wp, a.Hp);
+    N.pb = bilin_setup(up - 0.5f, vp - 0.5f, a.Wp, a.Hp);
     N.ep = bilin_fetch(a.Ep, N.pb, a.Wp, a.Hp);
     N.G = a.k_proj * cpz * cs / r2;
     N.sp = spec_eval(S.n, S.wo, wp, S.rough, a.ks, a.f0, N.dsp);
-    N.fp = mk3(S.rho.x * DPCS_INV_PI_F + N.sp, S.rho.y * DPCS_INV_PI_F + N.sp, S.rho.z * DPCS_INV_PI_F + N.sp);
+    N.fp = lambert_plus(S.rho, N.sp);
     return true;
 }
 
@@ -727,8 +747,7 @@ __device__ __forceinline__ bool continue_prepare(const RenderArgs &a, uint32_t p
     }
     C.si = spec_eval(S.n, S.wo, C.wi, S.rough, a.ks, a.f0, C.dsi);
     C.cw = dot(S.n, C.wi) / (pdf * qrr);
-    const f3 fi = mk3(S.rho.x * DPCS_INV_PI_F + C.si, S.rho.y * DPCS_INV_PI_F + C.si,
-                      S.rho.z * DPCS_INV_PI_F + C.si);
+    const f3 fi = lambert_plus(S.rho, C.si);
     C.w = fi * C.cw;
     return true;
 }

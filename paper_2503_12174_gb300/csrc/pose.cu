@@ -289,7 +289,7 @@ __device__ void pose_trace(const RenderArgs &a, const float4 *__restrict__ mat, 
                         }
                     }
                     beta = beta * C.w;
-                    ext_o = S.x + S.n * kRayEps;
+                    ext_o = madd(S.x, S.n, kRayEps);
                     ext_d = C.wi;
                     has_ext = true;
                 }
@@ -339,7 +339,7 @@ __device__ void pose_trace(const RenderArgs &a, const float4 *__restrict__ mat, 
                         }
                     }
                     beta = beta * C.w;
-                    ext_o = S.x + S.n * kRayEps;
+                    ext_o = madd(S.x, S.n, kRayEps);
                     ext_d = C.wi;
                     has_ext = true;
                 }

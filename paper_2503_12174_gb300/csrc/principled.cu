@@ -336,9 +336,9 @@ __device__ __forceinline__ void pbr_lanes(const RenderArgs &a, const float4 *__r
                     // traversal) keeps the lane in phase with the others
                     shadow = true;
                     nulls = true;
-                    ray.o = S.x + S.n * kRayEps;
+                    ray.o = madd(S.x, S.n, kRayEps);
 #else
-                    ray = make_ray(S.x + S.n * kRayEps, ed);
+                    ray = make_ray(madd(S.x, S.n, kRayEps), ed);
                     ++b;
 #endif
                 } else {

@@ -20,6 +20,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "tile.cuh"
 
 namespace dpcs {
 
@@ -124,6 +125,20 @@ __global__ void k_pack_tex(const float *__restrict__ albedo, const float *__rest
 __device__ __forceinline__ float crf(float ec, float gain, float wb, float gamma) {
     const float a = gain * wb * ec;
     return a > 0.0f ? powf(a, gamma) : 0.0f;
+}
+
+// Eqs. 4 and 5 of one pixel from the sum over its samples
+__device__ __forceinline__ void write_pixel(const RenderArgs &a, int64_t pix, f3 sum) {
+    const float inv = 1.0f / (float)a.spp;
+    const float ex = sum.x * inv, ey = sum.y * inv, ez = sum.z * inv;
+    if (a.Ec) {
+        a.Ec[3 * pix] = ex;
+        a.Ec[3 * pix + 1] = ey;
+        a.Ec[3 * pix + 2] = ez;
+    }
+    a.Ic[3 * pix] = crf(ex, a.gain_c, a.wb[0], a.gamma_c[0]);
+    a.Ic[3 * pix + 1] = crf(ey, a.gain_c, a.wb[1], a.gamma_c[1]);
+    a.Ic[3 * pix + 2] = crf(ez, a.gain_c, a.wb[2], a.gamma_c[2]);
 }
 
 // Forward megakernel.  Every loop iteration traces exactly one ray per lane --
@@ -235,9 +250,9 @@ __device__ __forceinline__ void render_lanes(const RenderArgs &a, int64_t pix, i
                     // traversal) keeps the lane in phase with the others
                     shadow = true;
                     nulls = true;
-                    ray.o = S.x + S.n * kRayEps;
+                    ray.o = madd(S.x, S.n, kRayEps);
 #else
-                    ray = make_ray(S.x + S.n * kRayEps, ed);
+                    ray = make_ray(madd(S.x, S.n, kRayEps), ed);
                     ++b;
 #endif
                 } else {
@@ -265,18 +280,7 @@ __device__ __forceinline__ void render_lanes(const RenderArgs &a, int64_t pix, i
         sum.y += __shfl_xor_sync(0xffffffffu, sum.y, off);
         sum.z += __shfl_xor_sync(0xffffffffu, sum.z, off);
     }
-    if (valid && sl == 0) {
-        const float inv = 1.0f / (float)a.spp;
-        const float ex = sum.x * inv, ey = sum.y * inv, ez = sum.z * inv;
-        if (a.Ec) {
-            a.Ec[3 * pix] = ex;
-            a.Ec[3 * pix + 1] = ey;
-            a.Ec[3 * pix + 2] = ez;
-        }
-        a.Ic[3 * pix] = crf(ex, a.gain_c, a.wb[0], a.gamma_c[0]);
-        a.Ic[3 * pix + 1] = crf(ey, a.gain_c, a.wb[1], a.gamma_c[1]);
-        a.Ic[3 * pix + 2] = crf(ez, a.gain_c, a.wb[2], a.gamma_c[2]);
-    }
+    if (valid && sl == 0) write_pixel(a, pix, sum);
 }
 
 __global__ void __launch_bounds__(kRenderBlock, DPCS_RENDER_MINB) k_render(const RenderArgs a) {
@@ -284,6 +288,37 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_RENDER_MINB) k_render(const
     const int64_t pix = gt >> a.log2L;
     render_lanes(a, pix, (int)(gt & ((1 << a.log2L) - 1)), pix < (int64_t)a.Hc * a.Wc);
 }
+
+// Forward render of the S path lanes from lane0 on over a block tile
+// (tile.cuh): the image of render_lanes bit for bit.  Lane 0 belongs to pixel
+// pix0, and there are nlane lanes.
+template <int B, int S>
+__device__ __forceinline__ void render_tile(const RenderArgs &a, Tile<S> &P, int64_t pix0, int64_t lane0, int64_t nlane) {
+    const int L = 1 << a.log2L;
+    Cnt cnt;
+    PlainCore core;
+    tile_clear_sums<S>(P, B);
+    const int rounds = a.root != kEmptyRoot ? (a.spp + L - 1) / L : 0;
+    for (int k = 0; k < rounds; ++k) tile_round<B, S>(a, core, P, pix0, lane0, nlane, k, cnt);
+    cnt.flush(a.counters);
+    __syncthreads();
+#pragma unroll 1
+    for (int slot = threadIdx.x; slot < S; slot += B) {
+        const int64_t gt = lane0 + slot;
+        const f3 sum = tile_pixel_sum<S>(P, slot, L);
+        if (gt < nlane && (gt & (L - 1)) == 0) write_pixel(a, pix0 + (gt >> a.log2L), sum);
+    }
+}
+
+template <int B, int S>
+__global__ void __launch_bounds__(B, 1024 / B) k_render_tile(const RenderArgs a) {
+    __shared__ Tile<S> P;
+    render_tile<B, S>(a, P, 0, (int64_t)blockIdx.x * S, ((int64_t)a.Hc * a.Wc) << a.log2L);
+}
+
+// Does a render with these arguments run in tiles (launch_render says why)?
+constexpr int32_t kTileTriangles = 32768;
+__host__ __device__ __forceinline__ bool tiled(const RenderArgs &a) { return a.bounces > 1 && a.T <= kTileTriangles; }
 
 // Batched persistent render: CTAs pull virtual blocks from a device counter;
 // virtual block vb belongs to the segment whose range [vb_begin, vb_begin +
@@ -566,9 +601,9 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_GRAD_MINB) k_replay(const R
                     // traversal) keeps the lane in phase with the others
                     shadow = true;
                     nulls = true;
-                    ray.o = S.x + S.n * kRayEps;
+                    ray.o = madd(S.x, S.n, kRayEps);
 #else
-                    ray = make_ray(S.x + S.n * kRayEps, ed);
+                    ray = make_ray(madd(S.x, S.n, kRayEps), ed);
                     ++b;
 #endif
                 } else {
@@ -717,9 +752,9 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_GRAD_MINB) k_render_grad(co
                     // traversal) keeps the lane in phase with the others
                     shadow = true;
                     nulls = true;
-                    ray.o = S.x + S.n * kRayEps;
+                    ray.o = madd(S.x, S.n, kRayEps);
 #else
-                    ray = make_ray(S.x + S.n * kRayEps, ed);
+                    ray = make_ray(madd(S.x, S.n, kRayEps), ed);
                     ++b;
 #endif
                 } else {
@@ -919,9 +954,9 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_GRAD_MINB)
                     // traversal) keeps the lane in phase with the others
                     shadow = true;
                     nulls = true;
-                    ray.o = S.x + S.n * kRayEps;
+                    ray.o = madd(S.x, S.n, kRayEps);
 #else
-                    ray = make_ray(S.x + S.n * kRayEps, ed);
+                    ray = make_ray(madd(S.x, S.n, kRayEps), ed);
                     ++b;
 #endif
                 } else {
@@ -952,18 +987,7 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_GRAD_MINB)
         sum.y += __shfl_xor_sync(0xffffffffu, sum.y, off);
         sum.z += __shfl_xor_sync(0xffffffffu, sum.z, off);
     }
-    if (valid && sl == 0) {
-        const float inv = 1.0f / (float)a.spp;
-        const float ex = sum.x * inv, ey = sum.y * inv, ez = sum.z * inv;
-        if (a.Ec) {
-            a.Ec[3 * pix] = ex;
-            a.Ec[3 * pix + 1] = ey;
-            a.Ec[3 * pix + 2] = ez;
-        }
-        a.Ic[3 * pix] = crf(ex, a.gain_c, a.wb[0], a.gamma_c[0]);
-        a.Ic[3 * pix + 1] = crf(ey, a.gain_c, a.wb[1], a.gamma_c[1]);
-        a.Ic[3 * pix + 2] = crf(ez, a.gain_c, a.wb[2], a.gamma_c[2]);
-    }
+    if (valid && sl == 0) write_pixel(a, pix, sum);
 }
 
 // The adjoint from the records k_render_keep wrote: the reverse sweep of
@@ -1098,6 +1122,8 @@ __global__ void k_finalize(const double *__restrict__ acc, float *__restrict__ d
     if (i < 11) dParams[i] += (float)acc[i];
 }
 
+constexpr int64_t kTileLanes = 500000;  // fewer (pixel, lane) pairs: small tiles
+
 inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
 }  // namespace
@@ -1113,8 +1139,21 @@ int launch_pack_tex(const float *albedo, const float *rough, int64_t ntex, float
 }
 
 int launch_render(const RenderArgs &a, cudaStream_t st) {
-    const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
-    k_render<<<grid_for(threads, kRenderBlock), kRenderBlock, 0, st>>>(a);
+    const int64_t lanes = ((int64_t)a.Hc * a.Wc) << a.log2L;
+    // Where the tiles pay (GB300, start -> lanes kernel / tiles): paths of one
+    // bounce have nothing to compact (plane 512 x 512 at 16 spp 206 -> 206 / 230
+    // us).  Above some tens of thousands of triangles the tree no longer sits in
+    // the L1 that the tiles' shared memory leaves (heightfields of 7,200 / 51,200
+    // / 199,712 triangles 1.47 -> 1.43 / 1.42 ms, 2.00 -> 1.96 / 2.08 ms,
+    // 8.41 -> 8.24 / 8.61 ms).  Small images want more, smaller tiles: tiles of 64
+    // / 256 lanes take 74 / 96 us at 147 k lanes, 156 / 161 us at 410 k, 206 /
+    // 195 us at 590 k.
+    if (!tiled(a))
+        k_render<<<grid_for(lanes, kRenderBlock), kRenderBlock, 0, st>>>(a);
+    else if (lanes < kTileLanes)
+        k_render_tile<64, 64><<<grid_for(lanes, 64), 64, 0, st>>>(a);
+    else
+        k_render_tile<128, 256><<<grid_for(lanes, 256), 128, 0, st>>>(a);
     return 1;
 }
 

@@ -1,0 +1,408 @@
+// tile.cuh -- path tracing over block tiles.
+//
+// A block owns S path lanes ("slots": the L lanes of its pixels, as in
+// render.cu) whose state lives in shared memory, and runs them one bounce at
+// a time in three phases with a barrier between them:
+//
+//   trace   the extension rays of the live slots and the shadow rays of the
+//           vertices shaded last, 32 rays per warp at a time;
+//   shade   every hit: surface, light, continuation;
+//   sort    the new extension rays by direction (octant and dominant axis).
+//
+// What bounds a path kernel here is instruction issue with few lanes active:
+// with one path per lane throughout, lanes wait for the longest traversal of
+// their warp, and lanes whose path has ended wait for the others' (13.5 of
+// 32 lanes active).  Phases compact both: a warp gets 32 live rays, neighbours
+// in direction, so their walks down the tree have similar lengths, and 32
+// hits to shade (21 of 32 lanes active, 0.82 G warp instructions instead of
+// 1.19 G; corner 256 x 256 at 64 spp, 3 bounces: 1.367 -> 1.047 ms on GB300;
+// 640 x 360 at 35 spp, whose second round has 3 lanes of 32: 4.12 -> 2.52 ms).
+// Of that the direction sort gives 5 %.  Tiles of one or three slots a thread
+// were 15 and 9 % slower than of two; letting a slot take its next sample as
+// soon as its path ended mixed bounces in the phases and was 9 % slower.
+//
+// Every slot runs its samples in order and adds its lit vertices in vertex
+// order, and the per-vertex arithmetic is device.cuh's, so a pixel's result
+// does not depend on the schedule.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "device.cuh"
+#include "internal.h"
+
+namespace dpcs {
+
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int32_t kDone = kEmptyRoot;  // no leaf reference: positions stay below 2^28
+constexpr int kBins = 24;              // directions: octant x dominant axis
+
+template <int S>
+struct Tile {
+    float o[3][S];         // origin of the slot's extension and shadow rays
+    float d[3][S];         // extension direction
+    float h[3][S];         // (leaf position, u, v) of the extension ray's hit
+    float beta[3][S];      // throughput entering the next vertex
+    float c[3][S];         // contribution waiting for its shadow ray
+    float sum[3][S];       // lane sum over the samples so far
+    uint16_t ext[S];       // slots with an extension ray to trace, by direction
+    uint16_t shadow[S];    // slots with a shadow ray to trace
+    uint16_t hits[S];      // slots to shade
+    uint16_t rank[S];      // rank of the slot's extension ray within its bin
+    uint8_t key[S];        // its bin, or 255: the path has ended
+    int bin[32];           // extension rays per bin
+    int next;              // 32-ray chunks taken by the trace phase
+    int nhit, nshadow;
+    int work;              // persistent kernels: the tile in hand
+};
+
+__device__ __forceinline__ f3 ld3(const float *p, int n, int i) { return mk3(p[i], p[n + i], p[2 * n + i]); }
+__device__ __forceinline__ void st3(float *p, int n, int i, f3 v) {
+    p[i] = v.x;
+    p[n + i] = v.y;
+    p[2 * n + i] = v.z;
+}
+
+// append v of the lanes with `take` to a list shared by the block
+__device__ __forceinline__ void tile_append(uint16_t *list, int *n, int v, bool take) {
+    const unsigned m = __ballot_sync(kFull, take);
+    if (!m) return;
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(n, __popc(m));
+    base = __shfl_sync(kFull, base, 0);
+    if (take) list[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)v;
+}
+
+__device__ __forceinline__ int dir_bin(f3 d) {
+    const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
+    const int k = ax > ay ? (ax > az ? 0 : 2) : (ay > az ? 1 : 2);
+    return 8 * k + (d.x < 0.f ? 1 : 0) + (d.y < 0.f ? 2 : 0) + (d.z < 0.f ? 4 : 0);
+}
+
+// ---------------------------------------------------------------------------
+// traversal
+// ---------------------------------------------------------------------------
+typedef unsigned long long u64;
+__device__ __forceinline__ u64 pk2(float a, float b) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void up2(u64 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+    u64 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// 32 bytes of a tree node (64-byte aligned) in one load
+__device__ __forceinline__ void ldg8(const float4 *p, float4 &a, float4 &b) {
+    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
+
+// slab() of device.cuh with the two planes of an axis in one packed FMA (the
+// same roundings; a node lists them side by side)
+__device__ __forceinline__ bool slab2(u64 x, u64 y, u64 z, u64 ix, u64 iy, u64 iz, u64 ox, u64 oy, u64 oz, float err,
+                                      float tmax, float &tnear) {
+    float tx0, tx1, ty0, ty1, tz0, tz1;
+    up2(fma2(x, ix, ox), tx0, tx1);
+    up2(fma2(y, iy, oy), ty0, ty1);
+    up2(fma2(z, iz, oz), tz0, tz1);
+    const float tn = fmax3f(fminf(tx0, tx1), fminf(ty0, ty1), fmaxf(fminf(tz0, tz1), 0.0f));
+    const float tf = fmin3f(fmaxf(tx0, tx1), fmaxf(ty0, ty1), fminf(fmaxf(tz0, tz1), tmax));
+    tnear = tn;
+    return tn <= fmaf(tf, 1.0000004f, err);
+}
+
+// One step down the tree: 50 instructions against the 54 of trav_resume's
+// (a chain of nodes with one child hit each).
+__device__ __forceinline__ void tree_node(const RenderArgs &a, const Ray &ray, float ht, int &node, int &sp, int *stack,
+                                          Cnt &cnt) {
+    cnt.add_warp(kCntTravWarpIter);
+    cnt.add(kCntNode);
+    const float4 *nd = reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(a.nodes) +
+                                                        (size_t)(uint32_t)node * 64u);
+    float4 n0, n1, n2, n3;
+    ldg8(nd, n0, n1);
+    ldg8(nd + 2, n2, n3);
+    const u64 ix = pk2(ray.inv.x, ray.inv.x), iy = pk2(ray.inv.y, ray.inv.y), iz = pk2(ray.inv.z, ray.inv.z);
+    const u64 ox = pk2(-ray.oinv.x, -ray.oinv.x), oy = pk2(-ray.oinv.y, -ray.oinv.y),
+              oz = pk2(-ray.oinv.z, -ray.oinv.z);
+    float tl, tr;
+    const bool hl = slab2(pk2(n0.x, n0.y), pk2(n0.z, n0.w), pk2(n2.x, n2.y), ix, iy, iz, ox, oy, oz, ray.err, ht, tl);
+    const bool hr = slab2(pk2(n1.x, n1.y), pk2(n1.z, n1.w), pk2(n2.z, n2.w), ix, iy, iz, ox, oy, oz, ray.err, ht, tr);
+    const int cl = __float_as_int(n3.x), cr = __float_as_int(n3.y);
+    const bool lf = tl <= tr;
+    if (hl | hr) {
+        const bool takel = hl & (lf | !hr);
+        node = takel ? cl : cr;
+        if (hl & hr) stack[sp++] = takel ? cr : cl;
+    } else {
+        node = sp > 0 ? stack[--sp] : kDone;
+    }
+}
+
+// Closest hit (any = false; ht = infinity at the start) or any hit before ht,
+// from node = a.root; lanes with node = kDone only take part in the warp's
+// votes.  hpos < 0: nothing hit.  The tree is at most kStack deep.
+__device__ __forceinline__ void tree_walk(const RenderArgs &a, const Ray &ray, bool any, int node, int &hpos, float &ht,
+                                          float &hu, float &hv, Cnt &cnt) {
+    int stack[kStack];
+    int sp = 0, left = a.visit_cap > 0 ? a.visit_cap : 2 * a.T + 16;  // tree steps before the ray gives up
+    while (true) {
+        while (node >= 0) {
+            --left;
+#ifdef DPCS_CHECK
+            if (node >= a.T - 1) {
+                atomicOr(a.status, kStatusBoundsCheck);
+                hpos = -1;
+                sp = 0;
+                node = kDone;
+                break;
+            }
+#endif
+            tree_node(a, ray, ht, node, sp, stack, cnt);
+        }
+        __syncwarp();
+#ifdef DPCS_CHECK
+        if (node != kDone && ~node >= a.T) {
+            atomicOr(a.status, kStatusBoundsCheck);
+            hpos = -1;
+            node = kDone;
+        }
+#endif
+        if (node != kDone) {
+            cnt.add_warp(kCntTravWarpIter);
+            cnt.add(kCntTri);
+            const int pos = ~node;
+            const float4 A = __ldg(a.tris + 3 * pos + 0);
+            const float4 B = __ldg(a.tris + 3 * pos + 1);
+            const float4 C = __ldg(a.tris + 3 * pos + 2);
+            float t, u, v;
+            if (tri_isect(ray, xyz(A), xyz(B), xyz(C), ht, t, u, v)) {
+                // ties in t to the lowest original triangle index
+                if (t < ht || (!any && hpos >= 0 && __float_as_int(A.w) < __float_as_int(__ldg(a.tris + 3 * hpos).w))) {
+                    hpos = pos;
+                    ht = t;
+                    hu = u;
+                    hv = v;
+                    if (any) sp = 0;
+                }
+            }
+            if (--left < 0) {
+                atomicOr(a.status, kStatusTraversalLimit);
+                hpos = -1;
+                sp = 0;
+            }
+            node = sp > 0 ? stack[--sp] : kDone;
+        }
+        if (__all_sync(kFull, node == kDone)) break;
+    }
+}
+
+// Trace the tile's ne extension rays and ns shadow rays, 32 of a kind per warp
+// at a time: closest hits into h and the list of hits; shadow rays (from o to
+// the projector's centre) add their contribution c to the slot's sum, or tell
+// the core that vertex v of round k is dark.
+template <int S, class Core>
+__device__ __forceinline__ void tile_trace(const RenderArgs &a, Core &core, Tile<S> &P, int ne, int ns, int k, int v,
+                                           Cnt &cnt) {
+    const int lane = threadIdx.x & 31;
+    const int ce = (ne + 31) >> 5, chunks = ce + ((ns + 31) >> 5);
+    while (true) {
+        int c = 0;
+        if (lane == 0) c = atomicAdd(&P.next, 1);
+        c = __shfl_sync(kFull, c, 0);
+        if (c >= chunks) break;
+        const bool any = c >= ce;
+        const int i = 32 * (any ? c - ce : c) + lane;
+        const bool on = i < (any ? ns : ne);
+        const int slot = on ? (any ? P.shadow[i] : P.ext[i]) : 0;
+        int node = kDone, hpos = -1;
+        float ht = INFINITY, hu = 0.f, hv = 0.f;
+        Ray ray;
+        if (on) {
+            const f3 o = ld3(&P.o[0][0], S, slot);
+            f3 d = ld3(&P.d[0][0], S, slot);
+            if (any) {  // nee_prepare's shadow ray from its origin
+                const f3 sv = mk3(a.cp[0], a.cp[1], a.cp[2]) - o;
+                const float sd = sqrtf(dot(sv, sv));
+                d = sv * (1.0f / sd);
+                ht = sd - kRayEps;
+            }
+            cnt.add(any ? kCntShadow : kCntRay);
+            ray = make_ray(o, d);
+            node = a.root;
+        }
+        cnt.add_warp(kCntPathWarpIter);
+        __syncwarp();
+        tree_walk(a, ray, any, node, hpos, ht, hu, hv, cnt);
+        if (any) {
+            if (on) {
+                if (hpos < 0) {
+                    st3(&P.sum[0][0], S, slot, ld3(&P.sum[0][0], S, slot) + ld3(&P.c[0][0], S, slot));
+                    cnt.add(kCntLit);
+                } else {
+                    core.dark(a, slot, k, v);
+                }
+            }
+        } else {
+            if (hpos >= 0) st3(&P.h[0][0], S, slot, mk3(__int_as_float(hpos), hu, hv));
+            tile_append(P.hits, &P.nhit, slot, hpos >= 0);
+        }
+        __syncwarp();
+    }
+}
+
+// What shading a vertex hands back to the tile.
+struct Shaded {
+    bool cand, ext;  // a shadow ray carrying c is due; the path goes on along wi with throughput beta
+    f3 c, so, wi, beta;
+};
+
+// Round k of the tile's slots: sample sl + k L of pixel `pix` for every slot
+// whose live(slot, pix) is true.  `lane0` is the first slot's lane among the
+// launch's (pixel, lane) pairs, `pix0` the pixel of lane 0, `nlane` the lanes
+// there are.  Every thread of the block calls it; it ends with a barrier.
+template <int B, int S, class Core>
+__device__ __forceinline__ void tile_round(const RenderArgs &a, Core &core, Tile<S> &P, int64_t pix0, int64_t lane0,
+                                           int64_t nlane, int k, Cnt &cnt) {
+    const int L = 1 << a.log2L, tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) P.next = P.nhit = P.nshadow = 0;
+    if (tid < 32) P.bin[tid] = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int slot = tid; slot < S; slot += B) {
+        const int64_t gt = lane0 + slot;
+        const uint32_t pix = (uint32_t)(pix0 + (gt >> a.log2L));
+        const int s = (int)(gt & (L - 1)) + k * L;
+        const bool live = gt < nlane && s < a.spp && core.begin(a, slot, pix, k);
+        if (live) {
+            f3 o, d;
+            camera_ray(a, pix, (uint32_t)s, o, d);
+            st3(&P.o[0][0], S, slot, o);
+            st3(&P.d[0][0], S, slot, d);
+            st3(&P.beta[0][0], S, slot, mk3(1.f, 1.f, 1.f));
+            cnt.add(kCntPath);
+        }
+        tile_append(P.ext, &P.bin[0], slot, live);
+    }
+    __syncthreads();
+    int ne = P.bin[0], ns = 0;
+    __syncthreads();
+    // Three barriers a bounce.  Each counter is cleared in a phase that
+    // neither adds to it nor reads it: the bins and the shadow count while
+    // the rays are traced, the hit count and the chunk counter after shading.
+    for (int b = 1;; ++b) {
+        if (tid < 32) P.bin[tid] = 0;
+        if (tid == 32) P.nshadow = 0;
+        tile_trace<S>(a, core, P, ne, ns, k, b - 2, cnt);
+        __syncthreads();
+        const int nh = P.nhit;
+        if (nh == 0) break;
+#pragma unroll 1
+        for (int i0 = tid & ~31; i0 < nh; i0 += B) {
+            const int i = i0 + lane;
+            const bool on = i < nh;
+            const int slot = on ? P.hits[i] : 0;
+            bool cand = false;
+            if (on) {
+                cnt.add(kCntVert);
+                const int64_t gt = lane0 + slot;
+                Hit h;
+                h.pos = __float_as_int(P.h[0][slot]);
+                h.u = P.h[1][slot];
+                h.v = P.h[2][slot];
+                Shaded R;
+                core.shade(a, slot, (uint32_t)(pix0 + (gt >> a.log2L)), (uint32_t)((int)(gt & (L - 1)) + k * L), k, b, h,
+                           ld3(&P.d[0][0], S, slot), ld3(&P.beta[0][0], S, slot), R);
+                cand = R.cand;
+                if (cand) st3(&P.c[0][0], S, slot, R.c);
+                int key = 255;
+                if (R.ext) {
+                    cnt.add(kCntCont);
+                    st3(&P.beta[0][0], S, slot, R.beta);
+                    st3(&P.d[0][0], S, slot, R.wi);
+                    key = dir_bin(R.wi);
+                    P.rank[slot] = (uint16_t)atomicAdd(&P.bin[key], 1);
+                }
+                P.key[slot] = (uint8_t)key;
+                st3(&P.o[0][0], S, slot, R.so);
+            }
+            __syncwarp();
+            tile_append(P.shadow, &P.nshadow, slot, cand);
+        }
+        __syncthreads();
+        if (tid == 0) P.nhit = P.next = 0;
+        // every warp scans the bins (one a lane) and places its share of the rays
+        const int count = P.bin[lane];
+        int end = count;
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(kFull, end, off);
+            if (lane >= off) end += y;
+        }
+        ne = __shfl_sync(kFull, end, 31);
+        ns = P.nshadow;
+#pragma unroll 1
+        for (int i0 = tid & ~31; i0 < nh; i0 += B) {
+            const int slot = i0 + lane < nh ? P.hits[i0 + lane] : 0;
+            const int key = i0 + lane < nh ? P.key[slot] : 255;
+            const int first = __shfl_sync(kFull, end - count, key & 31);
+            if (key != 255) P.ext[first + P.rank[slot]] = (uint16_t)slot;
+        }
+        __syncthreads();
+    }
+    __syncthreads();
+}
+
+template <int S>
+__device__ __forceinline__ void tile_clear_sums(Tile<S> &P, int B) {
+#pragma unroll 1
+    for (int slot = threadIdx.x; slot < S; slot += B) st3(&P.sum[0][0], S, slot, mk3(0.f, 0.f, 0.f));
+}
+
+// the slot's lane sum combined over the L lanes of its pixel (the xor tree of
+// render_lanes); every thread of the warp calls it with its slot
+template <int S>
+__device__ __forceinline__ f3 tile_pixel_sum(const Tile<S> &P, int slot, int L) {
+    f3 sum = ld3(&P.sum[0][0], S, slot);
+    for (int off = L >> 1; off > 0; off >>= 1) {
+        sum.x += __shfl_xor_sync(kFull, sum.x, off);
+        sum.y += __shfl_xor_sync(kFull, sum.y, off);
+        sum.z += __shfl_xor_sync(kFull, sum.z, off);
+    }
+    return sum;
+}
+
+// the Lambert + GGX material, nothing recorded
+struct PlainCore {
+    __device__ __forceinline__ bool begin(const RenderArgs &, int, uint32_t, int) { return true; }
+    __device__ __forceinline__ void dark(const RenderArgs &, int, int, int) {}
+    __device__ __forceinline__ void shade(const RenderArgs &a, int, uint32_t pix, uint32_t s, int, int b, const Hit &h,
+                                          f3 d, f3 beta, Shaded &R) {
+        const Surf F = surface_at(a, h, d);
+        Nee Q;
+        R.cand = nee_prepare(a, F, Q);
+        if (R.cand) {
+            unsigned unc;
+            R.c = nee_contrib(a, beta, Q, unc);
+        }
+        R.ext = false;
+        if (b < a.bounces) {
+            Cont C;
+            R.ext = continue_prepare(a, pix, s, b, F, C);
+            if (R.ext) {
+                R.beta = beta * C.w;
+                R.wi = C.wi;
+            }
+        }
+        R.so = madd(F.x, F.n, kRayEps);
+    }
+};
+
+}  // namespace dpcs

@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kWfBlock, DPCS_WF_SHADE_MINB) k_wf_shade(const
                     beta = beta * C.w;
                     // the extension ray starts where the shadow ray did, as in
                     // k_render (the same value, computed in the same place)
-                    const f3 o = cand ? N.so : S.x + S.n * kRayEps;
+                    const f3 o = cand ? N.so : madd(S.x, S.n, kRayEps);
                     w.ro[c] = make_float4(o.x, o.y, o.z, 0.f);
                     w.rd[c] = make_float4(C.wi.x, C.wi.y, C.wi.z, 0.f);
                     w.beta[c] = make_float4(beta.x, beta.y, beta.z, 0.f);

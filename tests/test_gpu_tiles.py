@@ -1,0 +1,51 @@
+"""The block-tile path kernels against the lanes kernels on the same paths.
+
+The server's relighting kernel traces one path per lane throughout, so a
+relit image is the lanes kernel's; dpcs_render picks tiles by size.  Both add
+the same values in the same order, so images are equal bit for bit, at sizes
+around the tiles' edges: fewer lanes than a tile, a last tile of a few lanes,
+samples that do not fill a round, either tile size, the longest paths."""
+import numpy as np
+import pytest
+
+from paper_2503_12174_gb300 import dpcs, scenes
+from gpu_util import need_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def _scene(mesh, H, W, spp, bounces):
+    if mesh == "corner":
+        sc = scenes.corner(res=32, tex=24, spp=spp, bounces=bounces, seed=5)
+    elif mesh == "sphere":
+        sc = scenes.sphere(subdiv=2, spp=spp, bounces=bounces, seed=5)
+    else:  # a single triangle: the tree has no inner node
+        sc = scenes.plane(res=32, spp=spp, seed=5)
+        sc = sc.replace(tris=sc.tris[:1], bounces=bounces)
+    return sc.replace(Kc=scenes.intrinsics(W, H, 40.0), Hc=H, Wc=W)
+
+
+@pytest.mark.parametrize("mesh,H,W,spp,bounces", [
+    ("corner", 1, 1, 1, 2), ("corner", 1, 3, 7, 3), ("corner", 5, 13, 1, 8), ("corner", 17, 31, 35, 3),
+    ("corner", 9, 57, 64, 2), ("corner", 127, 123, 32, 3), ("corner", 125, 125, 33, 3), ("corner", 128, 123, 33, 4),
+    ("sphere", 24, 24, 16, 8), ("triangle", 20, 20, 8, 3)])
+def test_tiles_render_what_lanes_render(mesh, H, W, spp, bounces):
+    torch = need_cuda()
+    sc = _scene(mesh, H, W, spp, bounces)
+    c = dpcs.Context(0)
+    h = c.upload(sc.verts, sc.tris, sc.uv)
+    alb, rough, Ip = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (sc.albedo, sc.rough, sc.Ip))
+    view, prm = dpcs.view_of(sc), dpcs.make_params(sc.params)
+    srv = dpcs.Server(c)
+    try:
+        Ic, _ = c.render(h, alb, rough, Ip, view, prm, spp, bounces, sc.seed)
+        c.sync()
+        out = torch.empty((H, W, 3)).pin_memory()
+        slot = srv.add_scene(h, alb, rough, view, prm, bounces)
+        srv.submit(dpcs.DPCS_REQ_RELIGHT, slot, H, W, spp, sc.seed, torch.from_numpy(sc.Ip), out)
+        srv.drain()
+        assert torch.equal(Ic.cpu(), out) and (mesh == "triangle" or out.abs().max() > 0)
+    finally:
+        srv.close()
+        c.free(h)
+        c.close()
