@@ -63,6 +63,8 @@ struct dpcs_ctx {
     Buf mat4, dmat4;  // principled material: (metallic, normal map) per texel and its gradient accumulators
     Buf dEp64, dtex64;  // FP64 gradient accumulators (dpcs_set_grad_accum(ctx, DPCS_ACCUM_F64))
     bool grad_f64 = false;
+    Buf recs;  // path records of the adjoint kernels' tiles (optional: see optional_scratch)
+    std::vector<void *> retired;  // smaller recs of earlier calls: a captured graph may still use them
     Buf wf;  // wavefront render: lane sums, per-chunk path state, queues
     int32_t render_path = DPCS_PATH_MEGAKERNEL;
     int64_t wf_chunk = int64_t(1) << 20;
@@ -135,6 +137,34 @@ dpcs_status ensure(dpcs_ctx *c, Buf &b, size_t bytes, const char *what) {
     dpcs_status s = dev_alloc(c, &b.p, bytes, what);
     if (s == DPCS_OK) b.n = bytes;
     return s;
+}
+
+// Scratch that a faster kernel wants but the call can do without: null when
+// `bytes` is 0, when the context has a memory budget (which is left for what
+// calls cannot do without), when it would have to be allocated while the
+// stream is being captured, or when the device has no room.  A smaller buffer
+// is kept until the context goes, since a captured graph may hold its address;
+// sizes double, so those come to less than the one in use.
+void *optional_scratch(dpcs_ctx *c, Buf &b, size_t bytes, cudaStream_t st) {
+    if (!bytes || c->budget) return nullptr;
+    if (b.n >= bytes) return b.p;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    size_t n = size_t(1) << 20;
+    while (n < bytes) n <<= 1;
+    void *p = nullptr;
+    if (cudaMalloc(&p, n) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (b.p) c->retired.push_back(b.p);
+    b.p = p;
+    b.n = n;
+    c->used += n;
+    return p;
 }
 
 dpcs_status set_device(dpcs_ctx *c) {
@@ -436,9 +466,10 @@ dpcs_status dpcs_destroy(dpcs_ctx *c) {
     }
     for (auto &kv : c->edges) cudaFree(kv.second.d);
     Buf *bufs[] = {&c->ep4, &c->tex4, &c->gE, &c->dEp4, &c->dtex4, &c->acc, &c->partial, &c->build, &c->upload, &c->pix,
-                   &c->kept, &c->mat4, &c->dmat4, &c->dEp64, &c->dtex64, &c->wf, &c->pose, &c->ploc};
+                   &c->kept, &c->mat4, &c->dmat4, &c->dEp64, &c->dtex64, &c->wf, &c->pose, &c->ploc, &c->recs};
     for (Buf *b : bufs)
         if (b->p) cudaFree(b->p);
+    for (void *p : c->retired) cudaFree(p);
     cudaFree(c->status);
     cudaFree(c->counters);
     for (TimedLaunch &t : c->timed) {
@@ -820,6 +851,7 @@ dpcs_status dpcs_render_backward(dpcs_ctx *c, dpcs_scene scene, const float *alb
     const bool want_tex = dAlbedo || dRough;  // otherwise the replay skips the texture scatters
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = grad_setup(c, np, nt, want_tex, st, a))) return s;
+    void *recs = optional_scratch(c, c->recs, grad_scratch_bytes(a, true, kRecWordsHost), st);
     double *acc = (double *)c->acc.p;
     cudaMemsetAsync(acc, 0, 16 * sizeof(double), st);
     int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
@@ -829,7 +861,7 @@ dpcs_status dpcs_render_backward(dpcs_ctx *c, dpcs_scene scene, const float *alb
     a.tex = (const float4 *)c->tex4.p;
     a.gE = (const float *)c->gE.p;
     TimedLaunch *tl = timing_begin(c, 1, st);
-    nl += launch_replay(a, st);
+    nl += launch_replay(a, acc, recs, st);
     timing_end(tl, st);
     nl += grad_finish(a, Ip, np, nt, params, dIp, dAlbedo, dRough, acc, st);
     if (dParams) nl += launch_finalize_params(acc, dParams, st);
@@ -1037,10 +1069,11 @@ dpcs_status dpcs_render_loss_backward(dpcs_ctx *c, dpcs_scene scene, const float
     a.tex = (const float4 *)c->tex4.p;
     a.Ic = Ic;
     const LossArgs l{target, scale, loss_kind, acc};
+    void *recs = optional_scratch(c, c->recs, grad_scratch_bytes(a, !fused, kRecWordsHost), st);
     if (fused) {
         a.Ec = Ec;
         TimedLaunch *tl = timing_begin(c, 0, st);
-        nl += launch_render_grad(a, l, st);
+        nl += launch_render_grad(a, l, recs, st);
         timing_end(tl, st);
     } else {  // render, per-pixel loss, Eq. 5 adjoint, replay
         float *dIc = (float *)c->pix.p, *ec = Ec ? Ec : (float *)c->pix.p + 3 * npix;
@@ -1053,7 +1086,7 @@ dpcs_status dpcs_render_loss_backward(dpcs_ctx *c, dpcs_scene scene, const float
                                   acc, st);
         a.gE = (const float *)c->gE.p;
         TimedLaunch *tr = timing_begin(c, 1, st);
-        nl += launch_replay(a, st);
+        nl += launch_replay(a, acc, recs, st);
         timing_end(tr, st);
     }
     nl += launch_loss_out(acc, loss, st);

@@ -95,22 +95,46 @@ __device__ __forceinline__ f3 operator+(f3 a, f3 b) { return mk3(a.x + b.x, a.y 
 __device__ __forceinline__ f3 operator-(f3 a, f3 b) { return mk3(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ __forceinline__ f3 operator*(f3 a, float s) { return mk3(a.x * s, a.y * s, a.z * s); }
 __device__ __forceinline__ f3 operator*(f3 a, f3 b) { return mk3(a.x * b.x, a.y * b.y, a.z * b.z); }
+#ifdef DPCS_FUSION_BY_COMPILER
+// for files whose paths no kernel elsewhere has to agree with
+__device__ __forceinline__ float muladd(float a, float b, float c) { return c + a * b; }
+__device__ __forceinline__ float mul1(float a, float b) { return a * b; }
+#else
+__device__ __forceinline__ float muladd(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float mul1(float a, float b) { return __fmul_rn(a, b); }
+#endif
 // a0 b0 + a1 b1 and a0 b0 - a1 b1 with one product rounded on its own
-__device__ __forceinline__ float sum2(float a0, float b0, float a1, float b1) { return fmaf(a0, b0, __fmul_rn(a1, b1)); }
-__device__ __forceinline__ float diff2(float a0, float b0, float a1, float b1) {
-    return fmaf(a0, b0, -__fmul_rn(a1, b1));
+__device__ __forceinline__ float sum2(float a0, float b0, float a1, float b1) {
+#ifdef DPCS_FUSION_BY_COMPILER
+    return a0 * b0 + a1 * b1;
+#else
+    return fmaf(a0, b0, __fmul_rn(a1, b1));
+#endif
 }
-__device__ __forceinline__ float dot(f3 a, f3 b) { return fmaf(a.z, b.z, sum2(a.x, b.x, a.y, b.y)); }
+__device__ __forceinline__ float diff2(float a0, float b0, float a1, float b1) {
+#ifdef DPCS_FUSION_BY_COMPILER
+    return a0 * b0 - a1 * b1;
+#else
+    return fmaf(a0, b0, -__fmul_rn(a1, b1));
+#endif
+}
+__device__ __forceinline__ float dot(f3 a, f3 b) { return muladd(a.z, b.z, sum2(a.x, b.x, a.y, b.y)); }
 __device__ __forceinline__ f3 cross(f3 a, f3 b) {
     return mk3(diff2(a.y, b.z, a.z, b.y), diff2(a.z, b.x, a.x, b.z), diff2(a.x, b.y, a.y, b.x));
 }
 // the same product sum with y rounded into x's place
-__device__ __forceinline__ float dot_yx(f3 a, f3 b) { return fmaf(a.z, b.z, sum2(a.y, b.y, a.x, b.x)); }
+__device__ __forceinline__ float dot_yx(f3 a, f3 b) {
+#ifdef DPCS_FUSION_BY_COMPILER
+    return dot(a, b);
+#else
+    return muladd(a.z, b.z, sum2(a.y, b.y, a.x, b.x));
+#endif
+}
 // a + b s
-__device__ __forceinline__ f3 madd(f3 a, f3 b, float s) { return mk3(fmaf(b.x, s, a.x), fmaf(b.y, s, a.y), fmaf(b.z, s, a.z)); }
+__device__ __forceinline__ f3 madd(f3 a, f3 b, float s) { return mk3(muladd(b.x, s, a.x), muladd(b.y, s, a.y), muladd(b.z, s, a.z)); }
 // a x + b y + c z
 __device__ __forceinline__ f3 combine(f3 a, float x, f3 b, float y, f3 c, float z) {
-    return mk3(fmaf(c.x, z, sum2(a.x, x, b.x, y)), fmaf(c.y, z, sum2(a.y, x, b.y, y)), fmaf(c.z, z, sum2(a.z, x, b.z, y)));
+    return mk3(muladd(c.x, z, sum2(a.x, x, b.x, y)), muladd(c.y, z, sum2(a.y, x, b.y, y)), muladd(c.z, z, sum2(a.z, x, b.z, y)));
 }
 __device__ __forceinline__ f3 normalize(f3 a) { return a * (1.0f / sqrtf(dot(a, a))); }
 __device__ __forceinline__ f3 xyz(float4 v) { return mk3(v.x, v.y, v.z); }
@@ -134,8 +158,8 @@ __device__ __forceinline__ float alpha_of(float r, float &dadr) {
 // cos^2 (a^2 - 1) + 1 is formed as s2 + a^2 cos^2 with s2 = |n x h|^2: the
 // textbook form cancels catastrophically in FP32 near the peak of sharp lobes.
 __device__ __forceinline__ float ggx_D(float ch, float s2, float a) {
-    const float a2 = __fmul_rn(a, a);
-    const float t = fmaf(a2 * ch, ch, s2);
+    const float a2 = mul1(a, a);
+    const float t = muladd(a2 * ch, ch, s2);
     return a2 / (DPCS_PI_F * t * t);
 }
 __device__ __forceinline__ float sin2(f3 n, f3 h) {
@@ -144,8 +168,8 @@ __device__ __forceinline__ float sin2(f3 n, f3 h) {
 }
 
 __device__ __forceinline__ float ggx_G1(float c, float a) {
-    const float a2 = __fmul_rn(a, a);
-    return 2.0f * c / (c + sqrtf(fmaf((1.0f - a2) * c, c, a2)));
+    const float a2 = mul1(a, a);
+    return 2.0f * c / (c + sqrtf(muladd((1.0f - a2) * c, c, a2)));
 }
 
 // ks * D G F / (4 ci co) and its derivative in roughness r (0 if ks == 0)
@@ -157,14 +181,14 @@ __device__ __forceinline__ float spec_eval(f3 n, f3 wo, f3 wi, float r, float ks
     const float a = alpha_of(r, dadr);
     const f3 h = normalize(wo + wi);
     const float ch = dot(n, h);
-    const float a2 = __fmul_rn(a, a), b2 = (1.0f - a2);
-    const float t = fmaf(a2 * ch, ch, sin2(n, h));
+    const float a2 = mul1(a, a), b2 = (1.0f - a2);
+    const float t = muladd(a2 * ch, ch, sin2(n, h));
     const float D = a2 / (DPCS_PI_F * t * t);
-    const float si = sqrtf(fmaf(b2 * ci, ci, a2)), so = sqrtf(fmaf(b2 * co, co, a2));
+    const float si = sqrtf(muladd(b2 * ci, ci, a2)), so = sqrtf(muladd(b2 * co, co, a2));
     const float G = (2.0f * ci / (ci + si)) * (2.0f * co / (co + so));
     float m = fmaxf(0.0f, 1.0f - dot_yx(wo, h));
     const float m2 = m * m;
-    const float F = fmaf(1.0f - f0, m2 * m2 * m, f0);
+    const float F = muladd(1.0f - f0, m2 * m2 * m, f0);
     const float spec = ks * D * G * F / (4.0f * ci * co);
     const float dlnD = 2.0f / a - 4.0f * a * ch * ch / t;
     const float dlnG = -(a * (1.0f - ci * ci) / si) / (ci + si) - (a * (1.0f - co * co) / so) / (co + so);
@@ -179,13 +203,13 @@ __device__ __forceinline__ void onb(f3 n, f3 &t, f3 &b) {
     const float sg = n.z >= -DPCS_INV_PI_F ? 1.0f : -1.0f;
     const float a = -1.0f / (sg + n.z);
     const float bb = n.x * n.y * a;
-    t = mk3(fmaf(sg * n.x * n.x, a, 1.0f), sg * bb, -sg * n.x);
-    b = mk3(bb, fmaf(n.y * n.y, a, sg), -n.y);
+    t = mk3(muladd(sg * n.x * n.x, a, 1.0f), sg * bb, -sg * n.x);
+    b = mk3(bb, muladd(n.y * n.y, a, sg), -n.y);
 }
 
 // rho / pi + spec per channel
 __device__ __forceinline__ f3 lambert_plus(f3 rho, float spec) {
-    return mk3(fmaf(rho.x, DPCS_INV_PI_F, spec), fmaf(rho.y, DPCS_INV_PI_F, spec), fmaf(rho.z, DPCS_INV_PI_F, spec));
+    return mk3(muladd(rho.x, DPCS_INV_PI_F, spec), muladd(rho.y, DPCS_INV_PI_F, spec), muladd(rho.z, DPCS_INV_PI_F, spec));
 }
 
 __device__ __forceinline__ float spec_prob(float ks) { return ks > 0.0f ? 0.5f : 0.0f; }
@@ -200,7 +224,7 @@ __device__ __forceinline__ float bsdf_pdf(f3 n, f3 wo, f3 wi, float r, float ks)
         const float a = alpha_of(r, dadr);
         const f3 h = normalize(wo + wi);
         const float q = ps * ggx_G1(co, a) * ggx_D(dot(n, h), sin2(n, h), a) / (4.0f * co);
-        p = fmaf((1.0f - ps) * ci, DPCS_INV_PI_F, q);
+        p = muladd((1.0f - ps) * ci, DPCS_INV_PI_F, q);
     }
     return p;
 }
@@ -225,11 +249,11 @@ __device__ __forceinline__ bool bsdf_sample(f3 n, f3 wo, float r, float ks, floa
         const f3 T1 = lsq > 0.0f ? mk3(-Vh.y, Vh.x, 0.0f) * (1.0f / sqrtf(lsq)) : mk3(1.0f, 0.0f, 0.0f);
         const f3 T2 = cross(Vh, T1);
         const float rr = sqrtf(u1);
-        const float t1 = __fmul_rn(rr, cp);
-        float t2 = __fmul_rn(rr, sp);
-        const float s = 0.5f * (1.0f + Vh.z), w1 = fmaf(-t1, t1, 1.0f);
+        const float t1 = mul1(rr, cp);
+        float t2 = mul1(rr, sp);
+        const float s = 0.5f * (1.0f + Vh.z), w1 = muladd(-t1, t1, 1.0f);
         t2 = sum2(1.0f - s, sqrtf(fmaxf(0.0f, w1)), s, t2);
-        const f3 Nh = combine(T1, t1, T2, t2, Vh, sqrtf(fmaxf(0.0f, fmaf(-t2, t2, w1))));
+        const f3 Nh = combine(T1, t1, T2, t2, Vh, sqrtf(fmaxf(0.0f, muladd(-t2, t2, w1))));
         const f3 Ne = normalize(mk3(a * Nh.x, a * Nh.y, fmaxf(0.0f, Nh.z)));
         l = madd(wl * -1.0f, Ne, 2.0f * dot(wl, Ne));
     }
@@ -276,10 +300,10 @@ __device__ __forceinline__ float4 bilin_fetch(const float4 *__restrict__ img, co
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float4 v = __ldg(img + idx[k]);
-        r.x = fmaf(w[k], v.x, r.x);
-        r.y = fmaf(w[k], v.y, r.y);
-        r.z = fmaf(w[k], v.z, r.z);
-        r.w = fmaf(w[k], v.w, r.w);
+        r.x = muladd(w[k], v.x, r.x);
+        r.y = muladd(w[k], v.y, r.y);
+        r.z = muladd(w[k], v.z, r.z);
+        r.w = muladd(w[k], v.w, r.w);
     }
     return r;
 }
@@ -668,9 +692,9 @@ __device__ __forceinline__ Surf surface_at(const RenderArgs &a, const Hit &h, f3
     const float2 t0 = __ldg(a.tuv + 3 * h.pos + 0), t1 = __ldg(a.tuv + 3 * h.pos + 1),
                  t2 = __ldg(a.tuv + 3 * h.pos + 2);
     const float w0 = 1.0f - h.u - h.v;
-    const float su = fmaf(h.v, t2.x, sum2(w0, t0.x, h.u, t1.x));
-    const float sv = fmaf(h.v, t2.y, sum2(w0, t0.y, h.u, t1.y));
-    S.tb = bilin_setup(fmaf(su, (float)a.Wt, -0.5f), fmaf(sv, (float)a.Ht, -0.5f), a.Wt, a.Ht);
+    const float su = muladd(h.v, t2.x, sum2(w0, t0.x, h.u, t1.x));
+    const float sv = muladd(h.v, t2.y, sum2(w0, t0.y, h.u, t1.y));
+    S.tb = bilin_setup(muladd(su, (float)a.Wt, -0.5f), muladd(sv, (float)a.Ht, -0.5f), a.Wt, a.Ht);
     const float4 tex = bilin_fetch(a.tex, S.tb, a.Wt, a.Ht);
     S.rho = mk3(tex.x, tex.y, tex.z);
     S.rough = tex.w;

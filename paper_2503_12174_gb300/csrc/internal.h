@@ -144,8 +144,14 @@ int launch_trace(const Scene &sc, const float *o, const float *d, int64_t n, flo
                  unsigned *status, cudaStream_t st);
 int launch_crf_backward(const float *dIc, const float *Ec, const float *Ic, int64_t npix, const float gamma_c[3],
                         float gain_c, const float wb[3], float *gE, double *acc, cudaStream_t st);
-int launch_replay(const RenderArgs &a, cudaStream_t st);
-int launch_render_grad(const RenderArgs &a, const LossArgs &l, cudaStream_t st);
+// The adjoint kernels run in tiles when they are given grad_scratch_bytes of
+// scratch (0: no tile kernel for these arguments); acc[kTileCounter] must be
+// zero then, as must the rest of acc.
+constexpr int kTileCounter = 15;
+// words: 32-bit words of a vertex record
+size_t grad_scratch_bytes(const RenderArgs &a, bool replay, int words);
+int launch_replay(const RenderArgs &a, double *acc, void *scratch, cudaStream_t st);
+int launch_render_grad(const RenderArgs &a, const LossArgs &l, void *scratch, cudaStream_t st);
 int launch_pixel_loss(const float *Ic, int64_t n, const LossArgs &l, float *dIc, cudaStream_t st);
 // principled material (principled.cu)
 int launch_pack_mat(const float *metallic, const float *normal, int64_t ntex, float4 *mat, cudaStream_t st);

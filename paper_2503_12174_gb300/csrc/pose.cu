@@ -43,6 +43,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#define DPCS_FUSION_BY_COMPILER  // see device.cuh
 #include "device.cuh"
 #include "internal.h"
 #include "pose.h"

@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#define DPCS_FUSION_BY_COMPILER  // these kernels share their arithmetic with no kernel outside this file
 #include "device.cuh"
 #include "internal.h"
 #include "principled.cuh"

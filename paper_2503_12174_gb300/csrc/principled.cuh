@@ -90,7 +90,7 @@ __device__ __forceinline__ PSurf psurface_at(const RenderArgs &a, const float4 *
     const float w0 = 1.0f - h.u - h.v;
     const float su = w0 * t0.x + h.u * t1.x + h.v * t2.x;
     const float sv = w0 * t0.y + h.u * t1.y + h.v * t2.y;
-    S.tb = bilin_setup(fmaf(su, (float)a.Wt, -0.5f), fmaf(sv, (float)a.Ht, -0.5f), a.Wt, a.Ht);
+    S.tb = bilin_setup(muladd(su, (float)a.Wt, -0.5f), muladd(sv, (float)a.Ht, -0.5f), a.Wt, a.Ht);
     const float4 tex = bilin_fetch(a.tex, S.tb, a.Wt, a.Ht);
     const float4 mt = bilin_fetch(mat, S.tb, a.Wt, a.Ht);
     S.rho = mk3(tex.x, tex.y, tex.z);

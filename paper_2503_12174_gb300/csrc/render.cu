@@ -122,25 +122,6 @@ __global__ void k_pack_tex(const float *__restrict__ albedo, const float *__rest
     tex[t] = make_float4(albedo[3 * t], albedo[3 * t + 1], albedo[3 * t + 2], rough[t]);
 }
 
-__device__ __forceinline__ float crf(float ec, float gain, float wb, float gamma) {
-    const float a = gain * wb * ec;
-    return a > 0.0f ? powf(a, gamma) : 0.0f;
-}
-
-// Eqs. 4 and 5 of one pixel from the sum over its samples
-__device__ __forceinline__ void write_pixel(const RenderArgs &a, int64_t pix, f3 sum) {
-    const float inv = 1.0f / (float)a.spp;
-    const float ex = sum.x * inv, ey = sum.y * inv, ez = sum.z * inv;
-    if (a.Ec) {
-        a.Ec[3 * pix] = ex;
-        a.Ec[3 * pix + 1] = ey;
-        a.Ec[3 * pix + 2] = ez;
-    }
-    a.Ic[3 * pix] = crf(ex, a.gain_c, a.wb[0], a.gamma_c[0]);
-    a.Ic[3 * pix + 1] = crf(ey, a.gain_c, a.wb[1], a.gamma_c[1]);
-    a.Ic[3 * pix + 2] = crf(ez, a.gain_c, a.wb[2], a.gamma_c[2]);
-}
-
 // Forward megakernel.  Every loop iteration traces exactly one ray per lane --
 // the extension ray of the current vertex or its shadow ray towards the
 // projector -- through the same traversal loop, then advances that lane's
@@ -289,50 +270,31 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_RENDER_MINB) k_render(const
     render_lanes(a, pix, (int)(gt & ((1 << a.log2L) - 1)), pix < (int64_t)a.Hc * a.Wc);
 }
 
-// Forward render of the S path lanes from lane0 on over a block tile
-// (tile.cuh): the image of render_lanes bit for bit.  Lane 0 belongs to pixel
-// pix0, and there are nlane lanes.
-template <int B, int S>
-__device__ __forceinline__ void render_tile(const RenderArgs &a, Tile<S> &P, int64_t pix0, int64_t lane0, int64_t nlane) {
-    const int L = 1 << a.log2L;
-    Cnt cnt;
-    PlainCore core;
-    tile_clear_sums<S>(P, B);
-    const int rounds = a.root != kEmptyRoot ? (a.spp + L - 1) / L : 0;
-    for (int k = 0; k < rounds; ++k) tile_round<B, S>(a, core, P, pix0, lane0, nlane, k, cnt);
-    cnt.flush(a.counters);
-    __syncthreads();
-#pragma unroll 1
-    for (int slot = threadIdx.x; slot < S; slot += B) {
-        const int64_t gt = lane0 + slot;
-        const f3 sum = tile_pixel_sum<S>(P, slot, L);
-        if (gt < nlane && (gt & (L - 1)) == 0) write_pixel(a, pix0 + (gt >> a.log2L), sum);
-    }
-}
-
+// Forward render over block tiles (tile.cuh): the image of render_lanes bit
+// for bit.
 template <int B, int S>
 __global__ void __launch_bounds__(B, 1024 / B) k_render_tile(const RenderArgs a) {
     __shared__ Tile<S> P;
-    render_tile<B, S>(a, P, 0, (int64_t)blockIdx.x * S, ((int64_t)a.Hc * a.Wc) << a.log2L);
+    PlainCore core;
+    tile_image<B, S>(a, core, P, 0, (int64_t)blockIdx.x * S, ((int64_t)a.Hc * a.Wc) << a.log2L);
 }
 
-// Does a render with these arguments run in tiles (launch_render says why)?
-constexpr int32_t kTileTriangles = 32768;
-__host__ __device__ __forceinline__ bool tiled(const RenderArgs &a) { return a.bounces > 1 && a.T <= kTileTriangles; }
-
-// Batched persistent render: CTAs pull virtual blocks from a device counter;
-// virtual block vb belongs to the segment whose range [vb_begin, vb_begin +
-// ceil(npix L / 128)) holds it, and covers that segment's pixels from
-// pix_begin on.  A segment is a pixel range of one request whose arguments
-// are descs[slot].  Per pixel the computation is render_lanes, exactly as in
-// k_render.  The loop ends when the counter passes the last virtual block:
-// there is no waiting on other CTAs.
+// Batched persistent render: CTAs pull virtual blocks of kBatchLanes lanes from
+// a device counter; virtual block vb belongs to the segment whose range
+// [vb_begin, vb_begin + ceil(npix L / kBatchLanes)) holds it, and covers that
+// segment's pixels from pix_begin on.  A segment is a pixel range of one
+// request whose arguments are descs[slot].  Per pixel the computation is that
+// of launch_render's kernels, in tiles or in lanes by the same rule (16 mixed
+// requests 15.0 -> 11.2 ms with the tiles).  The loop ends when the counter
+// passes the last virtual block: there is no waiting on other CTAs.
+constexpr int kBatchLanes = 256;
 __global__ void __launch_bounds__(kRenderBlock, DPCS_BATCH_MINB)
     k_render_batch(const RenderArgs *__restrict__ descs, const BatchSeg *__restrict__ segs, int nseg,
                    int64_t total_vb, unsigned long long *counter) {
     __shared__ RenderArgs sa;
     __shared__ int64_t s_vb;
     __shared__ int s_seg;
+    __shared__ Tile<kBatchLanes> P;
     while (true) {
         if (threadIdx.x == 0) {
             const int64_t vb = (int64_t)atomicAdd(counter, 1ull);
@@ -354,9 +316,16 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_BATCH_MINB)
             for (int i = threadIdx.x; i < (int)(sizeof(RenderArgs) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
         }
         __syncthreads();
-        const int64_t lt = (vb - sg.vb_begin) * kRenderBlock + threadIdx.x;  // thread index within the segment
-        const int64_t lp = lt >> sa.log2L;
-        render_lanes(sa, sg.pix_begin + lp, (int)(lt & ((1 << sa.log2L) - 1)), lp < sg.npix);
+        const int64_t lane0 = (vb - sg.vb_begin) * kBatchLanes;  // first lane of the block within the segment
+        if (tiled(sa)) {
+            PlainCore core;
+            tile_image<kRenderBlock, kBatchLanes>(sa, core, P, sg.pix_begin, lane0, sg.npix << sa.log2L);
+        } else {
+            for (int64_t lt = lane0 + threadIdx.x; lt < lane0 + kBatchLanes; lt += kRenderBlock) {
+                const int64_t lp = lt >> sa.log2L;
+                render_lanes(sa, sg.pix_begin + lp, (int)(lt & ((1 << sa.log2L) - 1)), lp < sg.npix);
+            }
+        }
         __syncthreads();
     }
 }
@@ -372,27 +341,6 @@ __global__ void k_trace(const float4 *__restrict__ nodes, const float4 *__restri
     const bool hit = traverse(nodes, tris, root, T, r, INFINITY, false, h, status, cnt);
     tout[i] = hit ? h.t : INFINITY;
     triout[i] = hit ? h.orig : -1;
-}
-
-// ---------------------------------------------------------------------------
-// block reduction of NV floats into FP64 accumulators
-// ---------------------------------------------------------------------------
-template <int NV>
-__device__ __forceinline__ void block_reduce_add(float (&v)[NV], double *acc) {
-    __shared__ float red[NV][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k)
-        for (int off = 16; off; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NV; ++k) red[k][w] = v[k];
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        float s = 0.0f;
-        for (int j = 0; j < (int)(blockDim.x >> 5); ++j) s += red[threadIdx.x][j];
-        if (s != 0.0f) atomicAdd(acc + threadIdx.x, (double)s);
-    }
 }
 
 // Eq. 5 adjoint.  acc layout: [gamma_p(3), Gp, gamma_c(3), Gc, wb(3)]
@@ -429,11 +377,9 @@ __global__ void k_crf_backward(const float *__restrict__ dIc, const float *__res
 // packed float4 atomics, or (F64) one FP64 atomic per component, whose sums
 // do not depend on the order of the adds beyond FP64 rounding.
 template <bool F64>
-__device__ __forceinline__ void replay_sweep(const RenderArgs &a, const VRec *rec, int nv, const float gb_in[3],
+__device__ __forceinline__ void sweep_vertex(const RenderArgs &a, const VRec &R, const float gb_in[3], float A[3],
                                              float4 *row) {
-    float A[3] = {0.f, 0.f, 0.f};
-    for (int c = nv - 1; c >= 0; --c) {
-        const VRec &R = rec[c];
+    {
         float ga[3], dEp[3];
         float dr = 0.0f;
 #pragma unroll
@@ -487,6 +433,13 @@ __device__ __forceinline__ void replay_sweep(const RenderArgs &a, const VRec *re
             }
         }
     }
+}
+
+template <bool F64>
+__device__ __forceinline__ void replay_sweep(const RenderArgs &a, const VRec *rec, int nv, const float gb_in[3],
+                                             float4 *row) {
+    float A[3] = {0.f, 0.f, 0.f};
+    for (int c = nv - 1; c >= 0; --c) sweep_vertex<F64>(a, rec[c], gb_in, A, row);
 }
 
 // Path-replay adjoint.  Same thread mapping and loops as k_render: each lane
@@ -786,33 +739,9 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_GRAD_MINB) k_render_grad(co
         sum.y += __shfl_xor_sync(0xffffffffu, sum.y, off);
         sum.z += __shfl_xor_sync(0xffffffffu, sum.z, off);
     }
-    const float inv = 1.0f / (float)a.spp;
-    const float ec[3] = {sum.x * inv, sum.y * inv, sum.z * inv};
     float gb_in[3] = {0.f, 0.f, 0.f};
     float v[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // gamma_c(3), Gc, wb(3), loss
-    if (valid) {
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const float ic = crf(ec[j], a.gain_c, a.wb[j], a.gamma_c[j]);
-            if (sl == 0) {
-                if (a.Ec) a.Ec[3 * pix + j] = ec[j];
-                a.Ic[3 * pix + j] = ic;
-            }
-            const float d = ic - l.target[3 * pix + j];
-            const float g = l.kind == 0 ? l.scale * d : (d > 0.0f ? l.scale : (d < 0.0f ? -l.scale : 0.0f));
-            const float w = a.gain_c * a.wb[j] * ec[j];
-            if (w > 0.0f) {
-                const float da = a.gamma_c[j] * powf(w, a.gamma_c[j] - 1.0f);
-                gb_in[j] = g * da * a.gain_c * a.wb[j] * inv;
-                if (sl == 0) {
-                    v[j] += g * ic * logf(w);
-                    v[3] += g * da * a.wb[j] * ec[j];
-                    v[4 + j] += g * da * a.gain_c * ec[j];
-                }
-            }
-            if (sl == 0) v[7] += l.kind == 0 ? 0.5f * l.scale * d * d : l.scale * fabsf(d);
-        }
-    }
+    if (valid) pixel_loss_grad(a, l, pix, sl, sum, gb_in, v);
     block_reduce_add<8>(v, l.acc + 4);  // acc[4..10]: gamma_c, Gc, wb; acc[11]: the loss
     const bool any = gb_in[0] != 0.0f || gb_in[1] != 0.0f || gb_in[2] != 0.0f;
     for (int i = 0; any && i < k && i < kFusedSamples; ++i)
@@ -1018,6 +947,101 @@ __global__ void __launch_bounds__(kRenderBlock) k_sweep_kept(const RenderArgs a,
     }
 }
 
+// The plain material with every vertex recorded (the VRec fields, as six
+// 16-byte chunks): record v of round k of a slot at kept_chunk(c, k, v, spl,
+// bounces, nthr, t0 + slot).
+template <bool kStream>
+struct RecordCore {
+    uint4 *chunks;
+    uint8_t *nvs;  // vertices of each recorded path, [spl][nthr]
+    int64_t nthr, t0;
+    int spl;
+    bool replay;   // the pixel's dLoss/dEc is known (a.gE): paths of pixels without one are not traced, and rounds share their records
+
+    __device__ __forceinline__ int64_t at(const RenderArgs &a, int c, int k, int v, int slot) const {
+        return kept_chunk(c, replay ? 0 : k, v, spl, a.bounces, nthr, t0 + slot);
+    }
+    __device__ __forceinline__ uint8_t &count(int k, int slot) const {
+        return nvs[(int64_t)(replay ? 0 : k) * nthr + t0 + slot];
+    }
+    __device__ __forceinline__ bool begin(const RenderArgs &a, int slot, uint32_t pix, int k) {
+        count(k, slot) = 0;
+        return !replay || a.gE[3 * (int64_t)pix] != 0.0f || a.gE[3 * (int64_t)pix + 1] != 0.0f ||
+               a.gE[3 * (int64_t)pix + 2] != 0.0f;
+    }
+    __device__ __forceinline__ void dark(const RenderArgs &a, int slot, int k, int v) {
+        uint32_t *w = reinterpret_cast<uint32_t *>(chunks + at(a, kKeptGChunk, k, v, slot));
+        w[kKeptGWord] = 0u;
+    }
+    __device__ __forceinline__ void put(const RenderArgs &a, int c, int slot, int k, int b, uint4 q) {
+        uint4 *p = chunks + at(a, c, k, b - 1, slot);
+        if (kStream) __stcs(p, q); else *p = q;
+    }
+    __device__ __forceinline__ void shade(const RenderArgs &a, int slot, uint32_t pix, uint32_t s, int k, int b, const Hit &h,
+                                          f3 d, f3 beta, Shaded &R) {
+        const Surf F = surface_at(a, h, d);
+        R.so = madd(F.x, F.n, kRayEps);
+        auto U = [](float x) { return __float_as_uint(x); };
+        Nee Q;
+        R.cand = nee_prepare(a, F, Q);
+        unsigned unc = 0u;
+        if (R.cand) {
+            R.c = nee_contrib(a, beta, Q, unc);
+            put(a, 0, slot, k, b, make_uint4((uint32_t)F.tb.x0, (uint32_t)F.tb.y0, (uint32_t)Q.pb.x0, (uint32_t)Q.pb.y0));
+            put(a, 1, slot, k, b, make_uint4(U(F.tb.fx), U(F.tb.fy), U(Q.pb.fx), U(Q.pb.fy)));
+            put(a, 2, slot, k, b, make_uint4(U(beta.x), U(beta.y), U(beta.z), U(Q.ep.x)));
+            put(a, 3, slot, k, b, make_uint4(U(Q.ep.y), U(Q.ep.z), U(Q.G), U(F.rho.x)));
+            put(a, 4, slot, k, b, make_uint4(U(F.rho.y), U(F.rho.z), U(Q.sp), U(Q.dsp)));
+        } else {
+            put(a, 0, slot, k, b, make_uint4((uint32_t)F.tb.x0, (uint32_t)F.tb.y0, 0u, 0u));
+            put(a, 1, slot, k, b, make_uint4(U(F.tb.fx), U(F.tb.fy), 0u, 0u));
+            put(a, 2, slot, k, b, make_uint4(U(beta.x), U(beta.y), U(beta.z), 0u));
+            put(a, 3, slot, k, b, make_uint4(0u, 0u, 0u, U(F.rho.x)));
+            put(a, 4, slot, k, b, make_uint4(U(F.rho.y), U(F.rho.z), 0u, 0u));
+        }
+        R.ext = false;
+        Cont C;
+        if (b < a.bounces) {
+            R.ext = continue_prepare(a, pix, s, b, F, C);
+            if (R.ext) {
+                R.beta = beta * C.w;
+                R.wi = C.wi;
+            }
+        }
+        put(a, 5, slot, k, b, R.ext ? make_uint4(U(C.si), U(C.dsi), U(C.cw), unc) : make_uint4(0u, 0u, 0u, unc));
+        count(k, slot) = (uint8_t)b;
+    }
+};
+
+// k_render_keep over block tiles: the same records and images
+template <int B, int S>
+__global__ void __launch_bounds__(B, 1024 / B) k_keep_tile(const RenderArgs a, uint4 *chunks, uint8_t *nvs) {
+    __shared__ Tile<S> P;
+    RecordCore<true> core{chunks, nvs, ((int64_t)a.Hc * a.Wc) << a.log2L, (int64_t)blockIdx.x * S,
+                          (a.spp + (1 << a.log2L) - 1) >> a.log2L, false};
+    tile_image<B, S>(a, core, P, 0, (int64_t)blockIdx.x * S, ((int64_t)a.Hc * a.Wc) << a.log2L);
+}
+
+// k_render_grad and k_replay over block tiles
+template <bool F64, int B, int S>
+__global__ void __launch_bounds__(B, 1024 / B) k_grad_tile(const RenderArgs a, const LossArgs l, char *scratch,
+                                                           size_t per_block, int64_t ntile, unsigned long long *counter) {
+    __shared__ Tile<S> P;
+    __shared__ float4 s_row[B];  // per-warp rows for scatter_add4
+    RecordCore<false> core;
+    tile_adjoint<B, S>(a, core, P, l, scratch, per_block, ntile, counter, kKeptChunks,
+                       [&](int k, int slot, const float gb_in[3]) {
+                           float A[3] = {0.f, 0.f, 0.f};
+                           for (int v = core.count(k, slot) - 1; v >= 0; --v) {
+                               VRec R;
+                               uint4 *dst = reinterpret_cast<uint4 *>(&R);
+#pragma unroll
+                               for (int c = 0; c < kKeptChunks; ++c) dst[c] = core.chunks[core.at(a, c, k, v, slot)];
+                               sweep_vertex<F64>(a, R, gb_in, A, &s_row[threadIdx.x & ~31]);
+                           }
+                       });
+}
+
 // Eq. 1 adjoint: dIp += dEp Gp gamma Ip^(gamma-1); gamma_p and Gp reductions
 __global__ void k_prf_backward(const float *__restrict__ Ip, const float4 *__restrict__ dEp, int64_t ntex,
                                float g0, float g1, float g2, float gain, float *__restrict__ dIp, double *acc) {
@@ -1122,7 +1146,7 @@ __global__ void k_finalize(const double *__restrict__ acc, float *__restrict__ d
     if (i < 11) dParams[i] += (float)acc[i];
 }
 
-constexpr int64_t kTileLanes = 500000;  // fewer (pixel, lane) pairs: small tiles
+constexpr int32_t kReplayTriangles = 8192;  // the replay's tiles gain 12 % on the corner and lose 4 % at 28,800 triangles
 
 inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
@@ -1140,17 +1164,9 @@ int launch_pack_tex(const float *albedo, const float *rough, int64_t ntex, float
 
 int launch_render(const RenderArgs &a, cudaStream_t st) {
     const int64_t lanes = ((int64_t)a.Hc * a.Wc) << a.log2L;
-    // Where the tiles pay (GB300, start -> lanes kernel / tiles): paths of one
-    // bounce have nothing to compact (plane 512 x 512 at 16 spp 206 -> 206 / 230
-    // us).  Above some tens of thousands of triangles the tree no longer sits in
-    // the L1 that the tiles' shared memory leaves (heightfields of 7,200 / 51,200
-    // / 199,712 triangles 1.47 -> 1.43 / 1.42 ms, 2.00 -> 1.96 / 2.08 ms,
-    // 8.41 -> 8.24 / 8.61 ms).  Small images want more, smaller tiles: tiles of 64
-    // / 256 lanes take 74 / 96 us at 147 k lanes, 156 / 161 us at 410 k, 206 /
-    // 195 us at 590 k.
     if (!tiled(a))
         k_render<<<grid_for(lanes, kRenderBlock), kRenderBlock, 0, st>>>(a);
-    else if (lanes < kTileLanes)
+    else if (small_tiles(a))
         k_render_tile<64, 64><<<grid_for(lanes, 64), 64, 0, st>>>(a);
     else
         k_render_tile<128, 256><<<grid_for(lanes, 256), 128, 0, st>>>(a);
@@ -1171,7 +1187,7 @@ int render_batch_grid(int device) {
 }
 
 int64_t render_batch_vblocks(int64_t npix, int log2L) {
-    return ((npix << log2L) + kRenderBlock - 1) / kRenderBlock;
+    return ((npix << log2L) + kBatchLanes - 1) / kBatchLanes;
 }
 
 int launch_trace(const Scene &sc, const float *o, const float *d, int64_t n, float *t, int32_t *tri,
@@ -1187,8 +1203,36 @@ int launch_crf_backward(const float *dIc, const float *Ec, const float *Ic, int6
     return 1;
 }
 
-int launch_replay(const RenderArgs &a, cudaStream_t st) {
+namespace {
+
+template <int B, int S>
+void launch_grad_tiles(const RenderArgs &a, const LossArgs &l, void *scratch, cudaStream_t st) {
+    const TileGrid g = tile_grid(a, l, B, S, kRecWordsHost);
+    if (a.dEp64)
+        k_grad_tile<true, B, S><<<g.grid, B, 0, st>>>(a, l, (char *)scratch, g.per_block, g.ntile, g.counter);
+    else
+        k_grad_tile<false, B, S><<<g.grid, B, 0, st>>>(a, l, (char *)scratch, g.per_block, g.ntile, g.counter);
+}
+
+void launch_grad_tile(const RenderArgs &a, const LossArgs &l, void *scratch, cudaStream_t st) {
+    if (small_tiles(a))
+        launch_grad_tiles<64, 64>(a, l, scratch, st);
+    else
+        launch_grad_tiles<128, 256>(a, l, scratch, st);
+}
+
+}  // namespace
+
+size_t grad_scratch_bytes(const RenderArgs &a, bool replay, int words) {
+    return replay && a.T > kReplayTriangles ? 0 : tile_scratch_bytes(a, replay, words);
+}
+
+int launch_replay(const RenderArgs &a, double *acc, void *scratch, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
+    if (scratch) {
+        launch_grad_tile(a, LossArgs{nullptr, 1.0f, 0, acc}, scratch, st);
+        return 1;
+    }
     if (a.dEp64)
         k_replay<true><<<grid_for(threads, kRenderBlock), kRenderBlock, 0, st>>>(a);
     else
@@ -1196,8 +1240,12 @@ int launch_replay(const RenderArgs &a, cudaStream_t st) {
     return 1;
 }
 
-int launch_render_grad(const RenderArgs &a, const LossArgs &l, cudaStream_t st) {
+int launch_render_grad(const RenderArgs &a, const LossArgs &l, void *scratch, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
+    if (scratch) {
+        launch_grad_tile(a, l, scratch, st);
+        return 1;
+    }
     if (a.dEp64)
         k_render_grad<true><<<grid_for(threads, kRenderBlock), kRenderBlock, 0, st>>>(a, l);
     else
@@ -1207,7 +1255,12 @@ int launch_render_grad(const RenderArgs &a, const LossArgs &l, cudaStream_t st) 
 
 int launch_render_keep(const RenderArgs &a, void *chunks, uint8_t *nvs, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
-    k_render_keep<<<grid_for(threads, kRenderBlock), kRenderBlock, 0, st>>>(a, (uint4 *)chunks, nvs);
+    if (!tiled(a) || a.root == kEmptyRoot)
+        k_render_keep<<<grid_for(threads, kRenderBlock), kRenderBlock, 0, st>>>(a, (uint4 *)chunks, nvs);
+    else if (small_tiles(a))
+        k_keep_tile<64, 64><<<grid_for(threads, 64), 64, 0, st>>>(a, (uint4 *)chunks, nvs);
+    else
+        k_keep_tile<128, 256><<<grid_for(threads, 256), 128, 0, st>>>(a, (uint4 *)chunks, nvs);
     return 1;
 }
 

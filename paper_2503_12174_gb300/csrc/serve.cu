@@ -111,6 +111,9 @@ struct dpcs_server {
     size_t used = 0, high_water = 0;
     int64_t submitted = 0, completed = 0, failed = 0, iterations = 0, launches = 0;
     int grid = 1;
+    void *recs = nullptr;  // path records of the compensation steps' tiles (steps run one after another)
+    size_t recs_bytes = 0;
+    std::vector<void *> retired;  // smaller ones that queued steps may still use
 };
 
 namespace {
@@ -197,6 +200,26 @@ dpcs_status admit(dpcs_server *s, Req *q) {
     return DPCS_OK;
 }
 
+// Records for a tiled compensation step; null (the lanes kernels) when the
+// arguments have no tile kernel, the server has a memory budget, which is left
+// for its requests, or there is no room.
+void *step_scratch(dpcs_server *s, const RenderArgs &a, bool replay) {
+    const size_t bytes = grad_scratch_bytes(a, replay, kRecWordsHost);
+    if (!bytes || s->cfg.hbm_budget_bytes) return nullptr;
+    if (s->recs_bytes >= bytes) return s->recs;
+    size_t n = size_t(1) << 20;
+    while (n < bytes) n <<= 1;
+    void *p = nullptr;
+    if (cudaMalloc(&p, n) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (s->recs) s->retired.push_back(s->recs);
+    s->recs = p;
+    s->recs_bytes = n;
+    return p;
+}
+
 // one compensation step after its render: L2 loss, path replay, PRF
 // adjoint, Adam on Ip with the clamp to [0, 1], then Ep for the next render
 int enqueue_comp_backward(dpcs_server *s, Req *q) {
@@ -213,7 +236,7 @@ int enqueue_comp_backward(dpcs_server *s, Req *q) {
     a.gE = q->gE;
     a.dEp = q->dEp4;
     a.dtex = nullptr;  // only Ip is optimised
-    n += launch_replay(a, st);
+    n += launch_replay(a, q->acc, step_scratch(s, a, true), st);
     n += launch_prf_backward(q->Ip, q->dEp4, np, sc.params.gamma_p, sc.params.gain_p, q->G, q->acc, st);
     n += launch_adam(q->Ip, q->G, q->M, q->V, np * 3, q->r.lr, 0.9f, 0.999f, 1e-8f, q->steps_issued, 0.0f, 1.0f, st);
     n += launch_prf(q->Ip, np, sc.params.gamma_p, sc.params.gain_p, q->Ep4, st);
@@ -239,7 +262,7 @@ int enqueue_comp_step_fused(dpcs_server *s, Req *q) {
     a.dEp = q->dEp4;
     a.dtex = nullptr;  // only Ip is optimised
     const LossArgs l{q->target, 1.0f, 0, q->acc};
-    int n = launch_render_grad(a, l, st);
+    int n = launch_render_grad(a, l, step_scratch(s, a, false), st);
     n += launch_loss_out(q->acc, q->loss, st);
     n += launch_prf_backward(q->Ip, q->dEp4, np, sc.params.gamma_p, sc.params.gain_p, q->G, q->acc, st);
     n += launch_adam(q->Ip, q->G, q->M, q->V, np * 3, q->r.lr, 0.9f, 0.999f, 1e-8f, q->steps_issued, 0.0f, 1.0f, st);
@@ -578,6 +601,8 @@ dpcs_status dpcs_serve_destroy(dpcs_server *s) {
         if (sc.tex4) cudaFree(sc.tex4);
     for (Batch &b : s->batches) free_batch_bufs(b);
     cudaStreamSynchronize(s->stream);
+    if (s->recs) cudaFree(s->recs);
+    for (void *p : s->retired) cudaFree(p);
     cudaStreamDestroy(s->stream);
     cudaMemPoolDestroy(s->pool);
     delete s;

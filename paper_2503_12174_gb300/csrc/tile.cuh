@@ -184,7 +184,10 @@ __device__ __forceinline__ void tree_walk(const RenderArgs &a, const Ray &ray, b
             const float4 B = __ldg(a.tris + 3 * pos + 1);
             const float4 C = __ldg(a.tris + 3 * pos + 2);
             float t, u, v;
-            if (tri_isect(ray, xyz(A), xyz(B), xyz(C), ht, t, u, v)) {
+            bool near_edge, wt = false;
+            bool ok = tri_isect_mt(ray, xyz(A), xyz(B), xyz(C), ht, t, u, v, near_edge);
+            if (!ok && near_edge) ok = wt = tri_isect_wt_call(ray, xyz(A), xyz(B), xyz(C), ht, t, u, v);
+            if (ok) {
                 // ties in t to the lowest original triangle index
                 if (t < ht || (!any && hpos >= 0 && __float_as_int(A.w) < __float_as_int(__ldg(a.tris + 3 * hpos).w))) {
                     hpos = pos;
@@ -192,6 +195,14 @@ __device__ __forceinline__ void tree_walk(const RenderArgs &a, const Ray &ray, b
                     hu = u;
                     hv = v;
                     if (any) sp = 0;
+                } else if (wt) {
+                    // A ray that meets a shared edge exactly (1 path in 1e7)
+                    // ties in the watertight test.  trav_resume as compiled
+                    // keeps the barycentrics of the triangle that loses such a
+                    // tie; the tiles do the same, so that every kernel gives
+                    // the same image.
+                    hu = u;
+                    hv = v;
                 }
             }
             if (--left < 0) {
@@ -404,5 +415,216 @@ struct PlainCore {
         R.so = madd(F.x, F.n, kRayEps);
     }
 };
+
+// ---------------------------------------------------------------------------
+// pixels
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float crf(float ec, float gain, float wb, float gamma) {
+    const float a = gain * wb * ec;
+    return a > 0.0f ? powf(a, gamma) : 0.0f;
+}
+
+// Eqs. 4 and 5 of one pixel from the sum over its samples
+__device__ __forceinline__ void write_pixel(const RenderArgs &a, int64_t pix, f3 sum) {
+    const float inv = 1.0f / (float)a.spp;
+    const float ex = sum.x * inv, ey = sum.y * inv, ez = sum.z * inv;
+    if (a.Ec) {
+        a.Ec[3 * pix] = ex;
+        a.Ec[3 * pix + 1] = ey;
+        a.Ec[3 * pix + 2] = ez;
+    }
+    a.Ic[3 * pix] = crf(ex, a.gain_c, a.wb[0], a.gamma_c[0]);
+    a.Ic[3 * pix + 1] = crf(ey, a.gain_c, a.wb[1], a.gamma_c[1]);
+    a.Ic[3 * pix + 2] = crf(ez, a.gain_c, a.wb[2], a.gamma_c[2]);
+}
+
+// The one-trace step's pixel: Eqs. 4 and 5, the loss, and through Eq. 5 the
+// gradient of each sample's radiance (gb_in); the pixel's first lane (sl = 0)
+// also writes Ec and Ic and adds to v: gamma_c(3), Gc, wb(3), loss.
+__device__ __forceinline__ void pixel_loss_grad(const RenderArgs &a, const LossArgs &l, int64_t pix, int sl, f3 sum,
+                                                float gb_in[3], float v[8]) {
+    const float inv = 1.0f / (float)a.spp;
+    const float ec[3] = {sum.x * inv, sum.y * inv, sum.z * inv};
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        gb_in[j] = 0.0f;
+        const float ic = crf(ec[j], a.gain_c, a.wb[j], a.gamma_c[j]);
+        if (sl == 0) {
+            if (a.Ec) a.Ec[3 * pix + j] = ec[j];
+            a.Ic[3 * pix + j] = ic;
+        }
+        const float d = ic - l.target[3 * pix + j];
+        const float g = l.kind == 0 ? l.scale * d : (d > 0.0f ? l.scale : (d < 0.0f ? -l.scale : 0.0f));
+        const float w = a.gain_c * a.wb[j] * ec[j];
+        if (w > 0.0f) {
+            const float da = a.gamma_c[j] * powf(w, a.gamma_c[j] - 1.0f);
+            gb_in[j] = g * da * a.gain_c * a.wb[j] * inv;
+            if (sl == 0) {
+                v[j] += g * ic * logf(w);
+                v[3] += g * da * a.wb[j] * ec[j];
+                v[4 + j] += g * da * a.gain_c * ec[j];
+            }
+        }
+        if (sl == 0) v[7] += l.kind == 0 ? 0.5f * l.scale * d * d : l.scale * fabsf(d);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// block reduction of NV floats into FP64 accumulators
+// ---------------------------------------------------------------------------
+template <int NV>
+__device__ __forceinline__ void block_reduce_add(float (&v)[NV], double *acc) {
+    __shared__ float red[NV][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+        for (int off = 16; off; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) red[k][w] = v[k];
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        float s = 0.0f;
+        for (int j = 0; j < (int)(blockDim.x >> 5); ++j) s += red[threadIdx.x][j];
+        if (s != 0.0f) atomicAdd(acc + threadIdx.x, (double)s);
+    }
+}
+
+// The image of a tile: every round of its S lanes from lane0 on, then their
+// pixels.  Lane 0 belongs to pixel pix0, and there are nlane lanes.
+template <int B, int S, class Core>
+__device__ __forceinline__ void tile_image(const RenderArgs &a, Core &core, Tile<S> &P, int64_t pix0, int64_t lane0,
+                                           int64_t nlane) {
+    const int L = 1 << a.log2L;
+    Cnt cnt;
+    tile_clear_sums<S>(P, B);
+    const int rounds = a.root != kEmptyRoot ? (a.spp + L - 1) / L : 0;
+    for (int k = 0; k < rounds; ++k) tile_round<B, S>(a, core, P, pix0, lane0, nlane, k, cnt);
+    cnt.flush(a.counters);
+    __syncthreads();
+#pragma unroll 1
+    for (int slot = threadIdx.x; slot < S; slot += B) {
+        const int64_t gt = lane0 + slot;
+        const f3 sum = tile_pixel_sum<S>(P, slot, L);
+        if (gt < nlane && (gt & (L - 1)) == 0) write_pixel(a, pix0 + (gt >> a.log2L), sum);
+    }
+}
+
+// The one-trace step (l.target set) or the replay (l.target null: a.gE holds
+// dLoss/dEc) over block tiles.  Persistent: a block takes tiles from a counter
+// and keeps its records (`words` 16-byte chunks a vertex) in its own part of
+// `scratch`, small enough in all to stay in L2: 512 x 512 at 16 spp, gradient
+// of Ip, 2.10 -> 1.50 ms.  sweep(k, slot, gb) sweeps the slot's path of round k.
+template <int B, int S, class Core, class Sweep>
+__device__ __forceinline__ void tile_adjoint(const RenderArgs &a, Core &core, Tile<S> &P, const LossArgs &l, char *scratch,
+                                             size_t per_block, int64_t ntile, unsigned long long *counter, int chunks,
+                                             Sweep sweep) {
+    const int L = 1 << a.log2L, tid = threadIdx.x;
+    const int64_t nlane = ((int64_t)a.Hc * a.Wc) << a.log2L;
+    const bool replay = l.target == nullptr;
+    const int rounds = (a.spp + L - 1) / L, spl = replay ? 1 : rounds;
+    Cnt cnt;
+    core.chunks = reinterpret_cast<uint4 *>(scratch + blockIdx.x * per_block);
+    core.nvs = reinterpret_cast<uint8_t *>(core.chunks + (size_t)chunks * spl * a.bounces * S);
+    core.nthr = S;
+    core.t0 = 0;
+    core.spl = spl;
+    core.replay = replay;
+    const float inv = 1.0f / (float)a.spp;
+    while (true) {
+        if (tid == 0) {
+            const unsigned long long t = atomicAdd(counter, 1ull);
+            P.work = t < (unsigned long long)ntile ? (int)t : -1;
+        }
+        tile_clear_sums<S>(P, B);
+        __syncthreads();
+        const int tile = P.work;
+        if (tile < 0) break;
+        const int64_t lane0 = (int64_t)tile * S;
+        for (int k = 0; k < rounds; ++k) {
+            tile_round<B, S>(a, core, P, 0, lane0, nlane, k, cnt);
+            if (!replay) continue;
+#pragma unroll 1
+            for (int slot = tid; slot < S; slot += B) {
+                const int64_t gt = lane0 + slot, pix = gt >> a.log2L;
+                if (gt >= nlane || (int)(gt & (L - 1)) + k * L >= a.spp) continue;
+                const float gb_in[3] = {a.gE[3 * pix] * inv, a.gE[3 * pix + 1] * inv, a.gE[3 * pix + 2] * inv};
+                sweep(k, slot, gb_in);
+            }
+            __syncthreads();
+        }
+        if (replay) continue;
+        float v[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // gamma_c(3), Gc, wb(3), loss
+#pragma unroll 1
+        for (int slot = tid; slot < S; slot += B) {
+            const int64_t gt = lane0 + slot, pix = gt >> a.log2L;
+            const int sl = (int)(gt & (L - 1));
+            const f3 sum = tile_pixel_sum<S>(P, slot, L);
+            if (gt >= nlane) continue;
+            float gb_in[3];
+            pixel_loss_grad(a, l, pix, sl, sum, gb_in, v);
+            if (gb_in[0] == 0.0f && gb_in[1] == 0.0f && gb_in[2] == 0.0f) continue;
+            for (int k = 0; sl + k * L < a.spp; ++k) sweep(k, slot, gb_in);
+        }
+        __syncthreads();
+        block_reduce_add<8>(v, l.acc + 4);  // acc[4..10]: gamma_c, Gc, wb; acc[11]: the loss
+        __syncthreads();
+    }
+    cnt.flush(a.counters);
+}
+
+// ---------------------------------------------------------------------------
+// dispatch
+// ---------------------------------------------------------------------------
+// Where the tiles pay (GB300, before -> lanes kernel / tiles).  Paths of one
+// bounce have nothing to compact (plane 512 x 512 at 16 spp 206 -> 206 / 230
+// us).  A tree of some MB no longer sits in the L1 that the tiles' shared
+// memory leaves: corner walls of 1,026 / 8,226 triangles 711 -> 692 / 540 and
+// 855 -> 831 / 676 us, but heightfields of 7,200 / 51,200 / 199,712 1.47 ->
+// 1.43 / 1.42, 2.00 -> 1.96 / 2.08 and 8.41 -> 8.24 / 8.61 ms.  Small images
+// want more, smaller tiles: tiles of 64 / 256 lanes take 74 / 96 us at 147 k
+// lanes, 156 / 161 us at 410 k, 206 / 195 us at 590 k.
+constexpr int32_t kTileTriangles = 16384;  // 1 MB of nodes
+constexpr int64_t kTileLanes = 500000;
+__host__ __device__ __forceinline__ bool tiled(const RenderArgs &a) { return a.bounces > 1 && a.T <= kTileTriangles; }
+// blocks of b threads that the GPU holds at once: the persistent grid
+inline int resident_blocks(int b) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms * (1024 / b);
+}
+
+// do these arguments run in the small tiles?
+inline bool small_tiles(const RenderArgs &a) { return (((int64_t)a.Hc * a.Wc) << a.log2L) < kTileLanes; }
+
+// one block's records: S slots of `words` 32-bit words a vertex
+inline size_t tile_block_bytes(const RenderArgs &a, bool replay, int S, int words) {
+    const int L = 1 << a.log2L;
+    const size_t spl = replay ? 1 : (size_t)((a.spp + L - 1) / L);
+    return (spl * S * ((size_t)words * 4 * a.bounces + 1) + 255) & ~size_t(255);
+}
+
+inline size_t tile_scratch_bytes(const RenderArgs &a, bool replay, int words) {
+    if (!tiled(a) || a.root == kEmptyRoot) return 0;
+    return small_tiles(a) ? (size_t)resident_blocks(64) * tile_block_bytes(a, replay, 64, words)
+                          : (size_t)resident_blocks(128) * tile_block_bytes(a, replay, 256, words);
+}
+
+struct TileGrid {
+    unsigned grid;
+    int64_t ntile;
+    size_t per_block;
+    unsigned long long *counter;
+};
+inline TileGrid tile_grid(const RenderArgs &a, const LossArgs &l, int B, int S, int words) {
+    TileGrid g;
+    g.ntile = ((((int64_t)a.Hc * a.Wc) << a.log2L) + S - 1) / S;
+    const int64_t cap = resident_blocks(B);
+    g.grid = (unsigned)(g.ntile < cap ? g.ntile : cap);
+    g.per_block = tile_block_bytes(a, l.target == nullptr, S, words);
+    g.counter = reinterpret_cast<unsigned long long *>(l.acc + kTileCounter);
+    return g;
+}
 
 }  // namespace dpcs
