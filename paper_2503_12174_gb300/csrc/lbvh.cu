@@ -14,46 +14,54 @@ namespace {
 
 constexpr int kSortTile = 256;  // items (and threads) per radix-sort block
 
-// centroids (v0 + v1 + v2) * (1/3) in FP32 without contraction
-__global__ void k_centroids(const float *__restrict__ verts, const int32_t *__restrict__ tris, int T,
-                            float *__restrict__ cen) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T) return;
-    const float third = 1.0f / 3.0f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float a = verts[3 * tris[3 * i] + k], b = verts[3 * tris[3 * i + 1] + k], c = verts[3 * tris[3 * i + 2] + k];
-        cen[3 * i + k] = __fmul_rn(__fadd_rn(__fadd_rn(a, b), c), third);
-    }
+// floats as unsigned integers in the same order, for atomic min / max
+__device__ __forceinline__ uint32_t ordered(float f) {
+    const uint32_t u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float unordered(uint32_t u) {
+    return __uint_as_float((u & 0x80000000u) ? u & 0x7fffffffu : ~u);
 }
 
-// single-block min/max of the centroids -> bounds[0..2] lo, [3..5] hi
-__global__ void k_bounds(const float *__restrict__ cen, int T, float *__restrict__ bounds) {
-    __shared__ float slo[3][32], shi[3][32];
+// centroids (v0 + v1 + v2) * (1/3) in FP32 without contraction, and their
+// bounds -> bounds[0..2] lo (set to all ones before), [3..5] hi (set to zero
+// before), as ordered integers.  min and max do not depend on the order.
+__global__ void __launch_bounds__(256) k_centroids(const float *__restrict__ verts, const int32_t *__restrict__ tris,
+                                                   int T, float *__restrict__ cen, uint32_t *__restrict__ bounds) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const float third = 1.0f / 3.0f;
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int i = threadIdx.x; i < T; i += blockDim.x)
+    if (i < T) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            lo[k] = fminf(lo[k], cen[3 * i + k]);
-            hi[k] = fmaxf(hi[k], cen[3 * i + k]);
+            const float a = verts[3 * tris[3 * i] + k], b = verts[3 * tris[3 * i + 1] + k],
+                        c = verts[3 * tris[3 * i + 2] + k];
+            lo[k] = hi[k] = cen[3 * i + k] = __fmul_rn(__fadd_rn(__fadd_rn(a, b), c), third);
         }
+    }
+    __shared__ float slo[3][8], shi[3][8];
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 3; ++k) {
         for (int off = 16; off; off >>= 1) {
             lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], off));
             hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], off));
         }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0)
-        for (int k = 0; k < 3; ++k) { slo[k][w] = lo[k]; shi[k][w] = hi[k]; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < 3; ++k) {
-            float a = INFINITY, b = -INFINITY;
-            for (int j = 0; j < (int)(blockDim.x >> 5); ++j) { a = fminf(a, slo[k][j]); b = fmaxf(b, shi[k][j]); }
-            bounds[k] = a;
-            bounds[3 + k] = b;
+        if (l == 0) {
+            slo[k][w] = lo[k];
+            shi[k][w] = hi[k];
         }
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const int k = threadIdx.x;
+        float a = INFINITY, b = -INFINITY;
+        for (int j = 0; j < 8; ++j) {
+            a = fminf(a, slo[k][j]);
+            b = fmaxf(b, shi[k][j]);
+        }
+        atomicMin(bounds + k, ordered(a));
+        atomicMax(bounds + 3 + k, ordered(b));
     }
 }
 
@@ -67,14 +75,14 @@ __device__ __forceinline__ uint32_t expand10(uint32_t v) {
 }
 
 // 30-bit Morton code of the centroid normalised into the centroid bounds
-__global__ void k_morton(const float *__restrict__ cen, const float *__restrict__ bounds, int T,
+__global__ void k_morton(const float *__restrict__ cen, const uint32_t *__restrict__ bounds, int T,
                          uint32_t *__restrict__ codes, int32_t *__restrict__ idx) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= T) return;
     uint32_t q[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const float lo = bounds[k], ext = __fsub_rn(bounds[3 + k], lo);
+        const float lo = unordered(bounds[k]), ext = __fsub_rn(unordered(bounds[3 + k]), lo);
         const float inv = ext > 0.0f ? __frcp_rn(ext) : 0.0f;
         const float nrm = __fmul_rn(__fsub_rn(cen[3 * i + k], lo), inv);
         float f = floorf(__fmul_rn(nrm, 1024.0f));
@@ -97,33 +105,50 @@ __global__ void k_radix_hist(const uint32_t *__restrict__ keys, int n, int shift
     hist[threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
 }
 
-// exclusive scan of `total` counters in one block
-__global__ void k_radix_scan(uint32_t *__restrict__ hist, int total) {
-    __shared__ uint32_t part[1024];
-    const int per = (total + blockDim.x - 1) / blockDim.x;
-    const int b0 = threadIdx.x * per;
-    uint32_t s = 0;
-    for (int i = b0; i < min(b0 + per, total); ++i) s += hist[i];
-    part[threadIdx.x] = s;
+// exclusive prefix of v over a block of 256 threads; total: the block's sum
+__device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t &total) {
+    __shared__ uint32_t ws[8];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t x = v;
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
+    }
+    __syncthreads();  // ws may still be read from the call before
+    if (lane == 31) ws[w] = x;
     __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-        const uint32_t v = threadIdx.x >= (unsigned)off ? part[threadIdx.x - off] : 0u;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
+    uint32_t before = 0;
+    total = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        if (j < w) before += ws[j];
+        total += ws[j];
     }
-    uint32_t run = part[threadIdx.x] - s;
-    for (int i = b0; i < min(b0 + per, total); ++i) {
-        const uint32_t c = hist[i];
-        hist[i] = run;
-        run += c;
+    return before + x - v;
+}
+
+// Exclusive scan of each digit's counters over the blocks, one block per
+// digit, and the digit's total; the scatter adds the digits before it.
+__global__ void __launch_bounds__(256) k_radix_rows(uint32_t *__restrict__ hist, int nblocks, uint32_t *__restrict__ total) {
+    uint32_t *row = hist + (size_t)blockIdx.x * nblocks;
+    uint32_t carry = 0;
+    for (int i0 = 0; i0 < nblocks; i0 += 256) {
+        const int i = i0 + threadIdx.x;
+        const uint32_t v = i < nblocks ? row[i] : 0u;
+        uint32_t t;
+        const uint32_t e = block_prefix(v, t);
+        if (i < nblocks) row[i] = carry + e;
+        carry += t;
     }
+    if (threadIdx.x == 0) total[blockIdx.x] = carry;
 }
 
 __global__ void k_radix_scatter(const uint32_t *__restrict__ kin, const int32_t *__restrict__ vin,
                                 uint32_t *__restrict__ kout, int32_t *__restrict__ vout, int n, int shift,
-                                int nblocks, const uint32_t *__restrict__ offs) {
-    __shared__ uint32_t cnt[kSortTile / 32][256];
+                                int nblocks, const uint32_t *__restrict__ offs, const uint32_t *__restrict__ total) {
+    __shared__ uint32_t cnt[kSortTile / 32][256], first[256];
+    uint32_t all;
+    first[threadIdx.x] = block_prefix(total[threadIdx.x], all);
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int j = threadIdx.x; j < (kSortTile / 32) * 256; j += blockDim.x) (&cnt[0][0])[j] = 0u;
     __syncthreads();
@@ -139,7 +164,7 @@ __global__ void k_radix_scatter(const uint32_t *__restrict__ kin, const int32_t 
     if (valid) {
         uint32_t off = rank;
         for (int ww = 0; ww < w; ++ww) off += cnt[ww][digit];
-        const uint32_t dst = offs[digit * nblocks + blockIdx.x] + off;
+        const uint32_t dst = first[digit] + (offs ? offs[digit * nblocks + blockIdx.x] : 0u) + off;
         kout[dst] = key;
         vout[dst] = vin[i];
     }
@@ -237,11 +262,22 @@ __global__ void k_refit(const float *__restrict__ verts, const int32_t *__restri
     }
 }
 
+// Clusters left and the number of the next node to make, kept on the device:
+// round r reads state[r] and writes state[r + 1], so that the host need not
+// wait for a round to launch the next (its grids fit the clusters the host
+// last saw, and blocks past the present count do nothing).
+struct PlocState {
+    int32_t n, next;
+};
+
+__device__ __forceinline__ bool ploc_done(const PlocState *s) { return s->n == 1 && s->next == 0; }
+
 // parent of every internal node and leaf, read back from the child
 // references the Karras pass stored in the nodes
-__global__ void k_parents(const float4 *__restrict__ nodes, int T, int32_t *__restrict__ parent) {
+__global__ void k_parents(const float4 *__restrict__ nodes, int T, int32_t *__restrict__ parent,
+                          const PlocState *state) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T - 1) return;
+    if (i >= T - 1 || (state && !ploc_done(state))) return;
     const float4 r = nodes[4 * i + 3];
     const int left = __float_as_int(r.x), right = __float_as_int(r.y);
     parent[left >= 0 ? left : T - 1 + ~left] = i;
@@ -288,8 +324,10 @@ __global__ void k_ploc_init(const float4 *__restrict__ tris, int T, int32_t *__r
 
 // nearest neighbour of each of the n clusters within the radius; the block's
 // clusters and the radius on either side are staged in shared memory
-__global__ void __launch_bounds__(kPlocBlock) k_ploc_nn(const float4 *__restrict__ cbox, int n,
-                                                       int32_t *__restrict__ nn) {
+__global__ void __launch_bounds__(kPlocBlock) k_ploc_nn(const float4 *__restrict__ cbox,
+                                                       const PlocState *__restrict__ state, int32_t *__restrict__ nn) {
+    const int n = state->n;
+    if (n < 2 || blockIdx.x * kPlocBlock >= n) return;
     __shared__ float4 sb[2 * (kPlocBlock + 2 * kPlocRadius)];
     const int base = blockIdx.x * kPlocBlock - kPlocRadius;
     for (int k = threadIdx.x; k < kPlocBlock + 2 * kPlocRadius; k += blockDim.x) {
@@ -318,44 +356,63 @@ __global__ void __launch_bounds__(kPlocBlock) k_ploc_nn(const float4 *__restrict
     nn[i] = bj;
 }
 
-// merge flag (the lower of a mutual pair) and keep flag (not the higher one)
-__global__ void k_ploc_flags(const int32_t *__restrict__ nn, int n, uint32_t *__restrict__ mflag,
-                             uint32_t *__restrict__ kflag) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int j = nn[i];
-    const bool mutual = nn[j] == i;
-    mflag[i] = (mutual && i < j) ? 1u : 0u;
-    kflag[i] = (mutual && i > j) ? 0u : 1u;
+// per block of 256 clusters: merges (lower of a mutual pair) and survivors
+// (not the higher of one)
+__global__ void __launch_bounds__(256) k_ploc_count(const int32_t *__restrict__ nn, const PlocState *__restrict__ state,
+                                                    uint2 *__restrict__ counts) {
+    const int n = state->n;
+    if (n < 2 || blockIdx.x * 256 >= n) return;
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    const int j = i < n ? nn[i] : 0;
+    const bool mutual = i < n && nn[j] == i;
+    const int m = __syncthreads_count(mutual && i < j), k = __syncthreads_count(i < n && !(mutual && i > j));
+    if (threadIdx.x == 0) counts[blockIdx.x] = make_uint2((uint32_t)m, (uint32_t)k);
 }
 
-// with mscan / kscan the exclusive prefix sums of the flags: write the new
-// nodes (ids next - 1 - mscan[i]) and the surviving clusters in order;
-// counts = (clusters left, merges)
-__global__ void k_ploc_compact(const int32_t *__restrict__ nn, int n, const uint32_t *__restrict__ mscan,
-                               const uint32_t *__restrict__ kscan, int next, const int32_t *__restrict__ cid,
-                               const float4 *__restrict__ cbox, int32_t *__restrict__ cid_out,
-                               float4 *__restrict__ cbox_out, float4 *__restrict__ nodes,
-                               int32_t *__restrict__ counts) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int j = nn[i];
-    const bool mutual = nn[j] == i;
-    if (i == n - 1) {
-        counts[0] = (int32_t)(kscan[i] + ((mutual && i > j) ? 0u : 1u));
-        counts[1] = (int32_t)(mscan[i] + ((mutual && i < j) ? 1u : 0u));
+__device__ __forceinline__ void ploc_merge(float4 *nodes, int id, int ca, int cb, float4 lo, float4 hi, float4 rlo,
+                                           float4 rhi) {
+    float4 *nd = nodes + 4 * (int64_t)id;
+    nd[0] = make_float4(lo.x, hi.x, lo.y, hi.y);
+    nd[1] = make_float4(rlo.x, rhi.x, rlo.y, rhi.y);
+    nd[2] = make_float4(lo.z, hi.z, rlo.z, rhi.z);
+    nd[3] = make_float4(__int_as_float(ca), __int_as_float(cb), 0.0f, 0.0f);
+}
+
+// New nodes (numbers next - 1 - rank of the merge) and the surviving clusters
+// in order.  Every block adds up the counts of the blocks before it itself:
+// up to 780 of them at 200k triangles, read once by each block in one sweep,
+// where a scan in a kernel of its own with a single block took longer than
+// the rest of the round.
+__global__ void __launch_bounds__(256) k_ploc_compact(const int32_t *__restrict__ nn, PlocState *__restrict__ state,
+                                                      const uint2 *__restrict__ counts, const int32_t *__restrict__ cid,
+                                                      const float4 *__restrict__ cbox, int32_t *__restrict__ cid_out,
+                                                      float4 *__restrict__ cbox_out, float4 *__restrict__ nodes) {
+    const int n = state->n, next = state->next;
+    if (n < 2) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) state[1] = state[0];
+        return;
     }
-    if (mutual && i > j) return;  // merged into j
-    const uint32_t o = kscan[i];
+    if (blockIdx.x * 256 >= n) return;
+    uint32_t pm = 0, pk = 0;
+    for (int j = threadIdx.x; j < (int)blockIdx.x; j += 256) {
+        const uint2 c = counts[j];
+        pm += c.x;
+        pk += c.y;
+    }
+    uint32_t mbase, kbase, tm, tk;
+    block_prefix(pm, mbase);
+    block_prefix(pk, kbase);
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    const int j = i < n ? nn[i] : 0;
+    const bool mutual = i < n && nn[j] == i, merge = mutual && i < j, keep = i < n && !(mutual && i > j);
+    const uint32_t m = mbase + block_prefix(merge ? 1u : 0u, tm), o = kbase + block_prefix(keep ? 1u : 0u, tk);
+    if (i == n - 1) state[1] = PlocState{(int32_t)(kbase + tk), next - (int32_t)(mbase + tm)};
+    if (!keep) return;  // merged into j
     const float4 lo = cbox[2 * i], hi = cbox[2 * i + 1];
-    if (mutual) {
-        const int id = next - 1 - (int)mscan[i];
+    if (merge) {
+        const int id = next - 1 - (int)m;
         const float4 rlo = cbox[2 * j], rhi = cbox[2 * j + 1];
-        float4 *nd = nodes + 4 * (int64_t)id;
-        nd[0] = make_float4(lo.x, hi.x, lo.y, hi.y);
-        nd[1] = make_float4(rlo.x, rhi.x, rlo.y, rhi.y);
-        nd[2] = make_float4(lo.z, hi.z, rlo.z, rhi.z);
-        nd[3] = make_float4(__int_as_float(cid[i]), __int_as_float(cid[j]), 0.0f, 0.0f);
+        ploc_merge(nodes, id, cid[i], cid[j], lo, hi, rlo, rhi);
         cid_out[o] = id;
         cbox_out[2 * o] = make_float4(fminf(lo.x, rlo.x), fminf(lo.y, rlo.y), fminf(lo.z, rlo.z), 0.f);
         cbox_out[2 * o + 1] = make_float4(fmaxf(hi.x, rhi.x), fmaxf(hi.y, rhi.y), fmaxf(hi.z, rhi.z), 0.f);
@@ -366,11 +423,95 @@ __global__ void k_ploc_compact(const int32_t *__restrict__ nn, int n, const uint
     }
 }
 
+// The last rounds, from kPlocSmall clusters on, in one block with the clusters
+// in shared memory: the same rounds without the launches (a round of so few
+// clusters is all launch latency).  Stops at the first round that merges
+// nothing, which the host sees from the count left.
+constexpr int kPlocSmall = 1024;
+__global__ void __launch_bounds__(kPlocSmall) k_ploc_small(PlocState *__restrict__ state, const int32_t *__restrict__ cid,
+                                                           const float4 *__restrict__ cbox, float4 *__restrict__ nodes) {
+    __shared__ float4 slo[kPlocSmall], shi[kPlocSmall];
+    __shared__ int32_t sid[kPlocSmall], snn[kPlocSmall];
+    __shared__ uint32_t wm[32], wk[32];
+    int n = state->n, next = state->next;
+    const int i = threadIdx.x, lane = i & 31, w = i >> 5;
+    if (i < n) {
+        sid[i] = cid[i];
+        slo[i] = cbox[2 * i];
+        shi[i] = cbox[2 * i + 1];
+    }
+    __syncthreads();
+    while (n > 1) {
+        float4 lo, hi;
+        int32_t id = 0;
+        if (i < n) {
+            lo = slo[i];
+            hi = shi[i];
+            id = sid[i];
+            float best = INFINITY;
+            int bj = i > 0 ? i - 1 : i + 1;
+            const int j0 = max(0, i - kPlocRadius), j1 = min(n - 1, i + kPlocRadius);
+            for (int j = j0; j <= j1; ++j) {
+                if (j == i) continue;
+                const float a = union_area(lo, hi, slo[j], shi[j]);
+                if (a < best) {
+                    best = a;
+                    bj = j;
+                }
+            }
+            snn[i] = bj;
+        }
+        __syncthreads();
+        const int j = i < n ? snn[i] : 0;
+        const bool mutual = i < n && snn[j] == i, merge = mutual && i < j, keep = i < n && !(mutual && i > j);
+        const unsigned bm = __ballot_sync(0xffffffffu, merge), bk = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) {
+            wm[w] = __popc(bm);
+            wk[w] = __popc(bk);
+        }
+        float4 rlo, rhi;
+        int32_t rid = 0;
+        if (merge) {
+            rlo = slo[j];
+            rhi = shi[j];
+            rid = sid[j];
+        }
+        __syncthreads();
+        uint32_t m = __popc(bm & ((1u << lane) - 1u)), o = __popc(bk & ((1u << lane) - 1u)), tm = 0, tk = 0;
+        for (int q = 0; q < 32; ++q) {
+            if (q < w) {
+                m += wm[q];
+                o += wk[q];
+            }
+            tm += wm[q];
+            tk += wk[q];
+        }
+        if (keep) {
+            if (merge) {
+                const int node = next - 1 - (int)m;
+                ploc_merge(nodes, node, id, rid, lo, hi, rlo, rhi);
+                id = node;
+                lo = make_float4(fminf(lo.x, rlo.x), fminf(lo.y, rlo.y), fminf(lo.z, rlo.z), 0.f);
+                hi = make_float4(fmaxf(hi.x, rhi.x), fmaxf(hi.y, rhi.y), fmaxf(hi.z, rhi.z), 0.f);
+            }
+            sid[o] = id;
+            slo[o] = lo;
+            shi[o] = hi;
+        }
+        __syncthreads();
+        if (tm == 0) break;
+        n = (int)tk;
+        next -= (int)tm;
+    }
+    if (i == 0) *state = PlocState{n, next};
+}
+
 // deepest leaf: internal nodes on its path from the root (stops counting
 // past `limit`, so a malformed tree cannot loop)
-__global__ void k_tree_depth(const int32_t *__restrict__ parent, int T, int limit, int32_t *__restrict__ depth) {
+__global__ void k_tree_depth(const int32_t *__restrict__ parent, int T, int limit, int32_t *__restrict__ depth,
+                             const PlocState *state) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= T) return;
+    if (p >= T || !ploc_done(state)) return;
     int d = 1, node = parent[T - 1 + p];
     while (node != 0 && d <= limit) {
         node = parent[node];
@@ -379,12 +520,14 @@ __global__ void k_tree_depth(const int32_t *__restrict__ parent, int T, int limi
     atomicMax(depth, d);
 }
 
+constexpr int kPlocBatch = 8;  // rounds launched before the host looks at the count
+
 }  // namespace
 
 size_t ploc_scratch_bytes(int32_t T) {
     const size_t n = (size_t)(T > 0 ? T : 1);
     return 2 * align256(n * 4) + 2 * align256(n * 32) + align256(n * 4) + 2 * align256(n * 4) +
-           align256(n * 64) + align256(2 * n * 4) + align256(4 * 4);
+           align256(n * 64) + align256(2 * n * 4) + align256((kPlocBatch + 2) * sizeof(PlocState));
 }
 
 int launch_ploc(Scene &sc, void *scratch, size_t scratch_bytes, int max_depth, cudaStream_t st, int32_t *depth_out) {
@@ -402,43 +545,56 @@ int launch_ploc(Scene &sc, void *scratch, size_t scratch_bytes, int max_depth, c
     int32_t *cid[2] = {(int32_t *)take(n * 4), (int32_t *)take(n * 4)};
     float4 *cbox[2] = {(float4 *)take(n * 32), (float4 *)take(n * 32)};
     int32_t *nn = (int32_t *)take(n * 4);
-    uint32_t *mflag = (uint32_t *)take(n * 4), *kflag = (uint32_t *)take(n * 4);
+    uint2 *bcount = (uint2 *)take(2 * align256(n * 4));
     float4 *nodes = (float4 *)take(n * 64);
     int32_t *parent = (int32_t *)take(2 * n * 4);
-    int32_t *counts = (int32_t *)take(4 * 4);
+    PlocState *state = (PlocState *)take((kPlocBatch + 2) * sizeof(PlocState));
+    int32_t *depth = (int32_t *)(state + kPlocBatch + 1);
     const int tb = 256;
     int launches = 0;
     k_ploc_init<<<(T + tb - 1) / tb, tb, 0, st>>>(sc.tris, T, cid[0], cbox[0]);
     ++launches;
-    int cur = 0, count = T, next = T - 1;
-    while (count > 1) {
-        const int g = (count + tb - 1) / tb;
-        k_ploc_nn<<<(count + kPlocBlock - 1) / kPlocBlock, kPlocBlock, 0, st>>>(cbox[cur], count, nn);
-        k_ploc_flags<<<g, tb, 0, st>>>(nn, count, mflag, kflag);
-        k_radix_scan<<<1, 1024, 0, st>>>(mflag, count);
-        k_radix_scan<<<1, 1024, 0, st>>>(kflag, count);
-        k_ploc_compact<<<g, tb, 0, st>>>(nn, count, mflag, kflag, next, cid[cur], cbox[cur], cid[1 - cur],
-                                         cbox[1 - cur], nodes, counts);
-        launches += 5;
-        int32_t h[2];
-        cudaError_t e = cudaMemcpyAsync(h, counts, sizeof h, cudaMemcpyDeviceToHost, st);
+    PlocState h{T, T - 1};
+    int cur = 0;
+    cudaError_t e = cudaMemcpyAsync(state, &h, sizeof h, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return DPCS_ERR_CUDA;
+    while (h.n > kPlocSmall) {
+        // a round leaves about two thirds of the clusters: stop the batch where
+        // the small kernel can take over
+        int rounds = 0;
+        for (double left = h.n; rounds < kPlocBatch && left > kPlocSmall; ++rounds) left *= 0.66;
+        const int g = (h.n + tb - 1) / tb;
+        for (int r = 0; r < rounds; ++r) {
+            k_ploc_nn<<<(h.n + kPlocBlock - 1) / kPlocBlock, kPlocBlock, 0, st>>>(cbox[cur], state + r, nn);
+            k_ploc_count<<<g, tb, 0, st>>>(nn, state + r, bcount);
+            k_ploc_compact<<<g, tb, 0, st>>>(nn, state + r, bcount, cid[cur], cbox[cur], cid[1 - cur], cbox[1 - cur], nodes);
+            launches += 3;
+            cur = 1 - cur;
+        }
+        const int32_t before = h.n;
+        e = cudaMemcpyAsync(&h, state + rounds, sizeof h, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return DPCS_ERR_CUDA;
-        if (h[1] < 1 || h[0] != count - h[1] || h[1] > next) return DPCS_ERR_DEVICE_CHECK;  // every round merges
-        count = h[0];
-        next -= h[1];
-        cur = 1 - cur;
+        // every round merges; each merge takes one cluster and makes one node
+        if (h.n < 1 || h.n >= before || h.next != h.n - 1) return DPCS_ERR_DEVICE_CHECK;
+        e = cudaMemcpyAsync(state, state + rounds, sizeof h, cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return DPCS_ERR_CUDA;
     }
-    if (next != 0) return DPCS_ERR_DEVICE_CHECK;
-    // depth of the new tree against the traversal stack
-    k_parents<<<(T - 1 + tb - 1) / tb, tb, 0, st>>>(nodes, T, parent);
-    cudaMemsetAsync(counts, 0, 4, st);
-    k_tree_depth<<<(T + tb - 1) / tb, tb, 0, st>>>(parent, T, max_depth + 1, counts);
+    if (h.n > 1) {
+        k_ploc_small<<<1, kPlocSmall, 0, st>>>(state, cid[cur], cbox[cur], nodes);
+        ++launches;
+    }
+    // depth of the new tree against the traversal stack (only a finished tree is walked)
+    k_parents<<<(T - 1 + tb - 1) / tb, tb, 0, st>>>(nodes, T, parent, state);
+    cudaMemsetAsync(depth, 0, 4, st);
+    k_tree_depth<<<(T + tb - 1) / tb, tb, 0, st>>>(parent, T, max_depth + 1, depth, state);
     launches += 2;
     int32_t d = 0;
-    cudaError_t e = cudaMemcpyAsync(&d, counts, 4, cudaMemcpyDeviceToHost, st);
+    e = cudaMemcpyAsync(&h, state, sizeof h, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&d, depth, 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return DPCS_ERR_CUDA;
+    if (h.n != 1 || h.next != 0) return DPCS_ERR_DEVICE_CHECK;
     *depth_out = d;
     if (d > max_depth) return launches;  // too deep for the traversal stack: the radix tree stays
     e = cudaMemcpyAsync(sc.nodes, nodes, (n - 1) * 64, cudaMemcpyDeviceToDevice, st);
@@ -470,7 +626,7 @@ int launch_lbvh_refit(const float *d_verts, Scene &sc, void *scratch, size_t scr
     int launches = 0;
     if (T >= 2) {
         cudaMemsetAsync(flags, 0, n * 4, st);
-        k_parents<<<(T - 1 + tb - 1) / tb, tb, 0, st>>>(sc.nodes, T, parent);
+        k_parents<<<(T - 1 + tb - 1) / tb, tb, 0, st>>>(sc.nodes, T, parent, nullptr);
         ++launches;
     }
     k_refit<<<gb, tb, 0, st>>>(d_verts, sc.vidx, sc.uv, sc.order, T, sc.nodes, parent, flags, sc.tris, sc.tuv);
@@ -518,23 +674,27 @@ int launch_lbvh_build(const float *d_verts, int32_t V, const int32_t *d_tris, in
         return (void *)r;
     };
     float *cen = (float *)take(3 * n * 4);
-    float *bounds = (float *)take(6 * 4);
+    uint32_t *bounds = (uint32_t *)take(6 * 4);
     uint32_t *ka = (uint32_t *)take(n * 4), *kb = (uint32_t *)take(n * 4);
     int32_t *va = (int32_t *)take(n * 4), *vb = (int32_t *)take(n * 4);
     uint32_t *hist = (uint32_t *)take(256 * (size_t)nb * 4);
     int32_t *parent = (int32_t *)take(2 * n * 4);
     int32_t *flags = (int32_t *)take(n * 4);
+    // digit totals of a sort pass: the counters themselves when there is one
+    // block, else 1 KB of the flags, which only the refit uses
+    uint32_t *dtotal = nb == 1 ? hist : (uint32_t *)flags;
     int launches = 0;
     const int tb = 256, gb = (T + tb - 1) / tb;
-    k_centroids<<<gb, tb, 0, st>>>(d_verts, d_tris, T, cen);
-    k_bounds<<<1, 1024, 0, st>>>(cen, T, bounds);
+    cudaMemsetAsync(bounds, 0xff, 3 * 4, st);
+    cudaMemsetAsync(bounds + 3, 0, 3 * 4, st);
+    k_centroids<<<gb, tb, 0, st>>>(d_verts, d_tris, T, cen, bounds);
     k_morton<<<gb, tb, 0, st>>>(cen, bounds, T, ka, va);
-    launches += 3;
+    launches += 2;
     for (int shift = 0; shift < 32; shift += 8) {
         k_radix_hist<<<nb, kSortTile, 0, st>>>(ka, T, shift, nb, hist);
-        k_radix_scan<<<1, 1024, 0, st>>>(hist, 256 * nb);
-        k_radix_scatter<<<nb, kSortTile, 0, st>>>(ka, va, kb, vb, T, shift, nb, hist);
-        launches += 3;
+        if (nb > 1) k_radix_rows<<<256, 256, 0, st>>>(hist, nb, dtotal);
+        k_radix_scatter<<<nb, kSortTile, 0, st>>>(ka, va, kb, vb, T, shift, nb, nb > 1 ? hist : nullptr, dtotal);
+        launches += nb > 1 ? 3 : 2;
         uint32_t *tk = ka; ka = kb; kb = tk;
         int32_t *tv = va; va = vb; vb = tv;
     }
