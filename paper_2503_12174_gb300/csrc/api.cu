@@ -955,7 +955,8 @@ dpcs_status dpcs_render_backward_principled(dpcs_ctx *c, dpcs_scene scene, const
     a.gE = (const float *)c->gE.p;
     a.dEp = (float4 *)c->dEp4.p;
     a.dtex = want_tex ? (float4 *)c->dtex4.p : nullptr;
-    nl += launch_replay_pbr(a, (const float4 *)c->mat4.p, want_mat ? (float4 *)c->dmat4.p : nullptr, st);
+    void *recs = optional_scratch(c, c->recs, grad_scratch_bytes(a, true, kPRecWordsHost), st);
+    nl += launch_replay_pbr(a, (const float4 *)c->mat4.p, want_mat ? (float4 *)c->dmat4.p : nullptr, acc, recs, st);
     nl += launch_prf_backward(Ip, (const float4 *)c->dEp4.p, np, params->gamma_p, params->gain_p, dIp, acc, st);
     if (want_tex) nl += launch_tex_backward((const float4 *)c->dtex4.p, nt, dAlbedo, dRough, st);
     if (want_mat) nl += launch_mat_backward((const float4 *)c->dmat4.p, nt, dMetallic, dNormal, st);
@@ -1265,9 +1266,10 @@ dpcs_status dpcs_render_loss_backward_principled(dpcs_ctx *c, dpcs_scene scene, 
     const float4 *m4 = (const float4 *)c->mat4.p;
     float4 *dm4 = want_mat ? (float4 *)c->dmat4.p : nullptr;
     const LossArgs l{target, scale, loss_kind, acc};
+    void *recs = optional_scratch(c, c->recs, grad_scratch_bytes(a, !fused, kPRecWordsHost), st);
     if (fused) {
         a.Ec = Ec;
-        nl += launch_render_grad_pbr(a, m4, dm4, l, st);
+        nl += launch_render_grad_pbr(a, m4, dm4, l, recs, st);
     } else {  // render, per-pixel loss, Eq. 5 adjoint, replay
         float *dIc = (float *)c->pix.p, *ec = Ec ? Ec : (float *)c->pix.p + 3 * npix;
         a.Ec = ec;
@@ -1276,7 +1278,7 @@ dpcs_status dpcs_render_loss_backward_principled(dpcs_ctx *c, dpcs_scene scene, 
         nl += launch_crf_backward(dIc, ec, Ic, npix, params->gamma_c, params->gain_c, params->wb, (float *)c->gE.p,
                                   acc, st);
         a.gE = (const float *)c->gE.p;
-        nl += launch_replay_pbr(a, m4, dm4, st);
+        nl += launch_replay_pbr(a, m4, dm4, acc, recs, st);
     }
     nl += launch_loss_out(acc, loss, st);
     nl += launch_prf_backward(Ip, (const float4 *)c->dEp4.p, np, params->gamma_p, params->gain_p, dIp, acc, st);

@@ -144,6 +144,8 @@ int launch_trace(const Scene &sc, const float *o, const float *d, int64_t n, flo
                  unsigned *status, cudaStream_t st);
 int launch_crf_backward(const float *dIc, const float *Ec, const float *Ic, int64_t npix, const float gamma_c[3],
                         float gain_c, const float wb[3], float *gE, double *acc, cudaStream_t st);
+constexpr int kRecWordsHost = 24;   // 32-bit words of one kept vertex record (VRec)
+constexpr int kPRecWordsHost = 52;  // and of a principled one (PRec)
 // The adjoint kernels run in tiles when they are given grad_scratch_bytes of
 // scratch (0: no tile kernel for these arguments); acc[kTileCounter] must be
 // zero then, as must the rest of acc.
@@ -156,16 +158,15 @@ int launch_pixel_loss(const float *Ic, int64_t n, const LossArgs &l, float *dIc,
 // principled material (principled.cu)
 int launch_pack_mat(const float *metallic, const float *normal, int64_t ntex, float4 *mat, cudaStream_t st);
 int launch_render_pbr(const RenderArgs &a, const float4 *mat, cudaStream_t st);
-int launch_replay_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, cudaStream_t st);
+int launch_replay_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, double *acc, void *scratch, cudaStream_t st);
 int launch_mat_backward(const float4 *dmat, int64_t ntex, float *dMetallic, float *dNormal, cudaStream_t st);
-int launch_render_grad_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, const LossArgs &l, cudaStream_t st);
+int launch_render_grad_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, const LossArgs &l, void *scratch,
+                           cudaStream_t st);
 // kept principled records: kPRecWordsHost 32-bit words per vertex
-constexpr int kPRecWordsHost = 52;
 int launch_render_keep_pbr(const RenderArgs &a, const float4 *mat, void *chunks, uint8_t *nvs, cudaStream_t st);
 int launch_sweep_kept_pbr(const RenderArgs &a, const void *chunks, const uint8_t *nvs, float4 *dmat, cudaStream_t st);
 int launch_render_keep(const RenderArgs &a, void *chunks, uint8_t *nvs, cudaStream_t st);
 int launch_sweep_kept(const RenderArgs &a, const void *chunks, const uint8_t *nvs, cudaStream_t st);
-constexpr int kRecWordsHost = 24;  // 32-bit words of one kept vertex record (VRec)
 int launch_loss_out(const double *acc, float *loss, cudaStream_t st);
 int launch_prf_backward(const float *Ip, const float4 *dEp, int64_t ntex, const float gamma_p[3], float gain_p,
                         float *dIp, double *acc, cudaStream_t st);

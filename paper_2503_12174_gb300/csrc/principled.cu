@@ -23,15 +23,16 @@
 // pixel's loss gradient through Eq. 5, then the sweeps; k_render_keep_pbr and
 // k_sweep_kept_pbr keep the records in device memory for losses that couple
 // pixels (the Eq. 11 filter), as k_render_keep / k_sweep_kept do;
+// the *_pbr_tile kernels run the same paths over block tiles (tile.cuh);
 // k_mat_backward adds the metallic and normal-map gradients to the caller's
 // buffers.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#define DPCS_FUSION_BY_COMPILER  // these kernels share their arithmetic with no kernel outside this file
 #include "device.cuh"
 #include "internal.h"
 #include "principled.cuh"
+#include "tile.cuh"
 
 namespace dpcs {
 
@@ -76,11 +77,9 @@ struct PRec {
 //   d/d r:     dS/dr F_j
 //   d/d ns:    ln_e (F_j dS/dn + f_j wp / cs) + cont (F_j dS/dn + f_j wi / ci),
 // then ns = u / |u|, u = v_x T + v_y B + v_z N, v = 2 Vn - 1.
-__device__ __forceinline__ void psweep(const RenderArgs &a, float4 *__restrict__ dmat, const PRec *rec, int nv,
-                                       const float gb_in[3]) {
-    float A[3] = {0.f, 0.f, 0.f};
-    for (int c = nv - 1; c >= 0; --c) {
-        const PRec &R = rec[c];
+__device__ __forceinline__ void psweep_vertex(const RenderArgs &a, float4 *__restrict__ dmat, const PRec &R,
+                                              const float gb_in[3], float A[3]) {
+    {
         float ga[3], dEp[3];
         float dr = 0.0f, dm = 0.0f;
         f3 gn = mk3(0.f, 0.f, 0.f);
@@ -131,6 +130,12 @@ __device__ __forceinline__ void psweep(const RenderArgs &a, float4 *__restrict__
     }
 }
 
+__device__ __forceinline__ void psweep(const RenderArgs &a, float4 *__restrict__ dmat, const PRec *rec, int nv,
+                                       const float gb_in[3]) {
+    float A[3] = {0.f, 0.f, 0.f};
+    for (int c = nv - 1; c >= 0; --c) psweep_vertex(a, dmat, rec[c], gb_in, A);
+}
+
 __device__ __forceinline__ void prec_vertex(PRec &R, const PSurf &S, f3 beta) {
     R.tb = S.tb;
     R.pb.x0 = R.pb.y0 = 0;
@@ -173,6 +178,18 @@ __device__ __forceinline__ void pblock_reduce_add(float (&v)[NV], double *acc) {
 __device__ __forceinline__ float pcrf(float ec, float gain, float wb, float gamma) {
     const float v = gain * wb * ec;
     return v > 0.0f ? powf(v, gamma) : 0.0f;
+}
+
+// the light a vertex sends towards the camera's path, clipped per channel (Eq. 12)
+__device__ __forceinline__ f3 pnee_contrib(const RenderArgs &a, f3 beta, const PNee &N, unsigned &unc) {
+    f3 c = beta * N.fp * mk3(N.ep.x, N.ep.y, N.ep.z) * N.G;
+    unc = 7u;
+    if (a.clip > 0.0f) {
+        if (c.x > a.clip) { c.x = a.clip; unc &= ~1u; }
+        if (c.y > a.clip) { c.y = a.clip; unc &= ~2u; }
+        if (c.z > a.clip) { c.z = a.clip; unc &= ~4u; }
+    }
+    return c;
 }
 
 // One warp-synchronous pass over a lane's samples, as k_render and k_replay
@@ -289,13 +306,8 @@ __device__ __forceinline__ void pbr_lanes(const RenderArgs &a, const float4 *__r
                 PNee N;
                 const bool cand = pnee_prepare(a, S, N);
                 if (cand) {
-                    c = beta * N.fp * mk3(N.ep.x, N.ep.y, N.ep.z) * N.G;
-                    unsigned unc = 7u;
-                    if (a.clip > 0.0f) {
-                        if (c.x > a.clip) { c.x = a.clip; unc &= ~1u; }
-                        if (c.y > a.clip) { c.y = a.clip; unc &= ~2u; }
-                        if (c.z > a.clip) { c.z = a.clip; unc &= ~4u; }
-                    }
+                    unsigned unc;
+                    c = pnee_contrib(a, beta, N, unc);
                     if (kReplay) {
                         R->pb = N.pb;
                         R->Ep[0] = N.ep.x; R->Ep[1] = N.ep.y; R->Ep[2] = N.ep.z;
@@ -490,6 +502,157 @@ __global__ void __launch_bounds__(kPBlock) k_sweep_kept_pbr(const RenderArgs a, 
     }
 }
 
+// ---------------------------------------------------------------------------
+// The same over block tiles, chosen by render.cu's rule (tile.cuh).  As for
+// the plain material, the lanes kernels run with half their lanes idle once
+// paths part and spill what the shading keeps across the traversal; here
+// every record goes to memory when its vertex is shaded.  64 registers: 80
+// and 128 spill less and are slower (render of the second size below 0.349
+// and 0.427 ms).  Corner scene, 3 bounces, lanes -> tiles, ms:
+//                      100 x 100 x 35    256 x 256 x 16    512 x 512 x 16
+//   render              0.253 -> 0.213    0.424 -> 0.325    1.56 -> 1.12
+//   render with records 0.397 -> 0.288    0.681 -> 0.414    2.73 -> 1.53
+//   one-trace step      0.538 -> 0.427    0.832 -> 0.620    3.34 -> 2.36
+//   replay              0.420 -> 0.375    0.714 -> 0.551    2.77 -> 2.00
+// ---------------------------------------------------------------------------
+struct PbrCore {
+    const float4 *mat;
+    __device__ __forceinline__ bool begin(const RenderArgs &, int, uint32_t, int) { return true; }
+    __device__ __forceinline__ void dark(const RenderArgs &, int, int, int) {}
+    __device__ __forceinline__ void shade(const RenderArgs &a, int, uint32_t pix, uint32_t s, int, int b, const Hit &h,
+                                          f3 d, f3 beta, Shaded &R) {
+        const PSurf S = psurface_at(a, mat, h, d);
+        PNee N;
+        R.cand = pnee_prepare(a, S, N);
+        unsigned unc;
+        if (R.cand) R.c = pnee_contrib(a, beta, N, unc);
+        R.ext = false;
+        if (b < a.bounces) {
+            PCont C;
+            R.ext = pcontinue_prepare(a, pix, s, b, S, C);
+            if (R.ext) {
+                R.beta = beta * C.w;
+                R.wi = C.wi;
+            }
+        }
+        R.so = madd(S.x, S.n, kRayEps);
+    }
+};
+
+// every vertex recorded: the PRec fields, as 13 chunks laid out like RecordCore's
+template <bool kStream>
+struct PbrRecordCore {
+    const float4 *mat;
+    uint4 *chunks;
+    uint8_t *nvs;
+    int64_t nthr, t0;
+    int spl;
+    bool replay;  // as RecordCore's
+
+    __device__ __forceinline__ int64_t at(const RenderArgs &a, int c, int k, int v, int slot) const {
+        return kept_chunk(c, replay ? 0 : k, v, spl, a.bounces, nthr, t0 + slot);
+    }
+    __device__ __forceinline__ uint8_t &count(int k, int slot) const {
+        return nvs[(int64_t)(replay ? 0 : k) * nthr + t0 + slot];
+    }
+    __device__ __forceinline__ bool begin(const RenderArgs &a, int slot, uint32_t pix, int k) {
+        count(k, slot) = 0;
+        return !replay || a.gE[3 * (int64_t)pix] != 0.0f || a.gE[3 * (int64_t)pix + 1] != 0.0f ||
+               a.gE[3 * (int64_t)pix + 2] != 0.0f;
+    }
+    __device__ __forceinline__ void dark(const RenderArgs &a, int slot, int k, int v) {
+        constexpr int kG = (int)(offsetof(PRec, G) / 4);
+        reinterpret_cast<uint32_t *>(chunks + at(a, kG / 4, k, v, slot))[kG % 4] = 0u;
+    }
+    __device__ __forceinline__ void shade(const RenderArgs &a, int slot, uint32_t pix, uint32_t s, int k, int b, const Hit &h,
+                                          f3 d, f3 beta, Shaded &R) {
+        auto put = [&](int c, float x, float y, float z, float w) {
+            const uint4 q = make_uint4(__float_as_uint(x), __float_as_uint(y), __float_as_uint(z), __float_as_uint(w));
+            uint4 *p = chunks + at(a, c, k, b - 1, slot);
+            if (kStream) __stcs(p, q); else *p = q;
+        };
+        const PSurf S = psurface_at(a, mat, h, d);
+        R.so = madd(S.x, S.n, kRayEps);
+        put(0, __int_as_float(S.tb.x0), __int_as_float(S.tb.y0), S.tb.fx, S.tb.fy);
+        put(10, S.T.y, S.T.z, S.B.x, S.B.y);
+        put(11, S.B.z, S.n.x, S.n.y, S.n.z);
+        put(12, S.ns.x, S.ns.y, S.ns.z, S.inv_ulen);
+        PNee N;
+        R.cand = pnee_prepare(a, S, N);
+        unsigned unc = 0u;
+        if (R.cand) {
+            R.c = pnee_contrib(a, beta, N, unc);
+            unc |= N.L.on > 0.0f ? 8u : 0u;
+            put(1, __int_as_float(N.pb.x0), __int_as_float(N.pb.y0), N.pb.fx, N.pb.fy);
+            put(2, beta.x, beta.y, beta.z, N.ep.x);
+            put(3, N.ep.y, N.ep.z, N.G, S.rho.x);
+            put(6, N.L.dSn.x, N.L.dSn.y, N.L.dSn.z, N.wp_cs.x);
+        } else {
+            N.L.S = N.L.dSr = N.L.s5 = 0.0f;
+            N.wp_cs = mk3(0.f, 0.f, 0.f);
+            put(1, 0.f, 0.f, 0.f, 0.f);
+            put(2, beta.x, beta.y, beta.z, 0.f);
+            put(3, 0.f, 0.f, 0.f, S.rho.x);
+            put(6, 0.f, 0.f, 0.f, 0.f);
+        }
+        R.ext = false;
+        PCont C;
+        if (b < a.bounces) {
+            R.ext = pcontinue_prepare(a, pix, s, b, S, C);
+            if (R.ext) {
+                R.beta = beta * C.w;
+                R.wi = C.wi;
+                unc |= C.L.on > 0.0f ? 16u : 0u;
+            }
+        }
+        if (!R.ext) {
+            C.cw = C.L.S = C.L.dSr = C.L.s5 = 0.0f;
+            C.L.dSn = C.wi_ci = mk3(0.f, 0.f, 0.f);
+        }
+        put(4, S.rho.y, S.rho.z, S.m, __uint_as_float(unc));
+        put(5, C.cw, N.L.S, N.L.dSr, N.L.s5);
+        put(7, N.wp_cs.y, N.wp_cs.z, C.L.S, C.L.dSr);
+        put(8, C.L.s5, C.L.dSn.x, C.L.dSn.y, C.L.dSn.z);
+        put(9, C.wi_ci.x, C.wi_ci.y, C.wi_ci.z, S.T.x);
+        count(k, slot) = (uint8_t)b;
+    }
+};
+
+template <int B, int S>
+__global__ void __launch_bounds__(B, 1024 / B) k_render_pbr_tile(const RenderArgs a, const float4 *mat) {
+    __shared__ Tile<S> P;
+    PbrCore core{mat};
+    tile_image<B, S>(a, core, P, 0, (int64_t)blockIdx.x * S, ((int64_t)a.Hc * a.Wc) << a.log2L);
+}
+
+template <int B, int S>
+__global__ void __launch_bounds__(B, 1024 / B) k_keep_pbr_tile(const RenderArgs a, const float4 *mat, uint4 *chunks, uint8_t *nvs) {
+    __shared__ Tile<S> P;
+    PbrRecordCore<true> core{mat, chunks, nvs, ((int64_t)a.Hc * a.Wc) << a.log2L, (int64_t)blockIdx.x * S,
+                             (a.spp + (1 << a.log2L) - 1) >> a.log2L, false};
+    tile_image<B, S>(a, core, P, 0, (int64_t)blockIdx.x * S, ((int64_t)a.Hc * a.Wc) << a.log2L);
+}
+
+template <int B, int S>
+__global__ void __launch_bounds__(B, 1024 / B)
+    k_grad_pbr_tile(const RenderArgs a, const float4 *mat, float4 *dmat, const LossArgs l, char *scratch,
+                    size_t per_block, int64_t ntile, unsigned long long *counter) {
+    __shared__ Tile<S> P;
+    PbrRecordCore<false> core;
+    core.mat = mat;
+    tile_adjoint<B, S>(a, core, P, l, scratch, per_block, ntile, counter, (int)(sizeof(PRec) / 16),
+                       [&](int k, int slot, const float gb_in[3]) {
+                           float A[3] = {0.f, 0.f, 0.f};
+                           for (int v = core.count(k, slot) - 1; v >= 0; --v) {
+                               PRec R;
+                               uint4 *dst = reinterpret_cast<uint4 *>(&R);
+#pragma unroll
+                               for (int c = 0; c < (int)(sizeof(PRec) / 16); ++c) dst[c] = core.chunks[core.at(a, c, k, v, slot)];
+                               psweep_vertex(a, dmat, R, gb_in, A);
+                           }
+                       });
+}
+
 __global__ void k_pack_mat(const float *__restrict__ metallic, const float *__restrict__ normal, int64_t ntex,
                            float4 *__restrict__ mat) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -524,21 +687,50 @@ int launch_pack_mat(const float *metallic, const float *normal, int64_t ntex, fl
 int launch_render_pbr(const RenderArgs &a, const float4 *mat, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
     if (threads <= 0) return 0;
-    k_render_pbr<<<grid1(threads, kPBlock), kPBlock, 0, st>>>(a, mat);
+    if (!tiled(a) || a.root == kEmptyRoot)
+        k_render_pbr<<<grid1(threads, kPBlock), kPBlock, 0, st>>>(a, mat);
+    else if (small_tiles(a))
+        k_render_pbr_tile<64, 64><<<grid1(threads, 64), 64, 0, st>>>(a, mat);
+    else
+        k_render_pbr_tile<128, 256><<<grid1(threads, 256), 128, 0, st>>>(a, mat);
     return 1;
 }
 
-int launch_replay_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, cudaStream_t st) {
+namespace {
+template <int B, int S>
+void launch_grad_pbr_tiles(const RenderArgs &a, const float4 *mat, float4 *dmat, const LossArgs &l, void *scratch,
+                           cudaStream_t st) {
+    const TileGrid g = tile_grid(a, l, B, S, kPRecWordsHost);
+    k_grad_pbr_tile<B, S><<<g.grid, B, 0, st>>>(a, mat, dmat, l, (char *)scratch, g.per_block, g.ntile, g.counter);
+}
+void launch_grad_pbr_tile(const RenderArgs &a, const float4 *mat, float4 *dmat, const LossArgs &l, void *scratch,
+                          cudaStream_t st) {
+    if (small_tiles(a))
+        launch_grad_pbr_tiles<64, 64>(a, mat, dmat, l, scratch, st);
+    else
+        launch_grad_pbr_tiles<128, 256>(a, mat, dmat, l, scratch, st);
+}
+}  // namespace
+
+int launch_replay_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, double *acc, void *scratch, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
     if (threads <= 0) return 0;
+    if (scratch) {
+        launch_grad_pbr_tile(a, mat, dmat, LossArgs{nullptr, 1.0f, 0, acc}, scratch, st);
+        return 1;
+    }
     k_replay_pbr<<<grid1(threads, kPBlock), kPBlock, 0, st>>>(a, mat, dmat);
     return 1;
 }
 
-int launch_render_grad_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, const LossArgs &l,
+int launch_render_grad_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, const LossArgs &l, void *scratch,
                            cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
     if (threads <= 0) return 0;
+    if (scratch) {
+        launch_grad_pbr_tile(a, mat, dmat, l, scratch, st);
+        return 1;
+    }
     k_render_grad_pbr<<<grid1(threads, kPBlock), kPBlock, 0, st>>>(a, mat, dmat, l);
     return 1;
 }
@@ -549,7 +741,12 @@ static_assert(sizeof(PRec) % 16 == 0, "PRec must be whole 16-byte chunks");
 int launch_render_keep_pbr(const RenderArgs &a, const float4 *mat, void *chunks, uint8_t *nvs, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
     if (threads <= 0) return 0;
-    k_render_keep_pbr<<<grid1(threads, kPBlock), kPBlock, 0, st>>>(a, mat, (uint4 *)chunks, nvs);
+    if (!tiled(a) || a.root == kEmptyRoot)
+        k_render_keep_pbr<<<grid1(threads, kPBlock), kPBlock, 0, st>>>(a, mat, (uint4 *)chunks, nvs);
+    else if (small_tiles(a))
+        k_keep_pbr_tile<64, 64><<<grid1(threads, 64), 64, 0, st>>>(a, mat, (uint4 *)chunks, nvs);
+    else
+        k_keep_pbr_tile<128, 256><<<grid1(threads, 256), 128, 0, st>>>(a, mat, (uint4 *)chunks, nvs);
     return 1;
 }
 

@@ -29,17 +29,17 @@ struct PLobe {
 __device__ __forceinline__ void plobe(f3 n, f3 wo, f3 wi, float r, float ks, PLobe &L) {
     L.on = L.S = L.dSr = L.s5 = 0.0f;
     L.dSn = mk3(0.f, 0.f, 0.f);
-    const float co = dot(n, wo), ci = dot(n, wi);
+    const float co = dot_yx(n, wo), ci = dot(n, wi);
     if (co <= 0.0f || ci <= 0.0f) return;
     L.on = 1.0f;
     if (ks <= 0.0f) return;
     float dadr;
     const float a = alpha_of(r, dadr);
     const f3 h = normalize(wo + wi);
-    const float ch = dot(n, h), a2 = a * a;
-    const float t = sin2(n, h) + a2 * ch * ch;
+    const float ch = dot(n, h), a2 = mul1(a, a), b2 = 1.0f - a2;
+    const float t = muladd(a2 * ch, ch, sin2(n, h));
     const float D = a2 / (DPCS_PI_F * t * t);
-    const float si = sqrtf(a2 + (1.0f - a2) * ci * ci), so = sqrtf(a2 + (1.0f - a2) * co * co);
+    const float si = sqrtf(muladd(b2 * ci, ci, a2)), so = sqrtf(muladd(b2 * co, co, a2));
     const float G = (2.0f * ci / (ci + si)) * (2.0f * co / (co + so));
     const float S = ks * D * G / (4.0f * ci * co);
     const float dlnD = 2.0f / a - 4.0f * a * ch * ch / t;
@@ -50,22 +50,22 @@ __device__ __forceinline__ void plobe(f3 n, f3 wo, f3 wi, float r, float ks, PLo
     const float ko = -(1.0f + (1.0f - a2) * co / so) / (co + so);
     const float ki = -(1.0f + (1.0f - a2) * ci / si) / (ci + si);
     L.dSn = (h * kh + wo * ko + wi * ki) * S;
-    const float m = fmaxf(0.0f, 1.0f - dot(wo, h));
+    const float m = fmaxf(0.0f, 1.0f - dot_yx(wo, h));
     const float m2 = m * m;
     L.s5 = m2 * m2 * m;
 }
 
 // Schlick F_j for F0_j = (1 - m) f0 + m rho_j
 __device__ __forceinline__ float pfresnel(float rho, float m, float f0, float s5) {
-    const float F0 = (1.0f - m) * f0 + m * rho;
-    return F0 + (1.0f - F0) * s5;
+    const float F0 = muladd(m, rho, mul1(1.0f - m, f0));
+    return muladd(1.0f - F0, s5, F0);
 }
 
 // f per channel from a lobe
 __device__ __forceinline__ f3 pbrdf(f3 rho, float m, float f0, const PLobe &L) {
     const float kd = L.on * (1.0f - m) * DPCS_INV_PI_F;
-    return mk3(kd * rho.x + L.S * pfresnel(rho.x, m, f0, L.s5), kd * rho.y + L.S * pfresnel(rho.y, m, f0, L.s5),
-               kd * rho.z + L.S * pfresnel(rho.z, m, f0, L.s5));
+    return mk3(sum2(kd, rho.x, L.S, pfresnel(rho.x, m, f0, L.s5)), sum2(kd, rho.y, L.S, pfresnel(rho.y, m, f0, L.s5)),
+               sum2(kd, rho.z, L.S, pfresnel(rho.z, m, f0, L.s5)));
 }
 
 // surface interaction with the principled maps
@@ -82,14 +82,14 @@ __device__ __forceinline__ PSurf psurface_at(const RenderArgs &a, const float4 *
     const float4 V1 = __ldg(a.tris + 3 * h.pos + 1);
     const float4 V2 = __ldg(a.tris + 3 * h.pos + 2);
     const f3 e1 = xyz(V1) - xyz(A), e2 = xyz(V2) - xyz(A);
-    S.x = xyz(A) + e1 * h.u + e2 * h.v;
+    S.x = madd(madd(xyz(A), e1, h.u), e2, h.v);
     S.n = normalize(cross(e1, e2));
     if (dot(S.n, d) > 0.0f) S.n = S.n * -1.0f;
     const float2 t0 = __ldg(a.tuv + 3 * h.pos + 0), t1 = __ldg(a.tuv + 3 * h.pos + 1),
                  t2 = __ldg(a.tuv + 3 * h.pos + 2);
     const float w0 = 1.0f - h.u - h.v;
-    const float su = w0 * t0.x + h.u * t1.x + h.v * t2.x;
-    const float sv = w0 * t0.y + h.u * t1.y + h.v * t2.y;
+    const float su = muladd(h.v, t2.x, sum2(w0, t0.x, h.u, t1.x));
+    const float sv = muladd(h.v, t2.y, sum2(w0, t0.y, h.u, t1.y));
     S.tb = bilin_setup(muladd(su, (float)a.Wt, -0.5f), muladd(sv, (float)a.Ht, -0.5f), a.Wt, a.Ht);
     const float4 tex = bilin_fetch(a.tex, S.tb, a.Wt, a.Ht);
     const float4 mt = bilin_fetch(mat, S.tb, a.Wt, a.Ht);
@@ -99,11 +99,11 @@ __device__ __forceinline__ PSurf psurface_at(const RenderArgs &a, const float4 *
     S.wo = d * -1.0f;
     // tangent: dp/du from e1 = dp/du du1 + dp/dv dv1 and e2 likewise
     const float du1 = t1.x - t0.x, dv1 = t1.y - t0.y, du2 = t2.x - t0.x, dv2 = t2.y - t0.y;
-    const float det = du1 * dv2 - du2 * dv1;
+    const float det = diff2(du1, dv2, du2, dv1);
     bool ok = false;
     if (det != 0.0f) {
-        const f3 dpdu = (e1 * dv2 - e2 * dv1) * (1.0f / det);
-        const f3 t = dpdu - S.n * dot(S.n, dpdu);
+        const f3 dpdu = mk3(diff2(e1.x, dv2, e2.x, dv1), diff2(e1.y, dv2, e2.y, dv1), diff2(e1.z, dv2, e2.z, dv1)) * (1.0f / det);
+        const f3 t = madd(dpdu, S.n, -dot(S.n, dpdu));
         const float l2 = dot(t, t);
         if (l2 > 1e-12f * dot(dpdu, dpdu)) {
             S.T = t * rsqrtf(l2);
@@ -115,7 +115,7 @@ __device__ __forceinline__ PSurf psurface_at(const RenderArgs &a, const float4 *
         onb(S.n, S.T, b);
     }
     S.B = cross(S.n, S.T);
-    const f3 u = S.T * (2.0f * mt.y - 1.0f) + S.B * (2.0f * mt.z - 1.0f) + S.n * (2.0f * mt.w - 1.0f);
+    const f3 u = combine(S.T, 2.0f * mt.y - 1.0f, S.B, 2.0f * mt.z - 1.0f, S.n, 2.0f * mt.w - 1.0f);
     const float ul2 = dot(u, u);
     if (ul2 > 1e-24f) {
         S.inv_ulen = rsqrtf(ul2);
@@ -150,7 +150,7 @@ __device__ __forceinline__ bool pnee_prepare(const RenderArgs &a, const PSurf &S
     const float cs = dot(S.ns, wp);
     if (!(cs > 0.0f && dot(S.n, wp) > 0.0f)) return false;
     const float cpz = X.z / sqrtf(dot(X, X));
-    N.so = S.x + S.n * kRayEps;
+    N.so = madd(S.x, S.n, kRayEps);
     const f3 sv = cp - N.so;
     const float sd = sqrtf(dot(sv, sv));
     N.sdir = sv * (1.0f / sd);

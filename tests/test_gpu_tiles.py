@@ -92,3 +92,52 @@ def test_tile_gradients_equal_lane_gradients(mesh, H, W, spp, bounces):
         assert abs(a[1] - b[1]) <= 1e-6 * abs(b[1])
         for x, y in zip(a[2:], b[2:]):
             np.testing.assert_allclose(x, y, rtol=1e-5, atol=1e-6 * np.abs(y).max())
+
+
+@pytest.mark.parametrize("mesh,H,W,spp,bounces,maps", [
+    ("corner", 1, 3, 7, 3, "both"), ("corner", 17, 31, 35, 3, "both"), ("corner", 9, 57, 100, 2, "metallic"),
+    ("corner", 125, 125, 33, 3, "both"), ("corner", 12, 11, 300, 3, "normal"), ("sphere", 24, 24, 16, 8, "both"),
+    ("triangle", 20, 20, 8, 3, "both")])
+def test_principled_tiles_equal_lanes(mesh, H, W, spp, bounces, maps):
+    """As above with the principled material, whose render and kept records
+    run in tiles with or without a budget: one-trace step, separate calls and
+    kept records against a budget's one-trace and separate steps.  Images are
+    equal bit for bit.  The FP32 gradient accumulators add n terms in any
+    order, so they differ by at most n 2^-23 of the terms' absolute sum, n
+    their number per texel; four times the largest gradient stands for that sum."""
+    torch = need_cuda()
+    sc = scenes.with_principled(_scene(mesh, H, W, spp, bounces), seed=8)
+    out = []
+    for budget in (0, 1 << 30):
+        c = dpcs.Context(0, hbm_budget_bytes=budget)
+        h = c.upload(sc.verts, sc.tris, sc.uv)
+        alb, rough, Ip, met, nrm = (torch.from_numpy(np.ascontiguousarray(x)).cuda()
+                                    for x in (sc.albedo, sc.rough, sc.Ip, sc.metallic, sc.normal))
+        met, nrm = (None if maps == "normal" else met), (None if maps == "metallic" else nrm)
+        view, prm = dpcs.view_of(sc), dpcs.make_params(sc.params)
+        tgt = torch.full((H, W, 3), 0.05, device="cuda")
+        Ec, Ic, dIc, loss = torch.empty_like(tgt), torch.empty_like(tgt), torch.empty_like(tgt), torch.zeros(1, device="cuda")
+        args = (h, alb, rough, met, nrm, Ip, view, prm, spp, bounces, sc.seed)
+        try:
+            for how in ("one", "two", "kept"):
+                g = [torch.zeros_like(x) for x in (Ip, alb, rough, alb[..., 0], alb)]
+                kw = dict(dIp=g[0], dAlbedo=g[1], dRough=g[2], dMetallic=None if met is None else g[3],
+                          dNormal=None if nrm is None else g[4])
+                if how == "one":
+                    c.render_loss_backward_principled(*args, tgt, loss, Ic=Ic, Ec=Ec, **kw)
+                else:
+                    c.render_principled(*args, Ic=Ic, Ec=Ec, keep=how == "kept")
+                    c.l2_loss(Ic, tgt, dIc, loss)
+                    c.render_backward_principled(*args, Ec, Ic, dIc, kept=how == "kept", **kw)
+                c.sync()
+                out.append([Ic.cpu().numpy().copy(), Ec.cpu().numpy().copy()] + [x.cpu().numpy().astype(np.float64) for x in g])
+            c.free(h)
+        finally:
+            c.close()
+    n = 4.0 * H * W * spp * bounces / min(sc.rough.size, sc.Ip.size // 3) + 4
+    ref = out[3]
+    for a in out:
+        np.testing.assert_array_equal(a[0], ref[0])
+        np.testing.assert_array_equal(a[1], ref[1])
+        for x, y in zip(a[2:], ref[2:]):
+            np.testing.assert_allclose(x, y, rtol=1e-5, atol=4 * n * 2.0 ** -23 * np.abs(y).max())
