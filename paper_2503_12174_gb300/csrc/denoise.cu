@@ -22,16 +22,12 @@
 #include "device.cuh"
 #include "internal.h"
 
-#ifndef DPCS_DENOISE_STRIP
-#define DPCS_DENOISE_STRIP 1  // 0: one output per thread (k_bilateral)
-#endif
-
 namespace dpcs {
 
 namespace {
 
 constexpr int kTile = 16;
-constexpr int kMaxRadius = 8;  // (16 + 16)^2 pixels x 48 B = 48 KiB of shared memory
+constexpr int kMaxRadius = 8;  // (16 + 16)^2 pixels x 40 B = 40 KiB of shared memory
 
 // First-hit guide through each camera pixel centre (a.jitter must be 0).
 __global__ void k_gbuffer(const RenderArgs a, float4 *__restrict__ guide) {
@@ -56,164 +52,181 @@ struct Widths {
     float ks, ka, kn, kd;  // 1 / (2 sigma^2) per term; 0 = term off
 };
 
-// kAdjoint = false: out = D(img), wsum = W (wsum may be null).
-// kAdjoint = true : out += D^T(img), where img is dD and wsum the forward W.
-template <bool kAdjoint>
-__global__ void __launch_bounds__(kTile *kTile)
-    k_bilateral(const float *__restrict__ img, const float4 *__restrict__ guide, const float *__restrict__ wsum_in,
-                int H, int W, int r, Widths k, float *__restrict__ out, float *__restrict__ wsum_out) {
-    extern __shared__ float4 smem[];
-    const int S = kTile + 2 * r;
-    float4 *sg0 = smem, *sg1 = smem + S * S, *si = smem + 2 * S * S;
-    const int tid = threadIdx.y * kTile + threadIdx.x;
-    const int y0 = blockIdx.y * kTile - r, x0 = blockIdx.x * kTile - r;
-    for (int i = tid; i < S * S; i += kTile * kTile) {
-        const int gy = y0 + i / S, gx = x0 + i % S;
-        if (gy >= 0 && gy < H && gx >= 0 && gx < W) {
-            const int64_t p = (int64_t)gy * W + gx;
-            sg0[i] = __ldg(guide + 2 * p);
-            float4 g1 = __ldg(guide + 2 * p + 1);
-            g1.w = 0.0f;  // inside the image
-            sg1[i] = g1;
-            float s = 1.0f;
-            if (kAdjoint) s = 1.0f / __ldg(wsum_in + p);
-            si[i] = make_float4(__ldg(img + 3 * p) * s, __ldg(img + 3 * p + 1) * s, __ldg(img + 3 * p + 2) * s, 0.0f);
-        } else {
-            sg1[i] = make_float4(0.f, 0.f, 0.f, -1.0f);  // outside: skipped
-        }
-    }
-    __syncthreads();
-    const int py = blockIdx.y * kTile + threadIdx.y, px = blockIdx.x * kTile + threadIdx.x;
-    if (py >= H || px >= W) return;
-    const int c = (threadIdx.y + r) * S + threadIdx.x + r;
-    const float4 c0 = sg0[c], c1 = sg1[c];
-    float ax = 0.f, ay = 0.f, az = 0.f, den = 0.f;
-    for (int dy = -r; dy <= r; ++dy) {
-        const int row = c + dy * S;
-        for (int dx = -r; dx <= r; ++dx) {
-            const int q = row + dx;
-            const float4 q1 = sg1[q];
-            if (q1.w < 0.0f) continue;
-            const float4 q0 = sg0[q];
-            const float da = (c0.x - q0.x) * (c0.x - q0.x) + (c0.y - q0.y) * (c0.y - q0.y) +
-                             (c0.z - q0.z) * (c0.z - q0.z);
-            const float dn = (c0.w - q0.w) * (c0.w - q0.w) + (c1.x - q1.x) * (c1.x - q1.x) +
-                             (c1.y - q1.y) * (c1.y - q1.y);
-            const float dt = (c1.z - q1.z) * (c1.z - q1.z);
-            const float e = (float)(dx * dx + dy * dy) * k.ks + da * k.ka + dn * k.kn + dt * k.kd;
-            const float w = expf(-e);
-            const float4 v = si[q];
-            ax += w * v.x;
-            ay += w * v.y;
-            az += w * v.z;
-            den += w;
-        }
-    }
-    const int64_t p = (int64_t)py * W + px;
-    if (kAdjoint) {
-        out[3 * p] += ax;
-        out[3 * p + 1] += ay;
-        out[3 * p + 2] += az;
-    } else {
-        const float inv = 1.0f / den;
-        out[3 * p] = ax * inv;
-        out[3 * p + 1] = ay * inv;
-        out[3 * p + 2] = az * inv;
-        if (wsum_out) wsum_out[p] = den;
-    }
+// two FP32 lanes in one instruction (each rounded as the scalar operation)
+typedef unsigned long long u64;
+__device__ __forceinline__ u64 pair(float a, float b) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ u64 pair(float2 v) { return pair(v.x, v.y); }
+__device__ __forceinline__ float2 unpair(u64 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+    u64 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+    u64 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ u64 add2(u64 a, u64 b) {
+    u64 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float ex2(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
-// The same filter with kStrip vertically stacked outputs per thread: each
-// tap loaded from shared memory serves every output of the strip whose
-// window contains it, so a thread issues (2r + kStrip) (2r + 1) tap loads
-// for kStrip outputs instead of kStrip (2r + 1)^2.  Each output still sums
-// its taps in the same order (rows, then columns), so the result is the one
-// k_bilateral computes.
-#ifndef DPCS_DENOISE_KSTRIP
-#define DPCS_DENOISE_KSTRIP 2  // measured: 2 is 9-15 % faster than 1 output per thread, 4 is 15-40 % slower
-#endif
-constexpr int kStrip = DPCS_DENOISE_KSTRIP;
+// The filter, two vertically stacked outputs per thread.
+// kAdjoint = false: out = D(img), wsum = W (wsum may be null).
+// kAdjoint = true : out += D^T(img), where img is dD and wsum the forward W.
+//
+// The taps are FP32 work on shared memory (121 taps x 24 operations an output
+// at r = 5; DRAM traffic is 4 % of the time), so the kernel counts
+// instructions.  The guide and the image sit in shared memory one feature a
+// plane, and a thread takes two horizontally adjacent taps at a time: one
+// 8-byte load a feature and packed FP32 operations, half the instructions of
+// one tap at a time.  Pairs start on even columns, so a window row is r pairs
+// and one tap left over at its right (even outputs) or left end, which runs as
+// a pair with itself and a distance term that makes the second weight 0; it
+// loads nothing outside the window, whose NaN would otherwise count.  The
+// widths carry log2(e), and a weight is one ex2 of the whole exponent
+// (against 64 bits the filter's error is 1.8e-7, with expf it was 2.7e-7).
+// 1024 x 1024 at r = 5, forward / adjoint, one tap at a time -> pairs: 0.193 /
+// 0.191 -> 0.148 / 0.165 ms; r = 8, 1000 x 700: 0.344 / 0.333 -> 0.216 / 0.231
+// ms (the packed FP32 pipe is 61 % busy).  Four outputs a thread instead of
+// two 2 to 8 % slower at r = 8 and as fast at 5; 64 registers (8 blocks an
+// SM) 16 % slower.
+constexpr int kFeat = 10;   // albedo 3, normal 3, depth, image 3
+constexpr int kStrip = 2;   // outputs per thread (the window tests below are written for two)
+constexpr float kFar = 1e30f;
 
 template <bool kAdjoint>
 __global__ void __launch_bounds__(kTile *kTile / kStrip)
-    k_bilateral_strip(const float *__restrict__ img, const float4 *__restrict__ guide,
-                      const float *__restrict__ wsum_in, int H, int W, int r, Widths k, float *__restrict__ out,
-                      float *__restrict__ wsum_out) {
-    extern __shared__ float4 smem[];
-    const int S = kTile + 2 * r;
-    float4 *sg0 = smem, *sg1 = smem + S * S, *si = smem + 2 * S * S;
+    k_bilateral(const float *__restrict__ img, const float4 *__restrict__ guide, const float *__restrict__ wsum_in,
+                int H, int W, int r, Widths k, float *__restrict__ out, float *__restrict__ wsum_out) {
+    extern __shared__ float smem[];
+    const int S = kTile + 2 * r, N = S * S;  // S is even
+    float2 *dist = reinterpret_cast<float2 *>(smem + kFeat * N);  // [parity][pair]: -dx^2 ks of the pair's taps
     constexpr int kThreads = kTile * kTile / kStrip;
+    constexpr float kLog2e = 1.44269504088896340736f;
+    const float nks = -k.ks * kLog2e;
     const int tid = threadIdx.y * kTile + threadIdx.x;
     const int y0 = blockIdx.y * kTile - r, x0 = blockIdx.x * kTile - r;
-    for (int i = tid; i < S * S; i += kThreads) {
-        const int gy = y0 + i / S, gx = x0 + i % S;
-        if (gy >= 0 && gy < H && gx >= 0 && gx < W) {
-            const int64_t p = (int64_t)gy * W + gx;
-            sg0[i] = __ldg(guide + 2 * p);
-            float4 g1 = __ldg(guide + 2 * p + 1);
-            g1.w = 0.0f;  // inside the image
-            sg1[i] = g1;
-            float s = 1.0f;
-            if (kAdjoint) s = 1.0f / __ldg(wsum_in + p);
-            si[i] = make_float4(__ldg(img + 3 * p) * s, __ldg(img + 3 * p + 1) * s, __ldg(img + 3 * p + 2) * s, 0.0f);
-        } else {
-            sg1[i] = make_float4(0.f, 0.f, 0.f, -1.0f);  // outside: skipped
+    for (int i = tid; i < N; i += kThreads) {
+        // a column beside the image repeats the guide of the nearest one, a tap
+        // of every window that reaches past it, with no image
+        const int gy = y0 + i / S, gx = x0 + i % S, cx = min(max(gx, 0), W - 1);
+        float f[kFeat] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (gy >= 0 && gy < H) {
+            const int64_t p = (int64_t)gy * W + cx;
+            const float4 g0 = __ldg(guide + 2 * p), g1 = __ldg(guide + 2 * p + 1);
+            const float s = kAdjoint ? 1.0f / __ldg(wsum_in + p) : 1.0f;
+            f[0] = g0.x; f[1] = g0.y; f[2] = g0.z; f[3] = g0.w;
+            f[4] = g1.x; f[5] = g1.y; f[6] = g1.z;
+            if (cx == gx) {
+                f[7] = __ldg(img + 3 * p) * s;
+                f[8] = __ldg(img + 3 * p + 1) * s;
+                f[9] = __ldg(img + 3 * p + 2) * s;
+            }
         }
+#pragma unroll
+        for (int q = 0; q < kFeat; ++q) smem[q * N + i] = f[q];
+    }
+    if (tid < 2 * r) {
+        const int d = 2 * (tid % r) - r + tid / r;  // first tap's dx
+        dist[tid] = make_float2((float)(d * d) * nks, (float)((d + 1) * (d + 1)) * nks);
     }
     __syncthreads();
     const int px = blockIdx.x * kTile + threadIdx.x;
     if (px >= W) return;
+    const int par = threadIdx.x & 1;
     const int ry = threadIdx.y * kStrip;  // the strip's first output row in the tile
-    float4 c0[kStrip], c1[kStrip];
-    float ax[kStrip], ay[kStrip], az[kStrip], den[kStrip];
+    const int py = blockIdx.y * kTile + ry;
+    u64 c[kStrip][7];
+    u64 ax[kStrip], ay[kStrip], az[kStrip], den[kStrip];
 #pragma unroll
     for (int o = 0; o < kStrip; ++o) {
-        const int c = (ry + o + r) * S + threadIdx.x + r;
-        c0[o] = sg0[c];
-        c1[o] = sg1[c];
-        ax[o] = ay[o] = az[o] = den[o] = 0.f;
+        const int at = (ry + o + r) * S + threadIdx.x + r;
+#pragma unroll
+        for (int q = 0; q < 7; ++q) c[o][q] = pair(smem[q * N + at], smem[q * N + at]);
+        ax[o] = ay[o] = az[o] = den[o] = 0ull;
     }
-    for (int j = -r; j < r + kStrip; ++j) {  // window rows, relative to the first output
-        const int row = (ry + j + r) * S + threadIdx.x + r;
-        for (int dx = -r; dx <= r; ++dx) {
-            const int q = row + dx;
-            const float4 q1 = sg1[q];
-            if (q1.w < 0.0f) continue;
-            const float4 q0 = sg0[q];
-            const float4 v = si[q];
+    const float ka = -k.ka * kLog2e, kn = -k.kn * kLog2e, kd = -k.kd * kLog2e;
+    const u64 nka = pair(ka, ka), nkn = pair(kn, kn), nkd = pair(kd, kd), neg = pair(-1.0f, -1.0f);
+    const bool edge = x0 < 0 || x0 + S > W;  // some taps fall off the image's sides
+    // window rows, relative to the first output, inside the image
+    const int j0 = max(-r, -py), j1 = min(r + kStrip - 1, H - 1 - py);
+    for (int j = j0; j <= j1; ++j) {
+        const float *row = smem + (ry + j + r) * S + threadIdx.x;
+        const bool on[kStrip] = {j <= r, j > -r};  // is the row in the output's window?
+        const u64 dy[kStrip] = {pair((float)(j * j) * nks, (float)(j * j) * nks),
+                                pair((float)((j - 1) * (j - 1)) * nks, (float)((j - 1) * (j - 1)) * nks)};
+        auto taps = [&](const u64 (&f)[kFeat], u64 dx) {
 #pragma unroll
             for (int o = 0; o < kStrip; ++o) {
-                const int dy = j - o;
-                if (dy < -r || dy > r) continue;
-                const float da = (c0[o].x - q0.x) * (c0[o].x - q0.x) + (c0[o].y - q0.y) * (c0[o].y - q0.y) +
-                                 (c0[o].z - q0.z) * (c0[o].z - q0.z);
-                const float dn = (c0[o].w - q0.w) * (c0[o].w - q0.w) + (c1[o].x - q1.x) * (c1[o].x - q1.x) +
-                                 (c1[o].y - q1.y) * (c1[o].y - q1.y);
-                const float dt = (c1[o].z - q1.z) * (c1[o].z - q1.z);
-                const float e = (float)(dx * dx + dy * dy) * k.ks + da * k.ka + dn * k.kn + dt * k.kd;
-                const float w = expf(-e);
-                ax[o] += w * v.x;
-                ay[o] += w * v.y;
-                az[o] += w * v.z;
-                den[o] += w;
+                if (!on[o]) continue;
+                u64 d[7];
+#pragma unroll
+                for (int n = 0; n < 7; ++n) d[n] = fma2(f[n], neg, c[o][n]);
+                const u64 da = fma2(d[2], d[2], fma2(d[1], d[1], mul2(d[0], d[0])));
+                const u64 dn = fma2(d[5], d[5], fma2(d[4], d[4], mul2(d[3], d[3])));
+                u64 e = add2(dx, dy[o]);
+                e = fma2(da, nka, e);
+                e = fma2(dn, nkn, e);
+                e = fma2(mul2(d[6], d[6]), nkd, e);
+                const float2 x = unpair(e);
+                const u64 w = pair(ex2(x.x), ex2(x.y));
+                ax[o] = fma2(w, f[7], ax[o]);
+                ay[o] = fma2(w, f[8], ay[o]);
+                az[o] = fma2(w, f[9], az[o]);
+                den[o] = add2(den[o], w);
             }
+        };
+        u64 f[kFeat];
+        for (int p = 0; p < r; ++p) {
+            const float2 *q = reinterpret_cast<const float2 *>(row + par + 2 * p);
+            float2 dx = dist[par * r + p];
+            if (edge) {
+                const int gx = x0 + (int)threadIdx.x + par + 2 * p;
+                if (gx < 0 || gx >= W) dx.x = -kFar;
+                if (gx + 1 < 0 || gx + 1 >= W) dx.y = -kFar;
+            }
+#pragma unroll
+            for (int n = 0; n < kFeat; ++n) f[n] = pair(q[n * (N / 2)]);
+            taps(f, pair(dx));
+        }
+        {  // the tap left over, at the window's right or left end
+            const int at = par ? 0 : 2 * r, gx = x0 + (int)threadIdx.x + at;
+#pragma unroll
+            for (int n = 0; n < kFeat; ++n) f[n] = pair(row[n * N + at], row[n * N + at]);
+            taps(f, pair(gx < 0 || gx >= W ? -kFar : (float)(r * r) * nks, -kFar));
         }
     }
 #pragma unroll
     for (int o = 0; o < kStrip; ++o) {
-        const int py = blockIdx.y * kTile + ry + o;
-        if (py >= H) break;
-        const int64_t p = (int64_t)py * W + px;
+        if (py + o >= H) break;
+        const int64_t p = (int64_t)(py + o) * W + px;
+        const float2 x = unpair(ax[o]), y = unpair(ay[o]), z = unpair(az[o]), n = unpair(den[o]);
         if (kAdjoint) {
-            out[3 * p] += ax[o];
-            out[3 * p + 1] += ay[o];
-            out[3 * p + 2] += az[o];
+            out[3 * p] += x.x + x.y;
+            out[3 * p + 1] += y.x + y.y;
+            out[3 * p + 2] += z.x + z.y;
         } else {
-            const float inv = 1.0f / den[o];
-            out[3 * p] = ax[o] * inv;
-            out[3 * p + 1] = ay[o] * inv;
-            out[3 * p + 2] = az[o] * inv;
-            if (wsum_out) wsum_out[p] = den[o];
+            const float dn = n.x + n.y, inv = 1.0f / dn;
+            out[3 * p] = (x.x + x.y) * inv;
+            out[3 * p + 1] = (y.x + y.y) * inv;
+            out[3 * p + 2] = (z.x + z.y) * inv;
+            if (wsum_out) wsum_out[p] = dn;
         }
     }
 }
@@ -247,15 +260,10 @@ template <bool kAdjoint>
 dpcs_status launch_bilateral(dpcs_ctx *c, const float *img, const float *guide, const float *wsum_in, int32_t Hc,
                              int32_t Wc, int r, const Widths &k, float *out, float *wsum_out, cudaStream_t st) {
     const int S = kTile + 2 * r;
-    const size_t shm = (size_t)3 * S * S * sizeof(float4);
+    const size_t shm = ((size_t)kFeat * S * S + 4 * r) * sizeof(float);
     const dim3 grid((Wc + kTile - 1) / kTile, (Hc + kTile - 1) / kTile);
-#if DPCS_DENOISE_STRIP
-    k_bilateral_strip<kAdjoint><<<grid, dim3(kTile, kTile / kStrip), shm, st>>>(img, (const float4 *)guide, wsum_in, Hc,
-                                                                            Wc, r, k, out, wsum_out);
-#else
-    k_bilateral<kAdjoint><<<grid, dim3(kTile, kTile), shm, st>>>(img, (const float4 *)guide, wsum_in, Hc, Wc, r, k,
-                                                                out, wsum_out);
-#endif
+    k_bilateral<kAdjoint><<<grid, dim3(kTile, kTile / kStrip), shm, st>>>(img, (const float4 *)guide, wsum_in, Hc, Wc, r, k,
+                                                                         out, wsum_out);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return ctx_fail(c, DPCS_ERR_CUDA, cudaGetErrorString(e));
     ctx_add_launches(c, 1);
