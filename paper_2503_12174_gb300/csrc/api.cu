@@ -181,7 +181,8 @@ dpcs_status check_launch(dpcs_ctx *c, int n, const char *what) {
 
 // Gradient accumulators of one adjoint call (dEp always, dtex when a texture
 // gradient is wanted): packed float4, or FP64 in the FP64 accumulation mode.
-// Zeroes them on `st` and points the kernel arguments at them.
+// Points the kernel arguments at them; zeroes the FP64 ones on `st` (the packed
+// ones are cleared by launch_inputs).
 dpcs_status grad_setup(dpcs_ctx *c, int64_t np, int64_t nt, bool want_tex, cudaStream_t st, RenderArgs &a) {
     dpcs_status s;
     a.dEp = nullptr;
@@ -201,25 +202,75 @@ dpcs_status grad_setup(dpcs_ctx *c, int64_t np, int64_t nt, bool want_tex, cudaS
     if ((s = ensure(c, c->dEp4, (size_t)np * 16, "dEp scratch")) ||
         (want_tex && (s = ensure(c, c->dtex4, (size_t)nt * 16, "dtex scratch"))))
         return s;
-    cudaMemsetAsync(c->dEp4.p, 0, (size_t)np * 16, st);
-    if (want_tex) cudaMemsetAsync(c->dtex4.p, 0, (size_t)nt * 16, st);
     a.dEp = (float4 *)c->dEp4.p;
     a.dtex = want_tex ? (float4 *)c->dtex4.p : nullptr;
     return DPCS_OK;
 }
 
-// Eq. 1 adjoint and the texture gradients from the accumulators grad_setup
-// chose; returns the kernels enqueued
+// the maps of a call for launch_inputs
+InputArgs input_args(dpcs_ctx *c, const float *Ip, int64_t np, const dpcs_params *params, const float *albedo,
+                     const float *rough, int64_t nt) {
+    InputArgs q{};
+    q.Ip = Ip;
+    q.Ep = (float4 *)c->ep4.p;
+    q.np = np;
+    q.nt = nt;
+    for (int j = 0; j < 3; ++j) q.gamma[j] = params->gamma_p[j];
+    q.gain = params->gain_p;
+    q.albedo = albedo;
+    q.rough = rough;
+    q.tex = (float4 *)c->tex4.p;
+    return q;
+}
+InputArgs input_args(dpcs_ctx *c, const float *Ip, int64_t np, const dpcs_params *params, const dpcs_material *mat,
+                     int64_t nt) {
+    InputArgs q = input_args(c, Ip, np, params, mat->albedo, mat->rough, nt);
+    q.metallic = mat->metallic;
+    q.normal = mat->normal;
+    q.mat = (float4 *)c->mat4.p;
+    return q;
+}
+// only the accumulators of an adjoint whose maps are packed already
+InputArgs clear_args(int64_t np, int64_t nt) {
+    InputArgs q{};
+    q.np = np;
+    q.nt = nt;
+    return q;
+}
+OutputArgs output_args(const float *Ip, const float4 *dEp, int64_t np, int64_t nt, const dpcs_params *params, float *dIp,
+                       const float *dParams, double *acc, float *loss) {
+    OutputArgs q{};
+    q.Ip = Ip;
+    q.dEp = dEp;
+    q.np = np;
+    q.nt = nt;
+    for (int j = 0; j < 3; ++j) q.gamma[j] = params->gamma_p[j];
+    q.gain = params->gain_p;
+    q.acc = acc;
+    q.want_params = dParams != nullptr;
+    q.dIp = dIp;
+    q.loss = loss;
+    return q;
+}
+
+// Eq. 1 adjoint, the texture gradients and the loss (null: none) from the
+// accumulators grad_setup chose, and the parameter gradients; returns the
+// kernels enqueued
 int grad_finish(const RenderArgs &a, const float *Ip, int64_t np, int64_t nt, const dpcs_params *params, float *dIp,
-                float *dAlbedo, float *dRough, double *acc, cudaStream_t st) {
-    int nl;
+                float *dAlbedo, float *dRough, float *dParams, double *acc, float *loss, cudaStream_t st) {
+    int nl = 0;
     if (a.dEp64) {
-        nl = launch_prf_backward64(Ip, a.dEp64, np, params->gamma_p, params->gain_p, dIp, acc, st);
+        if (loss) nl += launch_loss_out(acc, loss, st);
+        nl += launch_prf_backward64(Ip, a.dEp64, np, params->gamma_p, params->gain_p, dIp, acc, st);
         if (a.dtex64) nl += launch_tex_backward64(a.dtex64, nt, dAlbedo, dRough, st);
     } else {
-        nl = launch_prf_backward(Ip, a.dEp, np, params->gamma_p, params->gain_p, dIp, acc, st);
-        if (a.dtex) nl += launch_tex_backward(a.dtex, nt, dAlbedo, dRough, st);
+        OutputArgs q = output_args(Ip, a.dEp, np, nt, params, dIp, dParams, acc, loss);
+        q.dtex = a.dtex;
+        q.dAlbedo = dAlbedo;
+        q.dRough = dRough;
+        nl += launch_outputs(q, st);
     }
+    if (dParams) nl += launch_finalize_params(acc, dParams, st);
     return nl;
 }
 
@@ -835,8 +886,7 @@ dpcs_status dpcs_render(dpcs_ctx *c, dpcs_scene scene, const float *albedo, cons
     a.tex = (const float4 *)c->tex4.p;
     a.Ic = Ic;
     a.Ec = Ec;
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(albedo, rough, nt, (float4 *)c->tex4.p, st);
+    int nl = launch_inputs(input_args(c, Ip, np, params, albedo, rough, nt), st);
     TimedLaunch *tl = timing_begin(c, 0, st);
     nl += wf ? launch_render_wavefront(a, c->wf_chunk, c->wf.p, st) : launch_render(a, st);
     timing_end(tl, st);
@@ -866,9 +916,11 @@ dpcs_status dpcs_render_backward(dpcs_ctx *c, dpcs_scene scene, const float *alb
     if ((s = grad_setup(c, np, nt, want_tex, st, a))) return s;
     void *recs = optional_scratch(c, c->recs, grad_scratch_bytes(a, true, kRecWordsHost), st);
     double *acc = (double *)c->acc.p;
-    cudaMemsetAsync(acc, 0, 16 * sizeof(double), st);
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(albedo, rough, nt, (float4 *)c->tex4.p, st);
+    InputArgs in = input_args(c, Ip, np, params, albedo, rough, nt);
+    in.acc = acc;
+    in.dEp = a.dEp;
+    in.dtex = a.dtex;
+    int nl = launch_inputs(in, st);
     nl += launch_crf_backward(dIc, Ec, Ic, npix, params->gamma_c, params->gain_c, params->wb, (float *)c->gE.p, acc, st);
     a.Ep = (const float4 *)c->ep4.p;
     a.tex = (const float4 *)c->tex4.p;
@@ -876,8 +928,7 @@ dpcs_status dpcs_render_backward(dpcs_ctx *c, dpcs_scene scene, const float *alb
     TimedLaunch *tl = timing_begin(c, 1, st);
     nl += launch_replay(a, acc, recs, st);
     timing_end(tl, st);
-    nl += grad_finish(a, Ip, np, nt, params, dIp, dAlbedo, dRough, acc, st);
-    if (dParams) nl += launch_finalize_params(acc, dParams, st);
+    nl += grad_finish(a, Ip, np, nt, params, dIp, dAlbedo, dRough, dParams, acc, nullptr, st);
     return check_launch(c, nl, "render_backward");
 }
 
@@ -904,9 +955,7 @@ dpcs_status dpcs_render_principled(dpcs_ctx *c, dpcs_scene scene, const dpcs_mat
     a.tex = (const float4 *)c->tex4.p;
     a.Ic = Ic;
     a.Ec = Ec;
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(mat->albedo, mat->rough, nt, (float4 *)c->tex4.p, st);
-    nl += launch_pack_mat(mat->metallic, mat->normal, nt, (float4 *)c->mat4.p, st);
+    int nl = launch_inputs(input_args(c, Ip, np, params, mat, nt), st);
     nl += launch_render_pbr(a, (const float4 *)c->mat4.p, st);
     return check_launch(c, nl, "render_principled");
 }
@@ -942,13 +991,12 @@ dpcs_status dpcs_render_backward_principled(dpcs_ctx *c, dpcs_scene scene, const
     if (want_mat && (s = ensure(c, c->dmat4, (size_t)nt * 16, "dmat scratch"))) return s;
     cudaStream_t st = (cudaStream_t)stream;
     double *acc = (double *)c->acc.p;
-    cudaMemsetAsync(acc, 0, 16 * sizeof(double), st);
-    cudaMemsetAsync(c->dEp4.p, 0, (size_t)np * 16, st);
-    if (want_tex) cudaMemsetAsync(c->dtex4.p, 0, (size_t)nt * 16, st);
-    if (want_mat) cudaMemsetAsync(c->dmat4.p, 0, (size_t)nt * 16, st);
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(mat->albedo, mat->rough, nt, (float4 *)c->tex4.p, st);
-    nl += launch_pack_mat(mat->metallic, mat->normal, nt, (float4 *)c->mat4.p, st);
+    InputArgs in = input_args(c, Ip, np, params, mat, nt);
+    in.acc = acc;
+    in.dEp = (float4 *)c->dEp4.p;
+    in.dtex = want_tex ? (float4 *)c->dtex4.p : nullptr;
+    in.dmat = want_mat ? (float4 *)c->dmat4.p : nullptr;
+    int nl = launch_inputs(in, st);
     nl += launch_crf_backward(dIc, Ec, Ic, npix, params->gamma_c, params->gain_c, params->wb, (float *)c->gE.p, acc, st);
     a.Ep = (const float4 *)c->ep4.p;
     a.tex = (const float4 *)c->tex4.p;
@@ -957,9 +1005,14 @@ dpcs_status dpcs_render_backward_principled(dpcs_ctx *c, dpcs_scene scene, const
     a.dtex = want_tex ? (float4 *)c->dtex4.p : nullptr;
     void *recs = optional_scratch(c, c->recs, grad_scratch_bytes(a, true, kPRecWordsHost), st);
     nl += launch_replay_pbr(a, (const float4 *)c->mat4.p, want_mat ? (float4 *)c->dmat4.p : nullptr, acc, recs, st);
-    nl += launch_prf_backward(Ip, (const float4 *)c->dEp4.p, np, params->gamma_p, params->gain_p, dIp, acc, st);
-    if (want_tex) nl += launch_tex_backward((const float4 *)c->dtex4.p, nt, dAlbedo, dRough, st);
-    if (want_mat) nl += launch_mat_backward((const float4 *)c->dmat4.p, nt, dMetallic, dNormal, st);
+    OutputArgs o = output_args(Ip, in.dEp, np, nt, params, dIp, dParams, acc, nullptr);
+    o.dtex = in.dtex;
+    o.dmat = in.dmat;
+    o.dAlbedo = dAlbedo;
+    o.dRough = dRough;
+    o.dMetallic = dMetallic;
+    o.dNormal = dNormal;
+    nl += launch_outputs(o, st);
     if (dParams) nl += launch_finalize_params(acc, dParams, st);
     return check_launch(c, nl, "render_backward_principled");
 }
@@ -984,8 +1037,7 @@ dpcs_status dpcs_render_keep(dpcs_ctx *c, dpcs_scene scene, const float *albedo,
         (s = ensure(c, c->kept, ((words + 255) & ~size_t(255)) + counts, "kept path records")))
         return s;
     cudaStream_t st = (cudaStream_t)stream;
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(albedo, rough, nt, (float4 *)c->tex4.p, st);
+    int nl = launch_inputs(input_args(c, Ip, np, params, albedo, rough, nt), st);
     a.Ep = (const float4 *)c->ep4.p;
     a.tex = (const float4 *)c->tex4.p;
     a.Ic = Ic;
@@ -1034,16 +1086,19 @@ dpcs_status dpcs_render_backward_kept(dpcs_ctx *c, dpcs_scene scene, const float
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = grad_setup(c, np, nt, want_tex, st, a))) return s;
     double *acc = (double *)c->acc.p;
-    cudaMemsetAsync(acc, 0, 16 * sizeof(double), st);
-    int nl = launch_crf_backward(dIc, Ec, Ic, npix, params->gamma_c, params->gain_c, params->wb, (float *)c->gE.p, acc,
+    InputArgs in = clear_args(np, nt);
+    in.acc = acc;
+    in.dEp = a.dEp;
+    in.dtex = a.dtex;
+    int nl = launch_inputs(in, st);
+    nl += launch_crf_backward(dIc, Ec, Ic, npix, params->gamma_c, params->gain_c, params->wb, (float *)c->gE.p, acc,
                                  st);
     a.gE = (const float *)c->gE.p;
     const char *kp = (const char *)c->kept.p;
     TimedLaunch *tl = timing_begin(c, 1, st);
     nl += launch_sweep_kept(a, kp, (const uint8_t *)(kp + ((words + 255) & ~size_t(255))), st);
     timing_end(tl, st);
-    nl += grad_finish(a, Ip, np, nt, params, dIp, dAlbedo, dRough, acc, st);
-    if (dParams) nl += launch_finalize_params(acc, dParams, st);
+    nl += grad_finish(a, Ip, np, nt, params, dIp, dAlbedo, dRough, dParams, acc, nullptr, st);
     return check_launch(c, nl, "render_backward_kept");
 }
 
@@ -1076,9 +1131,11 @@ dpcs_status dpcs_render_loss_backward(dpcs_ctx *c, dpcs_scene scene, const float
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = grad_setup(c, np, nt, want_tex, st, a))) return s;
     double *acc = (double *)c->acc.p;
-    cudaMemsetAsync(acc, 0, 16 * sizeof(double), st);
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(albedo, rough, nt, (float4 *)c->tex4.p, st);
+    InputArgs in = input_args(c, Ip, np, params, albedo, rough, nt);
+    in.acc = acc;
+    in.dEp = a.dEp;
+    in.dtex = a.dtex;
+    int nl = launch_inputs(in, st);
     a.Ep = (const float4 *)c->ep4.p;
     a.tex = (const float4 *)c->tex4.p;
     a.Ic = Ic;
@@ -1103,9 +1160,7 @@ dpcs_status dpcs_render_loss_backward(dpcs_ctx *c, dpcs_scene scene, const float
         nl += launch_replay(a, acc, recs, st);
         timing_end(tr, st);
     }
-    nl += launch_loss_out(acc, loss, st);
-    nl += grad_finish(a, Ip, np, nt, params, dIp, dAlbedo, dRough, acc, st);
-    if (dParams) nl += launch_finalize_params(acc, dParams, st);
+    nl += grad_finish(a, Ip, np, nt, params, dIp, dAlbedo, dRough, dParams, acc, loss, st);
     return check_launch(c, nl, "render_loss_backward");
 }
 
@@ -1134,9 +1189,7 @@ dpcs_status dpcs_render_keep_principled(dpcs_ctx *c, dpcs_scene scene, const dpc
         (s = ensure(c, c->kept, ((words + 255) & ~size_t(255)) + counts, "kept path records")))
         return s;
     cudaStream_t st = (cudaStream_t)stream;
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(mat->albedo, mat->rough, nt, (float4 *)c->tex4.p, st);
-    nl += launch_pack_mat(mat->metallic, mat->normal, nt, (float4 *)c->mat4.p, st);
+    int nl = launch_inputs(input_args(c, Ip, np, params, mat, nt), st);
     a.Ep = (const float4 *)c->ep4.p;
     a.tex = (const float4 *)c->tex4.p;
     a.Ic = Ic;
@@ -1194,11 +1247,13 @@ dpcs_status dpcs_render_backward_kept_principled(dpcs_ctx *c, dpcs_scene scene, 
         return s;
     cudaStream_t st = (cudaStream_t)stream;
     double *acc = (double *)c->acc.p;
-    cudaMemsetAsync(acc, 0, 16 * sizeof(double), st);
-    cudaMemsetAsync(c->dEp4.p, 0, (size_t)np * 16, st);
-    if (want_tex) cudaMemsetAsync(c->dtex4.p, 0, (size_t)nt * 16, st);
-    if (want_mat) cudaMemsetAsync(c->dmat4.p, 0, (size_t)nt * 16, st);
-    int nl = launch_crf_backward(dIc, Ec, Ic, npix, params->gamma_c, params->gain_c, params->wb, (float *)c->gE.p, acc,
+    InputArgs in = clear_args(np, nt);
+    in.acc = acc;
+    in.dEp = (float4 *)c->dEp4.p;
+    in.dtex = want_tex ? (float4 *)c->dtex4.p : nullptr;
+    in.dmat = want_mat ? (float4 *)c->dmat4.p : nullptr;
+    int nl = launch_inputs(in, st);
+    nl += launch_crf_backward(dIc, Ec, Ic, npix, params->gamma_c, params->gain_c, params->wb, (float *)c->gE.p, acc,
                                  st);
     a.gE = (const float *)c->gE.p;
     a.dEp = (float4 *)c->dEp4.p;
@@ -1206,9 +1261,14 @@ dpcs_status dpcs_render_backward_kept_principled(dpcs_ctx *c, dpcs_scene scene, 
     const char *kp = (const char *)c->kept.p;
     nl += launch_sweep_kept_pbr(a, kp, (const uint8_t *)(kp + ((words + 255) & ~size_t(255))),
                                 want_mat ? (float4 *)c->dmat4.p : nullptr, st);
-    nl += launch_prf_backward(Ip, (const float4 *)c->dEp4.p, np, params->gamma_p, params->gain_p, dIp, acc, st);
-    if (want_tex) nl += launch_tex_backward((const float4 *)c->dtex4.p, nt, dAlbedo, dRough, st);
-    if (want_mat) nl += launch_mat_backward((const float4 *)c->dmat4.p, nt, dMetallic, dNormal, st);
+    OutputArgs o = output_args(Ip, in.dEp, np, nt, params, dIp, dParams, acc, nullptr);
+    o.dtex = in.dtex;
+    o.dmat = in.dmat;
+    o.dAlbedo = dAlbedo;
+    o.dRough = dRough;
+    o.dMetallic = dMetallic;
+    o.dNormal = dNormal;
+    nl += launch_outputs(o, st);
     if (dParams) nl += launch_finalize_params(acc, dParams, st);
     return check_launch(c, nl, "render_backward_kept_principled");
 }
@@ -1251,13 +1311,12 @@ dpcs_status dpcs_render_loss_backward_principled(dpcs_ctx *c, dpcs_scene scene, 
         return s;
     cudaStream_t st = (cudaStream_t)stream;
     double *acc = (double *)c->acc.p;
-    cudaMemsetAsync(acc, 0, 16 * sizeof(double), st);
-    cudaMemsetAsync(c->dEp4.p, 0, (size_t)np * 16, st);
-    if (want_tex) cudaMemsetAsync(c->dtex4.p, 0, (size_t)nt * 16, st);
-    if (want_mat) cudaMemsetAsync(c->dmat4.p, 0, (size_t)nt * 16, st);
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(mat->albedo, mat->rough, nt, (float4 *)c->tex4.p, st);
-    nl += launch_pack_mat(mat->metallic, mat->normal, nt, (float4 *)c->mat4.p, st);
+    InputArgs in = input_args(c, Ip, np, params, mat, nt);
+    in.acc = acc;
+    in.dEp = (float4 *)c->dEp4.p;
+    in.dtex = want_tex ? (float4 *)c->dtex4.p : nullptr;
+    in.dmat = want_mat ? (float4 *)c->dmat4.p : nullptr;
+    int nl = launch_inputs(in, st);
     a.Ep = (const float4 *)c->ep4.p;
     a.tex = (const float4 *)c->tex4.p;
     a.Ic = Ic;
@@ -1280,10 +1339,14 @@ dpcs_status dpcs_render_loss_backward_principled(dpcs_ctx *c, dpcs_scene scene, 
         a.gE = (const float *)c->gE.p;
         nl += launch_replay_pbr(a, m4, dm4, acc, recs, st);
     }
-    nl += launch_loss_out(acc, loss, st);
-    nl += launch_prf_backward(Ip, (const float4 *)c->dEp4.p, np, params->gamma_p, params->gain_p, dIp, acc, st);
-    if (want_tex) nl += launch_tex_backward((const float4 *)c->dtex4.p, nt, dAlbedo, dRough, st);
-    if (want_mat) nl += launch_mat_backward((const float4 *)c->dmat4.p, nt, dMetallic, dNormal, st);
+    OutputArgs o = output_args(Ip, in.dEp, np, nt, params, dIp, dParams, acc, loss);
+    o.dtex = in.dtex;
+    o.dmat = in.dmat;
+    o.dAlbedo = dAlbedo;
+    o.dRough = dRough;
+    o.dMetallic = dMetallic;
+    o.dNormal = dNormal;
+    nl += launch_outputs(o, st);
     if (dParams) nl += launch_finalize_params(acc, dParams, st);
     return check_launch(c, nl, "render_loss_backward_principled");
 }
@@ -1371,9 +1434,13 @@ static dpcs_status pose_backward_impl(dpcs_ctx *c, dpcs_scene scene, const float
         (s = ensure(c, c->pose, (size_t)3 * gmax * 6 * sizeof(double), "pose partial sums")) ||
         (pbr && (s = ensure(c, c->mat4, (size_t)nt * 16, "material scratch"))))
         return s;
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, (float4 *)c->ep4.p, st);
-    nl += launch_pack_tex(albedo, rough, nt, (float4 *)c->tex4.p, st);
-    if (pbr) nl += launch_pack_mat(metallic, normal, nt, (float4 *)c->mat4.p, st);
+    InputArgs in = input_args(c, Ip, np, params, albedo, rough, nt);
+    if (pbr) {
+        in.metallic = metallic;
+        in.normal = normal;
+        in.mat = (float4 *)c->mat4.p;
+    }
+    int nl = launch_inputs(in, st);
     // dLoss/dEc through Eq. 5 (the response-parameter sums it also forms are not used)
     nl += launch_crf_backward(dIc, Ec, Ic, npix, params->gamma_c, params->gain_c, params->wb, (float *)c->gE.p,
                               (double *)c->acc.p, st);
@@ -1480,8 +1547,10 @@ extern "C" dpcs_status dpcs_render_noalloc(dpcs_ctx *c, dpcs_scene scene, const 
     a.tex = tex4;
     a.Ic = Ic;
     a.Ec = Ec;
-    int nl = launch_prf(Ip, np, params->gamma_p, params->gain_p, ep4, st);
-    nl += launch_pack_tex(albedo, rough, nt, tex4, st);
+    InputArgs in = input_args(c, Ip, np, params, albedo, rough, nt);
+    in.Ep = ep4;
+    in.tex = tex4;
+    int nl = launch_inputs(in, st);
     nl += launch_render(a, st);
     return check_launch(c, nl, "render_noalloc");
 }

@@ -109,6 +109,34 @@ struct BatchSeg {
     int32_t pad;
 };
 
+// The maps of one call, packed for its kernels, and an adjoint's FP32
+// accumulators to clear; any pointer may be null (left out).
+struct InputArgs {
+    const float *Ip;     // np x 3 projector image
+    float4 *Ep;          // np: Eq. 1
+    int64_t np, nt;
+    float gamma[3], gain;
+    const float *albedo, *rough;
+    float4 *tex;         // nt: albedo rgb, roughness
+    const float *metallic, *normal;  // null with mat set: 0 and (0.5, 0.5, 1)
+    float4 *mat;         // nt: metallic, normal map
+    float4 *dEp, *dtex, *dmat;
+    double *acc;         // 16 parameter accumulators
+};
+// What an adjoint adds to the caller's buffers (each null: not wanted).
+struct OutputArgs {
+    const float *Ip;
+    const float4 *dEp;
+    int64_t np, nt;
+    float gamma[3], gain;
+    double *acc;
+    bool want_params;    // reduce the gradients of gamma_p and Gp into acc[0..3]
+    float *dIp;
+    const float4 *dtex, *dmat;
+    float *dAlbedo, *dRough, *dMetallic, *dNormal;
+    float *loss;         // = acc[11]
+};
+
 // Launchers (render.cu, lbvh.cu, optim.cu).  Each returns the number of
 // kernels it enqueued, or a negative dpcs_status.
 int launch_lbvh_build(const float *d_verts, int32_t V, const int32_t *d_tris, int32_t T, const float *d_uv,
@@ -129,6 +157,8 @@ size_t ploc_scratch_bytes(int32_t T);
 int launch_ploc(Scene &sc, void *scratch, size_t scratch_bytes, int max_depth, cudaStream_t st, int32_t *depth_out);
 constexpr int kMaxTreeDepth = 64;  // internal nodes on a root-to-leaf path: the traversal stack's depth
 
+int launch_inputs(const InputArgs &q, cudaStream_t st);
+int launch_outputs(const OutputArgs &q, cudaStream_t st);
 int launch_prf(const float *Ip, int64_t ntex, const float gamma_p[3], float gain_p, float4 *Ep, cudaStream_t st);
 int launch_pack_tex(const float *albedo, const float *rough, int64_t ntex, float4 *tex, cudaStream_t st);
 int launch_render(const RenderArgs &a, cudaStream_t st);
@@ -156,10 +186,8 @@ int launch_replay(const RenderArgs &a, double *acc, void *scratch, cudaStream_t 
 int launch_render_grad(const RenderArgs &a, const LossArgs &l, void *scratch, cudaStream_t st);
 int launch_pixel_loss(const float *Ic, int64_t n, const LossArgs &l, float *dIc, cudaStream_t st);
 // principled material (principled.cu)
-int launch_pack_mat(const float *metallic, const float *normal, int64_t ntex, float4 *mat, cudaStream_t st);
 int launch_render_pbr(const RenderArgs &a, const float4 *mat, cudaStream_t st);
 int launch_replay_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, double *acc, void *scratch, cudaStream_t st);
-int launch_mat_backward(const float4 *dmat, int64_t ntex, float *dMetallic, float *dNormal, cudaStream_t st);
 int launch_render_grad_pbr(const RenderArgs &a, const float4 *mat, float4 *dmat, const LossArgs &l, void *scratch,
                            cudaStream_t st);
 // kept principled records: kPRecWordsHost 32-bit words per vertex
@@ -168,10 +196,7 @@ int launch_sweep_kept_pbr(const RenderArgs &a, const void *chunks, const uint8_t
 int launch_render_keep(const RenderArgs &a, void *chunks, uint8_t *nvs, cudaStream_t st);
 int launch_sweep_kept(const RenderArgs &a, const void *chunks, const uint8_t *nvs, cudaStream_t st);
 int launch_loss_out(const double *acc, float *loss, cudaStream_t st);
-int launch_prf_backward(const float *Ip, const float4 *dEp, int64_t ntex, const float gamma_p[3], float gain_p,
-                        float *dIp, double *acc, cudaStream_t st);
-int launch_tex_backward(const float4 *dtex, int64_t ntex, float *dAlbedo, float *dRough, cudaStream_t st);
-// the same from the FP64 accumulators (dEp64: 3 per texel, dtex64: 4 per texel)
+// outputs of the plain material from the FP64 accumulators (dEp64: 3 per texel, dtex64: 4 per texel)
 int launch_prf_backward64(const float *Ip, const double *dEp64, int64_t ntex, const float gamma_p[3], float gain_p,
                           float *dIp, double *acc, cudaStream_t st);
 int launch_tex_backward64(const double *dtex64, int64_t ntex, float *dAlbedo, float *dRough, cudaStream_t st);

@@ -13,7 +13,8 @@
 // continuations below the geometric surface are dropped.  metallic 0 and
 // Vn = (0.5, 0.5, 1) give the plain material.
 //
-// Kernels: k_pack_mat interleaves (metallic, Vn) into one float4 per texel;
+// Kernels (render.cu's k_inputs interleaves (metallic, Vn) into one float4 per
+// texel, its k_outputs adds their gradients to the caller's buffers):
 // k_render_pbr is k_render's loop (same thread mapping, same sample rounds,
 // same xor-shuffle pixel sum) with this material; k_replay_pbr re-traces the
 // paths, records each vertex and runs the reverse sweep with the material's
@@ -23,9 +24,7 @@
 // pixel's loss gradient through Eq. 5, then the sweeps; k_render_keep_pbr and
 // k_sweep_kept_pbr keep the records in device memory for losses that couple
 // pixels (the Eq. 11 filter), as k_render_keep / k_sweep_kept do;
-// the *_pbr_tile kernels run the same paths over block tiles (tile.cuh);
-// k_mat_backward adds the metallic and normal-map gradients to the caller's
-// buffers.
+// the *_pbr_tile kernels run the same paths over block tiles (tile.cuh).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -653,36 +652,9 @@ __global__ void __launch_bounds__(B, 1024 / B)
                        });
 }
 
-__global__ void k_pack_mat(const float *__restrict__ metallic, const float *__restrict__ normal, int64_t ntex,
-                           float4 *__restrict__ mat) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= ntex) return;
-    mat[t] = make_float4(metallic ? metallic[t] : 0.0f, normal ? normal[3 * t] : 0.5f, normal ? normal[3 * t + 1] : 0.5f,
-                         normal ? normal[3 * t + 2] : 1.0f);
-}
-
-__global__ void k_mat_backward(const float4 *__restrict__ dmat, int64_t ntex, float *__restrict__ dMetallic,
-                               float *__restrict__ dNormal) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= ntex) return;
-    const float4 g = dmat[t];
-    if (dMetallic) dMetallic[t] += g.x;
-    if (dNormal) {
-        dNormal[3 * t] += g.y;
-        dNormal[3 * t + 1] += g.z;
-        dNormal[3 * t + 2] += g.w;
-    }
-}
-
 inline unsigned grid1(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
 }  // namespace
-
-int launch_pack_mat(const float *metallic, const float *normal, int64_t ntex, float4 *mat, cudaStream_t st) {
-    if (ntex <= 0) return 0;
-    k_pack_mat<<<grid1(ntex, 256), 256, 0, st>>>(metallic, normal, ntex, mat);
-    return 1;
-}
 
 int launch_render_pbr(const RenderArgs &a, const float4 *mat, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
@@ -754,12 +726,6 @@ int launch_sweep_kept_pbr(const RenderArgs &a, const void *chunks, const uint8_t
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
     if (threads <= 0) return 0;
     k_sweep_kept_pbr<<<grid1(threads, kPBlock), kPBlock, 0, st>>>(a, (const uint4 *)chunks, nvs, dmat);
-    return 1;
-}
-
-int launch_mat_backward(const float4 *dmat, int64_t ntex, float *dMetallic, float *dNormal, cudaStream_t st) {
-    if (ntex <= 0 || (!dMetallic && !dNormal)) return 0;
-    k_mat_backward<<<grid1(ntex, 256), 256, 0, st>>>(dmat, ntex, dMetallic, dNormal);
     return 1;
 }
 

@@ -1,14 +1,14 @@
 // render.cu -- forward rendering and its path-replay adjoint.
 //
-// Forward (Eq. 7): k_prf maps the projector image through the PRF (Eq. 1),
-// k_pack_tex interleaves albedo and roughness into one float4 per texel, and
+// Forward (Eq. 7): k_inputs maps the projector image through the PRF (Eq. 1)
+// and interleaves albedo and roughness into one float4 per texel, and
 // k_render traces every camera path (Eqs. 3, 6, 10) and applies the camera
 // response (Eqs. 4, 5) in its epilogue.
 //
 // Adjoint: k_crf_backward turns dLoss/dIc into dLoss/dEc (Eq. 5), k_replay
 // re-traces each path from its Philox counters and scatters gradients into
-// the projector and texture accumulators, k_prf_backward applies Eq. 1's
-// derivative, and k_tex_backward / k_finalize add the results to the
+// the projector and texture accumulators, k_outputs applies Eq. 1's
+// derivative and k_outputs / k_finalize add the results to the
 // caller's buffers.
 //
 // Thread mapping: L = 2^log2L consecutive lanes of a warp share one camera
@@ -106,20 +106,35 @@ __device__ __forceinline__ void scatter_add4(float4 *base, int key, float4 v, fl
     atomic_add4(base + key, v);
 }
 
-__global__ void k_prf(const float *__restrict__ Ip, int64_t ntex, float g0, float g1, float g2, float gain,
-                      float4 *__restrict__ Ep) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= ntex) return;
-    const float a = Ip[3 * t], b = Ip[3 * t + 1], c = Ip[3 * t + 2];
-    Ep[t] = make_float4(a > 0.0f ? gain * powf(a, g0) : 0.0f, b > 0.0f ? gain * powf(b, g1) : 0.0f,
-                        c > 0.0f ? gain * powf(c, g2) : 0.0f, 0.0f);
-}
-
-__global__ void k_pack_tex(const float *__restrict__ albedo, const float *__restrict__ rough, int64_t ntex,
-                           float4 *__restrict__ tex) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= ntex) return;
-    tex[t] = make_float4(albedo[3 * t], albedo[3 * t + 1], albedo[3 * t + 2], rough[t]);
+// Eq. 1 on the projector image, the maps interleaved one texel a float4, and
+// an adjoint's accumulators cleared, in one launch: the first blocks take the
+// projector's texels, the others the maps'.  Each of the three to seven
+// launches and clears this replaces moved little and cost about 2 us of its
+// own (a render of the 64 x 64 plane, 1 bounce, 18 -> 16.5 us; a principled
+// step of 256 x 256, 659 -> 631 us).
+__global__ void __launch_bounds__(256) k_inputs(const InputArgs q, unsigned bp) {
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (blockIdx.x < bp) {
+        const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+        if (q.acc && t < 16) q.acc[t] = 0.0;
+        if (t >= q.np) return;
+        if (q.dEp) q.dEp[t] = zero;
+        if (q.Ep) {
+            const float a = q.Ip[3 * t], b = q.Ip[3 * t + 1], c = q.Ip[3 * t + 2];
+            q.Ep[t] = make_float4(a > 0.0f ? q.gain * powf(a, q.gamma[0]) : 0.0f,
+                                  b > 0.0f ? q.gain * powf(b, q.gamma[1]) : 0.0f,
+                                  c > 0.0f ? q.gain * powf(c, q.gamma[2]) : 0.0f, 0.0f);
+        }
+        return;
+    }
+    const int64_t t = (blockIdx.x - bp) * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= q.nt) return;
+    if (q.tex) q.tex[t] = make_float4(q.albedo[3 * t], q.albedo[3 * t + 1], q.albedo[3 * t + 2], q.rough[t]);
+    if (q.mat)
+        q.mat[t] = make_float4(q.metallic ? q.metallic[t] : 0.0f, q.normal ? q.normal[3 * t] : 0.5f,
+                               q.normal ? q.normal[3 * t + 1] : 0.5f, q.normal ? q.normal[3 * t + 2] : 1.0f);
+    if (q.dtex) q.dtex[t] = zero;
+    if (q.dmat) q.dmat[t] = zero;
 }
 
 // Forward megakernel.  Every loop iteration traces exactly one ray per lane --
@@ -1042,30 +1057,58 @@ __global__ void __launch_bounds__(B, 1024 / B) k_grad_tile(const RenderArgs a, c
                        });
 }
 
-// Eq. 1 adjoint: dIp += dEp Gp gamma Ip^(gamma-1); gamma_p and Gp reductions
-__global__ void k_prf_backward(const float *__restrict__ Ip, const float4 *__restrict__ dEp, int64_t ntex,
-                               float g0, float g1, float g2, float gain, float *__restrict__ dIp, double *acc) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    float v[4] = {0, 0, 0, 0};
-    if (t < ntex) {
-        const float4 g4 = dEp[t];
-        const float gs[3] = {g4.x, g4.y, g4.z}, gm[3] = {g0, g1, g2};
+// What an adjoint hands back, in one launch laid out as k_inputs: Eq. 1's
+// adjoint dIp += dEp Gp gamma Ip^(gamma-1) with the reductions over gamma_p
+// and Gp (left out when no parameter gradient is wanted), the gradients of the
+// maps, and the loss.
+__global__ void __launch_bounds__(256) k_outputs(const OutputArgs q, unsigned bp) {
+    if (blockIdx.x < bp) {
+        const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+        if (q.loss && t == 0) *q.loss = (float)q.acc[11];
+        float v[4] = {0, 0, 0, 0};
+        if (t < q.np) {
+            const float4 g4 = q.dEp[t];
+            const float gs[3] = {g4.x, g4.y, g4.z};
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const float ip = Ip[3 * t + j];
-            if (ip > 0.0f && gs[j] != 0.0f) {
-                const float pw = powf(ip, gm[j]);
-                if (dIp) dIp[3 * t + j] += gs[j] * gain * gm[j] * powf(ip, gm[j] - 1.0f);
-                v[j] += gs[j] * gain * pw * logf(ip);
-                v[3] += gs[j] * pw;
+            for (int j = 0; j < 3; ++j) {
+                const float ip = q.Ip[3 * t + j];
+                if (ip > 0.0f && gs[j] != 0.0f) {
+                    if (q.dIp) q.dIp[3 * t + j] += gs[j] * q.gain * q.gamma[j] * powf(ip, q.gamma[j] - 1.0f);
+                    if (q.want_params) {
+                        const float pw = powf(ip, q.gamma[j]);
+                        v[j] += gs[j] * q.gain * pw * logf(ip);
+                        v[3] += gs[j] * pw;
+                    }
+                }
             }
         }
+        if (q.want_params) block_reduce_add<4>(v, q.acc);
+        return;
     }
-    block_reduce_add<4>(v, acc);
+    const int64_t t = (blockIdx.x - bp) * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= q.nt) return;
+    if (q.dtex) {
+        const float4 g = q.dtex[t];
+        if (q.dAlbedo) {
+            q.dAlbedo[3 * t] += g.x;
+            q.dAlbedo[3 * t + 1] += g.y;
+            q.dAlbedo[3 * t + 2] += g.z;
+        }
+        if (q.dRough) q.dRough[t] += g.w;
+    }
+    if (q.dmat) {
+        const float4 g = q.dmat[t];
+        if (q.dMetallic) q.dMetallic[t] += g.x;
+        if (q.dNormal) {
+            q.dNormal[3 * t] += g.y;
+            q.dNormal[3 * t + 1] += g.z;
+            q.dNormal[3 * t + 2] += g.w;
+        }
+    }
 }
 
 // the same from FP64 accumulators: the per-texel factors Ip^gamma, its
-// derivative and ln Ip in FP32 (as k_prf_backward), the products and the
+// derivative and ln Ip in FP32 (as k_outputs), the products and the
 // reductions in FP64 before the result is rounded
 __global__ void k_prf_backward64(const float *__restrict__ Ip, const double *__restrict__ dEp, int64_t ntex,
                                  float g0, float g1, float g2, float gain, float *__restrict__ dIp, double *acc) {
@@ -1113,19 +1156,6 @@ __global__ void k_tex_backward64(const double *__restrict__ dtex, int64_t ntex, 
     if (dRough) dRough[t] += (float)dtex[4 * t + 3];
 }
 
-__global__ void k_tex_backward(const float4 *__restrict__ dtex, int64_t ntex, float *__restrict__ dAlbedo,
-                               float *__restrict__ dRough) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= ntex) return;
-    const float4 g = dtex[t];
-    if (dAlbedo) {
-        dAlbedo[3 * t] += g.x;
-        dAlbedo[3 * t + 1] += g.y;
-        dAlbedo[3 * t + 2] += g.z;
-    }
-    if (dRough) dRough[t] += g.w;
-}
-
 // the per-pixel loss of LossArgs as its own pass (when k_render_grad would
 // need more records than it keeps): dIc, and the loss into acc[11]
 __global__ void k_pixel_loss(const float *__restrict__ Ic, int64_t n, const LossArgs l, float *__restrict__ dIc) {
@@ -1152,14 +1182,30 @@ inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 
 
 }  // namespace
 
-int launch_prf(const float *Ip, int64_t ntex, const float gamma_p[3], float gain_p, float4 *Ep, cudaStream_t st) {
-    k_prf<<<grid_for(ntex, 256), 256, 0, st>>>(Ip, ntex, gamma_p[0], gamma_p[1], gamma_p[2], gain_p, Ep);
+int launch_inputs(const InputArgs &q, cudaStream_t st) {
+    const unsigned bp = grid_for(q.Ep || q.dEp ? q.np : (q.acc ? 1 : 0), 256);
+    const unsigned bt = grid_for(q.tex || q.mat || q.dtex || q.dmat ? q.nt : 0, 256);
+    k_inputs<<<bp + bt, 256, 0, st>>>(q, bp);
     return 1;
 }
 
+int launch_prf(const float *Ip, int64_t ntex, const float gamma_p[3], float gain_p, float4 *Ep, cudaStream_t st) {
+    InputArgs q{};
+    q.Ip = Ip;
+    q.np = ntex;
+    for (int j = 0; j < 3; ++j) q.gamma[j] = gamma_p[j];
+    q.gain = gain_p;
+    q.Ep = Ep;
+    return launch_inputs(q, st);
+}
+
 int launch_pack_tex(const float *albedo, const float *rough, int64_t ntex, float4 *tex, cudaStream_t st) {
-    k_pack_tex<<<grid_for(ntex, 256), 256, 0, st>>>(albedo, rough, ntex, tex);
-    return 1;
+    InputArgs q{};
+    q.albedo = albedo;
+    q.rough = rough;
+    q.nt = ntex;
+    q.tex = tex;
+    return launch_inputs(q, st);
 }
 
 int launch_render(const RenderArgs &a, cudaStream_t st) {
@@ -1283,15 +1329,9 @@ int launch_loss_out(const double *acc, float *loss, cudaStream_t st) {
     return 1;
 }
 
-int launch_prf_backward(const float *Ip, const float4 *dEp, int64_t ntex, const float gamma_p[3], float gain_p,
-                        float *dIp, double *acc, cudaStream_t st) {
-    k_prf_backward<<<grid_for(ntex, 256), 256, 0, st>>>(Ip, dEp, ntex, gamma_p[0], gamma_p[1], gamma_p[2], gain_p,
-                                                        dIp, acc);
-    return 1;
-}
-
-int launch_tex_backward(const float4 *dtex, int64_t ntex, float *dAlbedo, float *dRough, cudaStream_t st) {
-    k_tex_backward<<<grid_for(ntex, 256), 256, 0, st>>>(dtex, ntex, dAlbedo, dRough);
+int launch_outputs(const OutputArgs &q, cudaStream_t st) {
+    const unsigned bp = grid_for(q.np, 256), bt = grid_for(q.dtex || q.dmat ? q.nt : 0, 256);
+    k_outputs<<<bp + bt, 256, 0, st>>>(q, bp);
     return 1;
 }
 

@@ -220,6 +220,28 @@ void *step_scratch(dpcs_server *s, const RenderArgs &a, bool replay) {
     return p;
 }
 
+// a step's accumulators cleared, and Eq. 1's adjoint into G (with the loss of
+// a one-trace step)
+int clear_step(const Req *q, int64_t np, cudaStream_t st) {
+    InputArgs in{};
+    in.np = np;
+    in.dEp = q->dEp4;
+    in.acc = q->acc;
+    return launch_inputs(in, st);
+}
+int finish_step(const Req *q, const ServeScene &sc, int64_t np, float *loss, cudaStream_t st) {
+    OutputArgs o{};
+    o.Ip = q->Ip;
+    o.dEp = q->dEp4;
+    o.np = np;
+    for (int j = 0; j < 3; ++j) o.gamma[j] = sc.params.gamma_p[j];
+    o.gain = sc.params.gain_p;
+    o.acc = q->acc;
+    o.dIp = q->G;
+    o.loss = loss;
+    return launch_outputs(o, st);
+}
+
 // one compensation step after its render: L2 loss, path replay, PRF
 // adjoint, Adam on Ip with the clamp to [0, 1], then Ep for the next render
 int enqueue_comp_backward(dpcs_server *s, Req *q) {
@@ -227,8 +249,7 @@ int enqueue_comp_backward(dpcs_server *s, Req *q) {
     const int64_t np = (int64_t)sc.view.Hp * sc.view.Wp;
     cudaStream_t st = s->stream;
     int n = launch_l2_loss(q->Ic, q->target, q->npix * 3, q->dIc, q->loss, q->partial, st);
-    cudaMemsetAsync(q->acc, 0, 16 * 8, st);
-    cudaMemsetAsync(q->dEp4, 0, (size_t)np * 16, st);
+    n += clear_step(q, np, st);
     cudaMemsetAsync(q->G, 0, (size_t)np * 12, st);
     n += launch_crf_backward(q->dIc, q->Ec, q->Ic, q->npix, sc.params.gamma_c, sc.params.gain_c, sc.params.wb, q->gE,
                              q->acc, st);
@@ -237,7 +258,7 @@ int enqueue_comp_backward(dpcs_server *s, Req *q) {
     a.dEp = q->dEp4;
     a.dtex = nullptr;  // only Ip is optimised
     n += launch_replay(a, q->acc, step_scratch(s, a, true), st);
-    n += launch_prf_backward(q->Ip, q->dEp4, np, sc.params.gamma_p, sc.params.gain_p, q->G, q->acc, st);
+    n += finish_step(q, sc, np, nullptr, st);
     n += launch_adam(q->Ip, q->G, q->M, q->V, np * 3, q->r.lr, 0.9f, 0.999f, 1e-8f, q->steps_issued, 0.0f, 1.0f, st);
     n += launch_prf(q->Ip, np, sc.params.gamma_p, sc.params.gain_p, q->Ep4, st);
     return n;
@@ -255,16 +276,14 @@ int enqueue_comp_step_fused(dpcs_server *s, Req *q) {
     const ServeScene &sc = s->scenes[q->r.scene];
     const int64_t np = (int64_t)sc.view.Hp * sc.view.Wp;
     cudaStream_t st = s->stream;
-    cudaMemsetAsync(q->acc, 0, 16 * 8, st);
-    cudaMemsetAsync(q->dEp4, 0, (size_t)np * 16, st);
+    int n = clear_step(q, np, st);
     cudaMemsetAsync(q->G, 0, (size_t)np * 12, st);
     RenderArgs a = q->args;
     a.dEp = q->dEp4;
     a.dtex = nullptr;  // only Ip is optimised
     const LossArgs l{q->target, 1.0f, 0, q->acc};
-    int n = launch_render_grad(a, l, step_scratch(s, a, false), st);
-    n += launch_loss_out(q->acc, q->loss, st);
-    n += launch_prf_backward(q->Ip, q->dEp4, np, sc.params.gamma_p, sc.params.gain_p, q->G, q->acc, st);
+    n += launch_render_grad(a, l, step_scratch(s, a, false), st);
+    n += finish_step(q, sc, np, q->loss, st);
     n += launch_adam(q->Ip, q->G, q->M, q->V, np * 3, q->r.lr, 0.9f, 0.999f, 1e-8f, q->steps_issued, 0.0f, 1.0f, st);
     n += launch_prf(q->Ip, np, sc.params.gamma_p, sc.params.gain_p, q->Ep4, st);
     return n;
