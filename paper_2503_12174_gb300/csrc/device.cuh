@@ -531,6 +531,41 @@ struct Hit {
 // still traversing; it returns true once the ray is resolved.  Every call
 // advances by one or more steps, so a lane that keeps calling it finishes its
 // ray within the visit cap.
+typedef unsigned long long u64;
+__device__ __forceinline__ u64 pk2(float a, float b) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void up2(u64 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+    u64 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// 32 bytes of a tree node (64-byte aligned) in one load
+__device__ __forceinline__ void ldg8(const float4 *p, float4 &a, float4 &b) {
+    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
+
+// slab() with the two planes of an axis in one packed FMA (the
+// same roundings; a node lists them side by side)
+__device__ __forceinline__ bool slab2(u64 x, u64 y, u64 z, u64 ix, u64 iy, u64 iz, u64 ox, u64 oy, u64 oz, float err,
+                                      float tmax, float &tnear) {
+    float tx0, tx1, ty0, ty1, tz0, tz1;
+    up2(fma2(x, ix, ox), tx0, tx1);
+    up2(fma2(y, iy, oy), ty0, ty1);
+    up2(fma2(z, iz, oz), tz0, tz1);
+    const float tn = fmax3f(fminf(tx0, tx1), fminf(ty0, ty1), fmaxf(fminf(tz0, tz1), 0.0f));
+    const float tf = fmin3f(fmaxf(tx0, tx1), fmaxf(ty0, ty1), fminf(fmaxf(tz0, tz1), tmax));
+    tnear = tn;
+    return tn <= fmaf(tf, 1.0000004f, err);
+}
+
 struct Trav {
     int node, sp, visits;
     bool any;
@@ -575,13 +610,27 @@ __device__ __forceinline__ bool trav_resume(const float4 *__restrict__ nodes, co
 #endif
         if (node >= 0) {
             cnt.add(kCntNode);
-            const float4 n0 = __ldg(nodes + 4 * node + 0);
-            const float4 n1 = __ldg(nodes + 4 * node + 1);
-            const float4 n2 = __ldg(nodes + 4 * node + 2);
-            const float4 n3 = __ldg(nodes + 4 * node + 3);
+            float4 n0, n1, n2, n3;
             float tl, tr;
+#ifdef DPCS_FUSION_BY_COMPILER
+            n0 = __ldg(nodes + 4 * node + 0);
+            n1 = __ldg(nodes + 4 * node + 1);
+            n2 = __ldg(nodes + 4 * node + 2);
+            n3 = __ldg(nodes + 4 * node + 3);
             const bool hl = slab(ray, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, st.h.t, tl);
             const bool hr = slab(ray, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, st.h.t, tr);
+#else
+            // two loads a node and packed slabs: 200k-triangle heightfield,
+            // 1024 x 1024 x 16 spp, 8.24 -> 8.09 ms
+            const float4 *nd = nodes + 4 * (size_t)(uint32_t)node;
+            ldg8(nd, n0, n1);
+            ldg8(nd + 2, n2, n3);
+            const u64 ix = pk2(ray.inv.x, ray.inv.x), iy = pk2(ray.inv.y, ray.inv.y), iz = pk2(ray.inv.z, ray.inv.z);
+            const u64 ox = pk2(-ray.oinv.x, -ray.oinv.x), oy = pk2(-ray.oinv.y, -ray.oinv.y),
+                      oz = pk2(-ray.oinv.z, -ray.oinv.z);
+            const bool hl = slab2(pk2(n0.x, n0.y), pk2(n0.z, n0.w), pk2(n2.x, n2.y), ix, iy, iz, ox, oy, oz, ray.err, st.h.t, tl);
+            const bool hr = slab2(pk2(n1.x, n1.y), pk2(n1.z, n1.w), pk2(n2.z, n2.w), ix, iy, iz, ox, oy, oz, ray.err, st.h.t, tr);
+#endif
             const int cl = __float_as_int(n3.x), cr = __float_as_int(n3.y);
             if (hl && hr) {
                 if (st.sp >= kStack) {

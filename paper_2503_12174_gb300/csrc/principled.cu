@@ -713,7 +713,7 @@ static_assert(sizeof(PRec) % 16 == 0, "PRec must be whole 16-byte chunks");
 int launch_render_keep_pbr(const RenderArgs &a, const float4 *mat, void *chunks, uint8_t *nvs, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
     if (threads <= 0) return 0;
-    if (!tiled(a) || a.root == kEmptyRoot)
+    if (!tiled_records(a) || a.root == kEmptyRoot)
         k_render_keep_pbr<<<grid1(threads, kPBlock), kPBlock, 0, st>>>(a, mat, (uint4 *)chunks, nvs);
     else if (small_tiles(a))
         k_keep_pbr_tile<64, 64><<<grid1(threads, 64), 64, 0, st>>>(a, mat, (uint4 *)chunks, nvs);

@@ -41,12 +41,6 @@ constexpr int kRenderBlock = 128;
 // iterations and shade together; 0: it goes straight to its extension ray
 #define DPCS_ALIGN_SHADOW 1
 #endif
-#ifndef DPCS_RENDER_MINB
-// minimum resident blocks per SM requested from ptxas for k_render: 8 (64
-// registers) against 10 (48 registers, with spills) measured 2 % faster on
-// the corner and 2 % slower on the 200k-triangle heightfield
-#define DPCS_RENDER_MINB 8
-#endif
 #ifndef DPCS_GRAD_MINB
 // the same for the kernels that keep vertex records (replay, fused step,
 // kept records): 8 blocks (64 registers) measured 3-5 % faster than 10
@@ -279,7 +273,8 @@ __device__ __forceinline__ void render_lanes(const RenderArgs &a, int64_t pix, i
     if (valid && sl == 0) write_pixel(a, pix, sum);
 }
 
-__global__ void __launch_bounds__(kRenderBlock, DPCS_RENDER_MINB) k_render(const RenderArgs a) {
+template <int kMinBlocks>
+__global__ void __launch_bounds__(kRenderBlock, kMinBlocks) k_render(const RenderArgs a) {
     const int64_t gt = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t pix = gt >> a.log2L;
     render_lanes(a, pix, (int)(gt & ((1 << a.log2L) - 1)), pix < (int64_t)a.Hc * a.Wc);
@@ -1176,7 +1171,12 @@ __global__ void k_finalize(const double *__restrict__ acc, float *__restrict__ d
     if (i < 11) dParams[i] += (float)acc[i];
 }
 
-constexpr int32_t kReplayTriangles = 8192;  // the replay's tiles gain 12 % on the corner and lose 4 % at 28,800 triangles
+// A replay writes records only to read them once, so its tiles pay in small
+// trees: lanes / tiles 12 % faster on the corner, 0.90 / 0.99, 1.02 / 1.12 and
+// 1.10 / 1.22 ms on heightfields of 2,048, 3,872 and 7,200 triangles.  With
+// the principled material's larger records: 1.27 / 1.18, 1.48 / 1.38 (7,200)
+// and 1.76 / 1.81 ms (16,200), the line of the renders.
+constexpr int32_t kReplayTriangles = 1536;
 
 inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
@@ -1210,8 +1210,15 @@ int launch_pack_tex(const float *albedo, const float *rough, int64_t ntex, float
 
 int launch_render(const RenderArgs &a, cudaStream_t st) {
     const int64_t lanes = ((int64_t)a.Hc * a.Wc) << a.log2L;
-    if (!tiled(a))
-        k_render<<<grid_for(lanes, kRenderBlock), kRenderBlock, 0, st>>>(a);
+    // Resident blocks per SM of the lanes kernel.  10 (48 registers, with
+    // spills) hide more of a large tree's loads: 200k-triangle heightfield,
+    // 1024 x 1024 x 16 spp, at 7 / 8 / 9 / 10 / 12: 8.57 / 8.09 / 8.02 / 7.88 /
+    // 8.08 ms.  8 (64 registers) for single bounces in small scenes: the
+    // corner at 256 x 256 x 64 spp 0.331 ms with 10, 0.311 with 8.
+    if (!tiled(a) && a.T > kTileTriangles)
+        k_render<10><<<grid_for(lanes, kRenderBlock), kRenderBlock, 0, st>>>(a);
+    else if (!tiled(a))
+        k_render<8><<<grid_for(lanes, kRenderBlock), kRenderBlock, 0, st>>>(a);
     else if (small_tiles(a))
         k_render_tile<64, 64><<<grid_for(lanes, 64), 64, 0, st>>>(a);
     else
@@ -1270,7 +1277,8 @@ void launch_grad_tile(const RenderArgs &a, const LossArgs &l, void *scratch, cud
 }  // namespace
 
 size_t grad_scratch_bytes(const RenderArgs &a, bool replay, int words) {
-    return replay && a.T > kReplayTriangles ? 0 : tile_scratch_bytes(a, replay, words);
+    const int32_t most = words == kPRecWordsHost ? kTileTriangles : kReplayTriangles;
+    return replay && a.T > most ? 0 : tile_scratch_bytes(a, replay, words);
 }
 
 int launch_replay(const RenderArgs &a, double *acc, void *scratch, cudaStream_t st) {
@@ -1301,7 +1309,7 @@ int launch_render_grad(const RenderArgs &a, const LossArgs &l, void *scratch, cu
 
 int launch_render_keep(const RenderArgs &a, void *chunks, uint8_t *nvs, cudaStream_t st) {
     const int64_t threads = ((int64_t)a.Hc * a.Wc) << a.log2L;
-    if (!tiled(a) || a.root == kEmptyRoot)
+    if (!tiled_records(a) || a.root == kEmptyRoot)
         k_render_keep<<<grid_for(threads, kRenderBlock), kRenderBlock, 0, st>>>(a, (uint4 *)chunks, nvs);
     else if (small_tiles(a))
         k_keep_tile<64, 64><<<grid_for(threads, 64), 64, 0, st>>>(a, (uint4 *)chunks, nvs);

@@ -84,41 +84,6 @@ __device__ __forceinline__ int dir_bin(f3 d) {
 // ---------------------------------------------------------------------------
 // traversal
 // ---------------------------------------------------------------------------
-typedef unsigned long long u64;
-__device__ __forceinline__ u64 pk2(float a, float b) {
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void up2(u64 v, float &a, float &b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-    u64 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-// 32 bytes of a tree node (64-byte aligned) in one load
-__device__ __forceinline__ void ldg8(const float4 *p, float4 &a, float4 &b) {
-    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
-        : "l"(p));
-}
-
-// slab() of device.cuh with the two planes of an axis in one packed FMA (the
-// same roundings; a node lists them side by side)
-__device__ __forceinline__ bool slab2(u64 x, u64 y, u64 z, u64 ix, u64 iy, u64 iz, u64 ox, u64 oy, u64 oz, float err,
-                                      float tmax, float &tnear) {
-    float tx0, tx1, ty0, ty1, tz0, tz1;
-    up2(fma2(x, ix, ox), tx0, tx1);
-    up2(fma2(y, iy, oy), ty0, ty1);
-    up2(fma2(z, iz, oz), tz0, tz1);
-    const float tn = fmax3f(fminf(tx0, tx1), fminf(ty0, ty1), fmaxf(fminf(tz0, tz1), 0.0f));
-    const float tf = fmin3f(fmaxf(tx0, tx1), fmaxf(ty0, ty1), fminf(fmaxf(tz0, tz1), tmax));
-    tnear = tn;
-    return tn <= fmaf(tf, 1.0000004f, err);
-}
-
 // One step down the tree: 50 instructions against the 54 of trav_resume's
 // (a chain of nodes with one child hit each).
 __device__ __forceinline__ void tree_node(const RenderArgs &a, const Ray &ray, float ht, int &node, int &sp, int *stack,
@@ -576,17 +541,25 @@ __device__ __forceinline__ void tile_adjoint(const RenderArgs &a, Core &core, Ti
 // ---------------------------------------------------------------------------
 // dispatch
 // ---------------------------------------------------------------------------
-// Where the tiles pay (GB300, before -> lanes kernel / tiles).  Paths of one
-// bounce have nothing to compact (plane 512 x 512 at 16 spp 206 -> 206 / 230
-// us).  A tree of some MB no longer sits in the L1 that the tiles' shared
-// memory leaves: corner walls of 1,026 / 8,226 triangles 711 -> 692 / 540 and
-// 855 -> 831 / 676 us, but heightfields of 7,200 / 51,200 / 199,712 1.47 ->
-// 1.43 / 1.42, 2.00 -> 1.96 / 2.08 and 8.41 -> 8.24 / 8.61 ms.  Small images
-// want more, smaller tiles: tiles of 64 / 256 lanes take 74 / 96 us at 147 k
-// lanes, 156 / 161 us at 410 k, 206 / 195 us at 590 k.
-constexpr int32_t kTileTriangles = 16384;  // 1 MB of nodes
+// Where the tiles pay (GB300, lanes kernel / tiles).  Paths of one bounce have
+// nothing to compact (plane 512 x 512 at 16 spp 206 / 230 us).  A tree of some
+// MB no longer sits in the L1 that the tiles' shared memory leaves.  Renders:
+// corner walls of 1,026 / 8,226 triangles 692 / 540 and 831 / 676 us, but
+// heightfields (512 x 512 x 16 spp, fewer second bounces) of 2,048 / 7,200 /
+// 12,800 / 32,768 / 199,712 triangles 1.12 / 1.12, 1.38 / 1.44, 1.48 / 1.58,
+// 1.68 / 1.86 and 2.87 / 3.14 ms.  Kernels that keep vertex records win for
+// longer, since a tile writes them once: one-trace step 1.74 / 1.51, 2.02 /
+// 1.75, 2.18 / 1.95 (16,200), 2.31 / 2.13, 2.54 / 2.45 (64,800) and 3.52 /
+// 3.52 ms; kept records 1.39 / 1.21, 1.66 / 1.53, 1.82 / 1.76, 1.97 / 1.95,
+// 2.30 / 2.28 and 3.25 / 3.35 ms.  Small images want more, smaller tiles:
+// tiles of 64 / 256 lanes take 74 / 96 us at 147 k lanes, 156 / 161 us at
+// 410 k, 206 / 195 us at 590 k.
+constexpr int32_t kTileTriangles = 10240;
+constexpr int32_t kRecordTriangles = 65536;
 constexpr int64_t kTileLanes = 500000;
 __host__ __device__ __forceinline__ bool tiled(const RenderArgs &a) { return a.bounces > 1 && a.T <= kTileTriangles; }
+// kernels that record every vertex
+inline bool tiled_records(const RenderArgs &a) { return a.bounces > 1 && a.T <= kRecordTriangles; }
 // blocks of b threads that the GPU holds at once: the persistent grid
 inline int resident_blocks(int b) {
     int dev = 0, sms = 0;
@@ -606,7 +579,7 @@ inline size_t tile_block_bytes(const RenderArgs &a, bool replay, int S, int word
 }
 
 inline size_t tile_scratch_bytes(const RenderArgs &a, bool replay, int words) {
-    if (!tiled(a) || a.root == kEmptyRoot) return 0;
+    if (!tiled_records(a) || a.root == kEmptyRoot) return 0;
     return small_tiles(a) ? (size_t)resident_blocks(64) * tile_block_bytes(a, replay, 64, words)
                           : (size_t)resident_blocks(128) * tile_block_bytes(a, replay, 256, words);
 }
