@@ -582,6 +582,18 @@ __device__ __forceinline__ void trav_begin(Trav &st, int32_t root, float tmax, b
     st.h.t = tmax;
 }
 
+// kPacked: a node in two loads, its slabs in packed FMAs (the same results):
+// 200k-triangle heightfield, 1024 x 1024 x 16 spp, 8.24 -> 8.09 ms.  Not in
+// the server's batch kernel, whose single-bounce requests share it with the
+// tiles: 11.61 ms packed, 11.37 plain (16 mixed requests); nor where the
+// compiler chooses the fusions, which it would choose anew, nor in the
+// wavefront passes (not measured).
+#ifdef DPCS_FUSION_BY_COMPILER
+constexpr bool kPackedSlabs = false;
+#else
+constexpr bool kPackedSlabs = true;
+#endif
+template <bool kPacked = kPackedSlabs>
 __device__ __forceinline__ bool trav_resume(const float4 *__restrict__ nodes, const float4 *__restrict__ tris,
                                             int32_t root, int32_t T, const Ray &ray, Trav &st, int *stack,
                                             unsigned *status, Cnt &cnt, int min_active, int cap_override = 0) {
@@ -612,25 +624,24 @@ __device__ __forceinline__ bool trav_resume(const float4 *__restrict__ nodes, co
             cnt.add(kCntNode);
             float4 n0, n1, n2, n3;
             float tl, tr;
-#ifdef DPCS_FUSION_BY_COMPILER
-            n0 = __ldg(nodes + 4 * node + 0);
-            n1 = __ldg(nodes + 4 * node + 1);
-            n2 = __ldg(nodes + 4 * node + 2);
-            n3 = __ldg(nodes + 4 * node + 3);
-            const bool hl = slab(ray, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, st.h.t, tl);
-            const bool hr = slab(ray, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, st.h.t, tr);
-#else
-            // two loads a node and packed slabs: 200k-triangle heightfield,
-            // 1024 x 1024 x 16 spp, 8.24 -> 8.09 ms
-            const float4 *nd = nodes + 4 * (size_t)(uint32_t)node;
-            ldg8(nd, n0, n1);
-            ldg8(nd + 2, n2, n3);
-            const u64 ix = pk2(ray.inv.x, ray.inv.x), iy = pk2(ray.inv.y, ray.inv.y), iz = pk2(ray.inv.z, ray.inv.z);
-            const u64 ox = pk2(-ray.oinv.x, -ray.oinv.x), oy = pk2(-ray.oinv.y, -ray.oinv.y),
-                      oz = pk2(-ray.oinv.z, -ray.oinv.z);
-            const bool hl = slab2(pk2(n0.x, n0.y), pk2(n0.z, n0.w), pk2(n2.x, n2.y), ix, iy, iz, ox, oy, oz, ray.err, st.h.t, tl);
-            const bool hr = slab2(pk2(n1.x, n1.y), pk2(n1.z, n1.w), pk2(n2.z, n2.w), ix, iy, iz, ox, oy, oz, ray.err, st.h.t, tr);
-#endif
+            bool hl, hr;
+            if constexpr (kPacked) {
+                const float4 *nd = nodes + 4 * (size_t)(uint32_t)node;
+                ldg8(nd, n0, n1);
+                ldg8(nd + 2, n2, n3);
+                const u64 ix = pk2(ray.inv.x, ray.inv.x), iy = pk2(ray.inv.y, ray.inv.y), iz = pk2(ray.inv.z, ray.inv.z);
+                const u64 ox = pk2(-ray.oinv.x, -ray.oinv.x), oy = pk2(-ray.oinv.y, -ray.oinv.y),
+                          oz = pk2(-ray.oinv.z, -ray.oinv.z);
+                hl = slab2(pk2(n0.x, n0.y), pk2(n0.z, n0.w), pk2(n2.x, n2.y), ix, iy, iz, ox, oy, oz, ray.err, st.h.t, tl);
+                hr = slab2(pk2(n1.x, n1.y), pk2(n1.z, n1.w), pk2(n2.z, n2.w), ix, iy, iz, ox, oy, oz, ray.err, st.h.t, tr);
+            } else {
+                n0 = __ldg(nodes + 4 * node + 0);
+                n1 = __ldg(nodes + 4 * node + 1);
+                n2 = __ldg(nodes + 4 * node + 2);
+                n3 = __ldg(nodes + 4 * node + 3);
+                hl = slab(ray, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, st.h.t, tl);
+                hr = slab(ray, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, st.h.t, tr);
+            }
             const int cl = __float_as_int(n3.x), cr = __float_as_int(n3.y);
             if (hl && hr) {
                 if (st.sp >= kStack) {

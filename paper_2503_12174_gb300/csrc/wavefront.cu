@@ -68,7 +68,7 @@ __device__ __forceinline__ bool trace_one(const RenderArgs &a, const Ray &ray, f
     Trav st;
     int stack[kStack];
     trav_begin(st, a.root, tmax, any);
-    trav_resume(a.nodes, a.tris, a.root, a.T, ray, st, stack, a.status, cnt, 0, a.visit_cap);
+    trav_resume<false>(a.nodes, a.tris, a.root, a.T, ray, st, stack, a.status, cnt, 0, a.visit_cap);
     h = st.h;
     return h.pos >= 0;
 }
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kWfBlock, DPCS_WF_TRACE_MINB) k_wf_trace_refil
         if (!__any_sync(0xffffffffu, has)) break;
         if (has) {
             const int alive = __popc(__activemask());
-            if (trav_resume(a.nodes, a.tris, a.root, a.T, ray, st, stack, a.status, cnt, min(DPCS_WF_REFILL, alive),
+            if (trav_resume<false>(a.nodes, a.tris, a.root, a.T, ray, st, stack, a.status, cnt, min(DPCS_WF_REFILL, alive),
                             a.visit_cap)) {
                 w.hit[c] = make_float4(__int_as_float(st.h.pos), st.h.u, st.h.v, 0.f);
                 has = false;
