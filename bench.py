@@ -52,26 +52,27 @@ FWD_BWD_WORKLOAD = "corner scene T=1026 at 512x512 (camera, projector, textures)
                    "and the 11 PRF/CRF/white-balance parameters + Adam on Ip"
 L2_FLUSH_BYTES = 256 << 20
 
-# DRAM bytes (read + write) of one k_render launch of this workload, from an
+# DRAM bytes (read + write) of one k_render_tile launch of this workload, from an
 # ncu capture of the same command.  It holds only for the kernel sources it
 # was measured on; once they change, the roofline's traffic is reported as
 # null until a new capture is taken.
-RENDER_TRAFFIC = {"bytes": 20629504, "sources_sha256": "508f75db6f855332a222fba620eb55bc1b90fe365e09b9af620bbc64d8698124"}
-# Warp instructions one k_render launch of the forward workload issues, and
+RENDER_TRAFFIC = {"bytes": 12837888, "sources_sha256": "f56d3aaeccd4791c6a6d2ed6e8a153af4e7a39b8b60a3bed4b7664d4b0a89273"}
+# Warp instructions one k_render_tile launch of the forward workload issues, and
 # the active lanes per instruction, from the same ncu capture
 # (smsp__inst_executed.sum, smsp__thread_inst_executed_per_inst_executed);
 # reported while the kernel sources keep this hash.
-RENDER_ISSUE = {"warp_instructions": 1192796769, "lanes_per_instruction": 13.54,
-                "sources_sha256": "508f75db6f855332a222fba620eb55bc1b90fe365e09b9af620bbc64d8698124"}
-# The same two figures for one k_render_grad launch of the compensation step
+RENDER_ISSUE = {"warp_instructions": 813127652, "lanes_per_instruction": 21.23,
+                "sources_sha256": "f56d3aaeccd4791c6a6d2ed6e8a153af4e7a39b8b60a3bed4b7664d4b0a89273"}
+# The same two figures for one k_grad_tile launch of the compensation step
 # with every gradient requested.
-FWD_BWD_TRAFFIC = {"bytes": 1898995712,
-                   "sources_sha256": "508f75db6f855332a222fba620eb55bc1b90fe365e09b9af620bbc64d8698124"}
-FWD_BWD_ISSUE = {"warp_instructions": 1407314884, "lanes_per_instruction": 15.14,
-                 "sources_sha256": "508f75db6f855332a222fba620eb55bc1b90fe365e09b9af620bbc64d8698124"}
+FWD_BWD_TRAFFIC = {"bytes": 1418324480,
+                   "sources_sha256": "f56d3aaeccd4791c6a6d2ed6e8a153af4e7a39b8b60a3bed4b7664d4b0a89273"}
+FWD_BWD_ISSUE = {"warp_instructions": 1046747543, "lanes_per_instruction": 21.94,
+                 "sources_sha256": "f56d3aaeccd4791c6a6d2ed6e8a153af4e7a39b8b60a3bed4b7664d4b0a89273"}
 # the kernels' sources and the tree builder (its topology sets the node visits)
-KERNEL_SOURCES = ("paper_2503_12174_gb300/csrc/render.cu", "paper_2503_12174_gb300/csrc/device.cuh",
-                  "paper_2503_12174_gb300/csrc/internal.h", "paper_2503_12174_gb300/csrc/lbvh.cu")
+KERNEL_SOURCES = ("paper_2503_12174_gb300/csrc/render.cu", "paper_2503_12174_gb300/csrc/tile.cuh",
+                  "paper_2503_12174_gb300/csrc/device.cuh", "paper_2503_12174_gb300/csrc/internal.h",
+                  "paper_2503_12174_gb300/csrc/lbvh.cu")
 
 
 def kernel_sources_sha256() -> str:
@@ -582,7 +583,7 @@ def main():
     if flops:
         lbytes = sum(LOAD_BYTES[k] * counts[k] for k in LOAD_BYTES)
         l_tbs = lbytes / (kernel_ms / 1e3) / 1e12
-        roof_load = {"bound": "l2", "kernel": "k_render", "achieved": l_tbs, "peak": l2_gbs / 1e3, "unit": "TB/s",
+        roof_load = {"bound": "l2", "kernel": "k_render_tile", "achieved": l_tbs, "peak": l2_gbs / 1e3, "unit": "TB/s",
                      "frac": l_tbs / (l2_gbs / 1e3), "bytes_per_launch": lbytes,
                      "peak_basis": f"measured: dpcs_probe_l2_load (measurement library), {PROBE_L2_BYTES >> 20} MiB read with 16 B "
                                    "L2-only loads, best of 3",
@@ -590,7 +591,7 @@ def main():
     if replay_counts and replay_ms:
         n_atom = 4 * (replay_counts["vertices"] + replay_counts["lit"])
         r_ms = replay_ms
-        roof_atomic = {"bound": "atomic", "kernel": "k_replay", "achieved": n_atom / (r_ms / 1e3) / 1e9,
+        roof_atomic = {"bound": "atomic", "kernel": "k_grad_tile (replay)", "achieved": n_atom / (r_ms / 1e3) / 1e9,
                        "peak": atomic_g, "unit": "Gatomics/s", "frac": n_atom / (r_ms / 1e3) / 1e9 / atomic_g,
                        "atomics_per_launch": n_atom, "kernel_ms": r_ms,
                        "peak_basis": f"measured: dpcs_probe_atomic4, float4 adds at random texels of a "
@@ -603,7 +604,7 @@ def main():
             simt["traversal"] = (counts["node_visits"] + counts["tri_tests"]) / (32.0 * counts["trav_warp_iters"])
         if counts.get("path_warp_iters"):
             simt["path_loop"] = (counts["rays"] + counts["shadow_rays"]) / (32.0 * counts["path_warp_iters"])
-        roof = {"bound": "alu", "kernel": "k_render", "achieved": achieved, "peak": peak_tflops,
+        roof = {"bound": "alu", "kernel": "k_render_tile", "achieved": achieved, "peak": peak_tflops,
                 "unit": "TFLOP/s", "frac": achieved / peak_tflops, "traffic": traffic,
                 "flops_per_launch": flops, "kernel_ms": kernel_ms,
                 "peak_basis": f"{sms} SMs x 128 FP32 lanes x 2 FLOP/FMA x {sm_max_mhz:.0f} MHz (max SM clock)",
@@ -613,7 +614,7 @@ def main():
         fb_flops = sum(FLOP[k] * grad_counts[k] for k in FLOP) + SWEEP_FLOP_PER_VERTEX * grad_counts["vertices"]
         ach = fb_flops / (fused_ms / 1e3) / 1e12
         n_atom = 4 * (grad_counts["vertices"] + grad_counts["lit"])
-        roof_fb = {"bound": "alu", "kernel": "k_render_grad", "achieved": ach, "peak": peak_tflops, "unit": "TFLOP/s",
+        roof_fb = {"bound": "alu", "kernel": "k_grad_tile", "achieved": ach, "peak": peak_tflops, "unit": "TFLOP/s",
                    "frac": ach / peak_tflops, "flops_per_launch": fb_flops, "kernel_ms": fused_ms,
                    "float4_atomics_per_launch": n_atom,
                    "atomic_rate_g_per_s": n_atom / (fused_ms / 1e3) / 1e9, "atomic_peak_g_per_s": atomic_g,
@@ -634,7 +635,7 @@ def main():
         inst = RENDER_ISSUE["warp_instructions"]
         issue_peak = 4 * sms * sm_max_mhz * 1e6 / 1e9
         issue = inst / (kernel_ms / 1e3) / 1e9
-        roof_issue = {"bound": "issue", "kernel": "k_render", "achieved": issue, "peak": issue_peak,
+        roof_issue = {"bound": "issue", "kernel": "k_render_tile", "achieved": issue, "peak": issue_peak,
                       "unit": "G warp-instructions/s", "frac": issue / issue_peak, "kernel_ms": kernel_ms,
                       "warp_instructions_per_launch": inst,
                       "lanes_per_instruction": RENDER_ISSUE["lanes_per_instruction"],

@@ -97,7 +97,10 @@ typedef struct dpcs_view {
 } dpcs_view;
 
 /* Create a context on CUDA device `device`; scratch and scenes may use at
- * most `hbm_budget_bytes` (0 = no limit).  *out receives the context. */
+ * most `hbm_budget_bytes` (0 = no limit).  Without a limit the adjoint calls
+ * also take scratch for path records (up to 1 GB) where it is to be
+ * had; with one they do without, to the same results.  *out receives the
+ * context. */
 dpcs_status dpcs_create(int device, size_t hbm_budget_bytes, dpcs_ctx **out);
 
 /* Free every scene, scratch buffer and the context itself (synchronises). */
@@ -118,8 +121,9 @@ uint64_t dpcs_launch_count(const dpcs_ctx *ctx);
 
 /*
  * Kernel timing with CUDA events recorded on the launching stream around the
- * path-tracing kernels: kernel 0 = forward render (k_render), 1 = path replay
- * (k_replay), 2 = the pose-gradient kernels (dpcs_pose_backward).
+ * path-tracing kernels: kernel 0 = forward render (k_render, k_render_tile and
+ * the steps that render), 1 = path replay (k_replay, k_grad_tile), 2 = the
+ * pose-gradient kernels (dpcs_pose_backward).
  * dpcs_timing_enable(ctx, 1) clears and starts recording, (ctx, 0) stops it.
  * dpcs_timing_read waits for the recorded events and returns the summed
  * duration in milliseconds and the number of launches.
