@@ -19,6 +19,8 @@ def _scene(mesh, H, W, spp, bounces):
         sc = scenes.corner(res=32, tex=24, spp=spp, bounces=bounces, seed=5)
     elif mesh == "sphere":
         sc = scenes.sphere(subdiv=2, spp=spp, bounces=bounces, seed=5)
+    elif mesh == "field":  # 20,000 triangles: past the renders' limit, within the record kernels
+        sc = scenes.heightfield(spp=spp, cam=32, proj=(40, 56), tex=32, n_vert=101).replace(bounces=bounces)
     else:  # a single triangle: the tree has no inner node
         sc = scenes.plane(res=32, spp=spp, seed=5)
         sc = sc.replace(tris=sc.tris[:1], bounces=bounces)
@@ -53,7 +55,8 @@ def test_tiles_render_what_lanes_render(mesh, H, W, spp, bounces):
 
 @pytest.mark.parametrize("mesh,H,W,spp,bounces", [
     ("corner", 1, 1, 1, 2), ("corner", 1, 3, 7, 3), ("corner", 17, 31, 35, 3), ("corner", 9, 57, 100, 3),
-    ("corner", 125, 125, 33, 3), ("corner", 12, 11, 300, 3), ("sphere", 24, 24, 16, 8), ("triangle", 20, 20, 8, 3)])
+    ("corner", 125, 125, 33, 3), ("corner", 12, 11, 300, 3), ("sphere", 24, 24, 16, 8), ("triangle", 20, 20, 8, 3),
+    ("field", 31, 29, 8, 4)])
 def test_tile_gradients_equal_lane_gradients(mesh, H, W, spp, bounces):
     """A context with a memory budget gets no scratch for the tiles' records
     and runs the lanes kernels: the same paths, so the image is equal bit for
@@ -97,7 +100,7 @@ def test_tile_gradients_equal_lane_gradients(mesh, H, W, spp, bounces):
 @pytest.mark.parametrize("mesh,H,W,spp,bounces,maps", [
     ("corner", 1, 3, 7, 3, "both"), ("corner", 17, 31, 35, 3, "both"), ("corner", 9, 57, 100, 2, "metallic"),
     ("corner", 125, 125, 33, 3, "both"), ("corner", 12, 11, 300, 3, "normal"), ("sphere", 24, 24, 16, 8, "both"),
-    ("triangle", 20, 20, 8, 3, "both")])
+    ("triangle", 20, 20, 8, 3, "both"), ("field", 31, 29, 8, 4, "both")])
 def test_principled_tiles_equal_lanes(mesh, H, W, spp, bounces, maps):
     """As above with the principled material, whose render and kept records
     run in tiles with or without a budget: one-trace step, separate calls and
