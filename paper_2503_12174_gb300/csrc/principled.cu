@@ -515,6 +515,7 @@ __global__ void __launch_bounds__(kPBlock) k_sweep_kept_pbr(const RenderArgs a, 
 //   replay              0.420 -> 0.375    0.714 -> 0.551    2.77 -> 2.00
 // ---------------------------------------------------------------------------
 struct PbrCore {
+    static constexpr bool kUnrolled = true;  // tree_walk
     const float4 *mat;
     __device__ __forceinline__ bool begin(const RenderArgs &, int, uint32_t, int) { return true; }
     __device__ __forceinline__ void dark(const RenderArgs &, int, int, int) {}
@@ -541,6 +542,7 @@ struct PbrCore {
 // every vertex recorded: the PRec fields, as 13 chunks laid out like RecordCore's
 template <bool kStream>
 struct PbrRecordCore {
+    static constexpr bool kUnrolled = false;
     const float4 *mat;
     uint4 *chunks;
     uint8_t *nvs;

@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_BATCH_MINB)
         }
         __syncthreads();
         const int64_t lane0 = (vb - sg.vb_begin) * kBatchLanes;  // first lane of the block within the segment
-        if (tiled(sa)) {
+        if (tiled_paths(sa)) {
             PlainCore core;
             tile_image<kRenderBlock, kBatchLanes>(sa, core, P, sg.pix_begin, lane0, sg.npix << sa.log2L);
         } else {
@@ -963,6 +963,7 @@ __global__ void __launch_bounds__(kRenderBlock) k_sweep_kept(const RenderArgs a,
 // bounces, nthr, t0 + slot).
 template <bool kStream>
 struct RecordCore {
+    static constexpr bool kUnrolled = false;  // tree_walk
     uint4 *chunks;
     uint8_t *nvs;  // vertices of each recorded path, [spl][nthr]
     int64_t nthr, t0;
@@ -1173,11 +1174,21 @@ __global__ void k_finalize(const double *__restrict__ acc, float *__restrict__ d
 }
 
 // A replay writes records only to read them once, so its tiles pay in small
-// trees: lanes / tiles 12 % faster on the corner, 0.90 / 0.99, 1.02 / 1.12 and
-// 1.10 / 1.22 ms on heightfields of 2,048, 3,872 and 7,200 triangles.  With
-// the principled material's larger records: 1.27 / 1.18, 1.48 / 1.38 (7,200)
-// and 1.76 / 1.81 ms (16,200), the line of the renders.
+// trees where two things of three hold: paths of three bounces or more, 1 M
+// lanes, samples that do not fill their rounds.  In parts of the lanes kernel's
+// time before there were tiles (that kernel now 0.88 to 0.95): corner, 4
+// bounces, at 0.6 / 1 / 2.4 / 4.2 M lanes 0.95 / 0.86 / 0.81 / 0.80, with 2 bounces
+// 1.10 / 0.98 / 0.87 / 0.83, with 4 bounces and unfilled rounds 0.85 at 8 k, 0.76
+// at 100 k, 0.76 at 0.8 M; a heightfield of 512 triangles, 4 bounces, 0.99 to
+// 0.95 from 1 M on, 1.05 to 1.02 with 2, 0.93 to 0.86 with unfilled rounds; of
+// 2,048 triangles 1.02 to 0.98, 1.09 to 1.03.  With the principled material's
+// larger records tiles take 0.70 to 0.90 (lanes 0.84 to 0.98) up to the line of
+// the renders.
 constexpr int32_t kReplayTriangles = 1536;
+inline bool tiled_replay(const RenderArgs &a) {
+    return a.T <= kReplayTriangles && a.bounces > 1 &&
+           (a.bounces > 2) + (path_lanes(a) >= 2 * kTileLanes) + !full_rounds(a) >= 2;
+}
 
 inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
@@ -1214,9 +1225,10 @@ int launch_render(const RenderArgs &a, cudaStream_t st) {
     // Resident blocks per SM of the lanes kernel.  10 (48 registers, with
     // spills) hide more of a large tree's loads: 200k-triangle heightfield,
     // 1024 x 1024 x 16 spp, at 7 / 8 / 9 / 10 / 12: 8.57 / 8.09 / 8.02 / 7.88 /
-    // 8.08 ms.  8 (64 registers) for single bounces in small scenes: the
-    // corner at 256 x 256 x 64 spp 0.331 ms with 10, 0.311 with 8.
-    if (!tiled(a) && a.T > kTileTriangles)
+    // 8.08 ms.  8 (64 registers) for single bounces (that heightfield at 512 x
+    // 512 x 8 spp 0.768 ms with 10, 0.703 with 8; the corner at 256 x 256 x 64
+    // spp 0.331 and 0.311) and in small scenes.
+    if (!tiled(a) && a.T > kTileTriangles && a.bounces > 1)
         k_render<10><<<grid_for(lanes, kRenderBlock), kRenderBlock, 0, st>>>(a);
     else if (!tiled(a))
         k_render<8><<<grid_for(lanes, kRenderBlock), kRenderBlock, 0, st>>>(a);
@@ -1278,8 +1290,8 @@ void launch_grad_tile(const RenderArgs &a, const LossArgs &l, void *scratch, cud
 }  // namespace
 
 size_t grad_scratch_bytes(const RenderArgs &a, bool replay, int words) {
-    const int32_t most = words == kPRecWordsHost ? kTileTriangles : kReplayTriangles;
-    return replay && a.T > most ? 0 : tile_scratch_bytes(a, replay, words);
+    if (replay && (words == kPRecWordsHost ? a.T > kTileTriangles : !tiled_replay(a))) return 0;
+    return tile_scratch_bytes(a, replay, words);
 }
 
 int launch_replay(const RenderArgs &a, double *acc, void *scratch, cudaStream_t st) {

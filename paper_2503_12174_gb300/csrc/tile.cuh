@@ -116,19 +116,35 @@ __device__ __forceinline__ void tree_node(const RenderArgs &a, const Ray &ray, f
 
 // Closest hit (any = false; ht = infinity at the start) or any hit before ht,
 // from node = a.root; lanes with node = kDone only take part in the warp's
-// votes.  hpos < 0: nothing hit.  As in trav_resume every step, node or leaf,
-// counts towards the visit cap: a ray that would take one more reports it and
-// ends as a miss, so a walk ends whatever the tree holds.  The loop's one
-// comparison tests the node, the cap and the stack together, which costs renders
-// and steps 0.6 to 0.9 % (corner 256 x 256 at 64 spp 1.051 -> 1.058 ms, a
-// principled step of 256 x 256 628.7 -> 634.7 us); tested one by one, 1.3 to 2.4 %.
+// votes.  hpos < 0: nothing hit.
+//
+// A lane takes up to kBurst steps down the tree, then the warp meets and the
+// lanes at a leaf test it.  Without the limit all lanes wait for the one that
+// is longest on its way to a leaf, which curved surfaces, whose boxes overlap,
+// make long: a closed sphere of 1,280 triangles (384 x 384 x 16 spp, 4 bounces)
+// took 3.90 ms against 3.14 of the lanes kernel of its day and takes 3.05, an
+// open half sphere 0.97 -> 0.79 of that kernel's time.  Bursts of 1 / 2 / 3 / 4 /
+// 6: 1.09 / 0.98 / 0.97 / 0.97 / 0.99 of it on the sphere, 0.82 / 0.77 / 0.76 /
+// 0.75 / 0.75 on the corner, which gains nothing from them.  Unrolled, renders
+// are another 2 to 4 % faster and the kernels with a sweep 2 to 5 % slower.
+//
+// As in trav_resume every step, node or leaf, counts towards the visit cap: a
+// ray that would take one more reports it and ends as a miss, so a walk ends
+// whatever the tree holds.  The inner loop's one comparison tests the node, the
+// burst (which the cap cuts) and the stack together; tested one by one they
+// cost 1.3 to 2.4 % more.
+constexpr int kBurst = 4;
+template <bool kUnrolled>
 __device__ __forceinline__ void tree_walk(const RenderArgs &a, const Ray &ray, bool any, int node, int &hpos, float &ht,
                                           float &hu, float &hv, Cnt &cnt) {
     int stack[kStack + 1];
     int room = kStack, left = (a.visit_cap > 0 ? a.visit_cap : 2 * a.T + 16) - 1;  // steps after the next one
     while (true) {
-        while ((node | left | room) >= 0) {
-            --left;
+        const int most = min(kBurst - 1, left);
+        int go = most;
+#pragma unroll (kUnrolled ? kBurst : 1)
+        while ((node | go | room) >= 0) {
+            --go;
 #ifdef DPCS_CHECK
             if (node >= a.T - 1) {
                 atomicOr(a.status, kStatusBoundsCheck);
@@ -140,19 +156,20 @@ __device__ __forceinline__ void tree_walk(const RenderArgs &a, const Ray &ray, b
             tree_node(a, ray, ht, node, room, stack, cnt);
         }
         __syncwarp();
+        left -= most - go;
         if (node != kDone && (left | room) < 0) {
             atomicOr(a.status, kStatusTraversalLimit);
             hpos = -1;
             node = kDone;
         }
 #ifdef DPCS_CHECK
-        if (node != kDone && ~node >= a.T) {
+        if (node < 0 && node != kDone && ~node >= a.T) {
             atomicOr(a.status, kStatusBoundsCheck);
             hpos = -1;
             node = kDone;
         }
 #endif
-        if (node != kDone) {
+        if (node < 0 && node != kDone) {
             --left;
             cnt.add_warp(kCntTravWarpIter);
             cnt.add(kCntTri);
@@ -224,7 +241,7 @@ __device__ __forceinline__ void tile_trace(const RenderArgs &a, Core &core, Tile
         }
         cnt.add_warp(kCntPathWarpIter);
         __syncwarp();
-        tree_walk(a, ray, any, node, hpos, ht, hu, hv, cnt);
+        tree_walk<Core::kUnrolled>(a, ray, any, node, hpos, ht, hu, hv, cnt);
         if (any) {
             if (on) {
                 if (hpos < 0) {
@@ -364,6 +381,7 @@ __device__ __forceinline__ f3 tile_pixel_sum(const Tile<S> &P, int slot, int L) 
 
 // the Lambert + GGX material, nothing recorded
 struct PlainCore {
+    static constexpr bool kUnrolled = true;  // tree_walk
     __device__ __forceinline__ bool begin(const RenderArgs &, int, uint32_t, int) { return true; }
     __device__ __forceinline__ void dark(const RenderArgs &, int, int, int) {}
     __device__ __forceinline__ void shade(const RenderArgs &a, int, uint32_t pix, uint32_t s, int, int b, const Hit &h,
@@ -548,25 +566,50 @@ __device__ __forceinline__ void tile_adjoint(const RenderArgs &a, Core &core, Ti
 // ---------------------------------------------------------------------------
 // dispatch
 // ---------------------------------------------------------------------------
-// Where the tiles pay (GB300, lanes kernel / tiles).  Paths of one bounce have
-// nothing to compact (plane 512 x 512 at 16 spp 206 / 230 us).  A tree of some
-// MB no longer sits in the L1 that the tiles' shared memory leaves.  Renders:
-// corner walls of 1,026 / 8,226 triangles 692 / 540 and 831 / 676 us, but
-// heightfields (512 x 512 x 16 spp, fewer second bounces) of 2,048 / 7,200 /
-// 12,800 / 32,768 / 199,712 triangles 1.12 / 1.12, 1.38 / 1.44, 1.48 / 1.58,
-// 1.68 / 1.86 and 2.87 / 3.14 ms.  Kernels that keep vertex records win for
-// longer, since a tile writes them once: one-trace step 1.74 / 1.51, 2.02 /
-// 1.75, 2.18 / 1.95 (16,200), 2.31 / 2.13, 2.54 / 2.45 (64,800) and 3.52 /
-// 3.52 ms; kept records 1.39 / 1.21, 1.66 / 1.53, 1.82 / 1.76, 1.97 / 1.95,
-// 2.30 / 2.28 and 3.25 / 3.35 ms.  Small images want more, smaller tiles:
-// tiles of 64 / 256 lanes take 74 / 96 us at 147 k lanes, 156 / 161 us at
-// 410 k, 206 / 195 us at 590 k.
+// Where the tiles pay (GB300; in parts of the time that the lanes kernels took
+// before there were tiles, which their packed form takes 0.87 to 0.97 of).
+//
+// Paths of one bounce have nothing to compact (plane 512 x 512 at 16 spp 206 /
+// 230 us).  With two there is little, and images of 0.5 to 2 M lanes, whose last
+// wave of large tiles is long, take 0.94 to 1.06 (corner, heightfields, rooms,
+// spheres) where every round of samples is full: lanes there.  (Samples that
+// leave part of the last round's lanes idle cost tiles nothing: 0.77 of the
+// corner with 11 samples on 8 lanes, 1.3 M.)  Longer paths, 2.4 M lanes, 4 bounces: corner walls of
+// 1,026 / 8,226 triangles 0.74 / 0.76, a room of 2,352 / 8,112 0.92 / 0.89, a half
+// sphere 0.80, closed spheres of 1,280 / 5,120 0.97 / 0.94 (lanes 0.87 / 0.89),
+// heightfields of 2,048 / 7,200 0.93 / 0.93 (0.95 / 0.96).  A tree of some MB no
+// longer sits in the L1 that the tiles' shared memory leaves.
+//
+// Kernels that keep vertex records win for longer, since a tile writes them
+// once: one-trace steps, 2.4 M lanes, 4 bounces 0.70 (corner), 0.82 (20,000-
+// triangle heightfield, lanes 0.95), 0.98 (20,480-triangle sphere, 0.91).  Not in
+// small images, where the large trees' steps took 1.04 to 1.08.
+//
+// Small images want more, smaller tiles: tiles of 64 / 256 lanes take 0.82 /
+// 1.11 (corner), 0.88 / 1.33 (sphere), 0.94 / 1.18 (heightfield of 7,200) at
+// 147 k lanes and 0.93 / 0.81, 0.89 / 1.01, 1.03 / 0.96 at 1 M.
 constexpr int32_t kTileTriangles = 10240;
 constexpr int32_t kRecordTriangles = 65536;
 constexpr int64_t kTileLanes = 500000;
-__host__ __device__ __forceinline__ bool tiled(const RenderArgs &a) { return a.bounces > 1 && a.T <= kTileTriangles; }
+__host__ __device__ __forceinline__ int64_t path_lanes(const RenderArgs &a) { return ((int64_t)a.Hc * a.Wc) << a.log2L; }
+// the scenes and path lengths that pay (the server's batch kernel, whose grid stays full)
+__host__ __device__ __forceinline__ bool tiled_paths(const RenderArgs &a) { return a.bounces > 1 && a.T <= kTileTriangles; }
+// do these arguments run in the small tiles?
+inline bool small_tiles(const RenderArgs &a) { return path_lanes(a) < kTileLanes; }
+// do the samples fill the rounds of a pixel's lanes (35 samples on 32 lanes do not)?
+inline bool full_rounds(const RenderArgs &a) {
+    const int64_t L = int64_t(1) << a.log2L;
+    return 10 * (int64_t)a.spp >= 9 * ((a.spp + L - 1) / L) * L;
+}
+// renders
+inline bool tiled(const RenderArgs &a) {
+    const bool middle = path_lanes(a) >= kTileLanes && path_lanes(a) < 4 * kTileLanes;
+    return tiled_paths(a) && !(a.bounces == 2 && middle && full_rounds(a));
+}
 // kernels that record every vertex
-inline bool tiled_records(const RenderArgs &a) { return a.bounces > 1 && a.T <= kRecordTriangles; }
+inline bool tiled_records(const RenderArgs &a) {
+    return a.bounces > 1 && a.T <= (small_tiles(a) ? kTileTriangles : kRecordTriangles);
+}
 // blocks of b threads that the GPU holds at once: the persistent grid
 inline int resident_blocks(int b) {
     int dev = 0, sms = 0;
@@ -574,9 +617,6 @@ inline int resident_blocks(int b) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return sms * (1024 / b);
 }
-
-// do these arguments run in the small tiles?
-inline bool small_tiles(const RenderArgs &a) { return (((int64_t)a.Hc * a.Wc) << a.log2L) < kTileLanes; }
 
 // one block's records: S slots of `words` 32-bit words a vertex
 inline size_t tile_block_bytes(const RenderArgs &a, bool replay, int S, int words) {
