@@ -167,9 +167,13 @@ int launch_render(const RenderArgs &a, cudaStream_t st);
 size_t wavefront_scratch_bytes(const RenderArgs &a, int64_t chunk);
 int launch_render_wavefront(const RenderArgs &a, int64_t chunk, void *scratch, cudaStream_t st);
 int launch_render_batch(const RenderArgs *descs, const BatchSeg *segs, int nseg, int64_t total_vb,
-                        unsigned long long *counter, int grid, cudaStream_t st);
-int render_batch_grid(int device);
-int64_t render_batch_vblocks(int64_t npix, int log2L);
+                        unsigned long long *counter, bool tiles, int grid, cudaStream_t st);
+int render_batch_grid(int device, bool tiles);
+int64_t render_batch_vblocks(int64_t npix, int log2L, bool tiles);
+// may a batch's request run in tiles, and are these lanes, all that a launch has
+// in tiles, enough for them?
+bool render_batch_tiles(const RenderArgs &a);
+bool render_batch_fills(int64_t lanes);
 int launch_trace(const Scene &sc, const float *o, const float *d, int64_t n, float *t, int32_t *tri,
                  unsigned *status, cudaStream_t st);
 int launch_crf_backward(const float *dIc, const float *Ec, const float *Ic, int64_t npix, const float gamma_c[3],

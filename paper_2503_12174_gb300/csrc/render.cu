@@ -290,22 +290,27 @@ __global__ void __launch_bounds__(B, 1024 / B) k_render_tile(const RenderArgs a)
     tile_image<B, S>(a, core, P, 0, (int64_t)blockIdx.x * S, ((int64_t)a.Hc * a.Wc) << a.log2L);
 }
 
-// Batched persistent render: CTAs pull virtual blocks of kBatchLanes lanes from
-// a device counter; virtual block vb belongs to the segment whose range
-// [vb_begin, vb_begin + ceil(npix L / kBatchLanes)) holds it, and covers that
-// segment's pixels from pix_begin on.  A segment is a pixel range of one
-// request whose arguments are descs[slot].  Per pixel the computation is that
-// of launch_render's kernels, in tiles or in lanes by the same rule (16 mixed
-// requests 15.0 -> 11.2 ms with the tiles).  The loop ends when the counter
-// passes the last virtual block: there is no waiting on other CTAs.
+// Batched persistent render: CTAs pull virtual blocks from a device counter;
+// virtual block vb belongs to the segment whose range [vb_begin, vb_begin +
+// render_batch_vblocks) holds it, and covers that segment's pixels from
+// pix_begin on.  A segment is a pixel range of one request whose arguments are
+// descs[slot].  Per pixel the computation is that of launch_render's kernels.
+// The loop ends when the counter passes the last virtual block: there is no
+// waiting on other CTAs.
+//
+// Segments in tiles and in lanes are launches of their own: a lanes block has
+// half a tile's lanes, which a single small request needs to fill the chip, and
+// the L1 that the tiles' shared memory would take.  In one kernel of 256-lane
+// blocks a relight of 128 x 128 at 16 spp took up to 2.1 times and 512 x 512 at
+// 64 spp of a 20,000-triangle surface 1.1 to 1.2 times as long as in lanes.
 constexpr int kBatchLanes = 256;
+template <bool kTiles>
 __global__ void __launch_bounds__(kRenderBlock, DPCS_BATCH_MINB)
     k_render_batch(const RenderArgs *__restrict__ descs, const BatchSeg *__restrict__ segs, int nseg,
                    int64_t total_vb, unsigned long long *counter) {
     __shared__ RenderArgs sa;
     __shared__ int64_t s_vb;
     __shared__ int s_seg;
-    __shared__ Tile<kBatchLanes> P;
     while (true) {
         if (threadIdx.x == 0) {
             const int64_t vb = (int64_t)atomicAdd(counter, 1ull);
@@ -327,15 +332,15 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_BATCH_MINB)
             for (int i = threadIdx.x; i < (int)(sizeof(RenderArgs) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
         }
         __syncthreads();
-        const int64_t lane0 = (vb - sg.vb_begin) * kBatchLanes;  // first lane of the block within the segment
-        if (tiled_paths(sa)) {
+        if constexpr (kTiles) {
+            __shared__ Tile<kBatchLanes> P;
             PlainCore core;
-            tile_image<kRenderBlock, kBatchLanes>(sa, core, P, sg.pix_begin, lane0, sg.npix << sa.log2L);
+            tile_image<kRenderBlock, kBatchLanes>(sa, core, P, sg.pix_begin, (vb - sg.vb_begin) * kBatchLanes,
+                                                  sg.npix << sa.log2L);
         } else {
-            for (int64_t lt = lane0 + threadIdx.x; lt < lane0 + kBatchLanes; lt += kRenderBlock) {
-                const int64_t lp = lt >> sa.log2L;
-                render_lanes<false>(sa, sg.pix_begin + lp, (int)(lt & ((1 << sa.log2L) - 1)), lp < sg.npix);
-            }
+            const int64_t lt = (vb - sg.vb_begin) * kRenderBlock + threadIdx.x;  // thread index within the segment
+            const int64_t lp = lt >> sa.log2L;
+            render_lanes<true>(sa, sg.pix_begin + lp, (int)(lt & ((1 << sa.log2L) - 1)), lp < sg.npix);
         }
         __syncthreads();
     }
@@ -1240,21 +1245,31 @@ int launch_render(const RenderArgs &a, cudaStream_t st) {
 }
 
 int launch_render_batch(const RenderArgs *descs, const BatchSeg *segs, int nseg, int64_t total_vb,
-                        unsigned long long *counter, int grid, cudaStream_t st) {
-    k_render_batch<<<grid, kRenderBlock, 0, st>>>(descs, segs, nseg, total_vb, counter);
+                        unsigned long long *counter, bool tiles, int grid, cudaStream_t st) {
+    if (tiles)
+        k_render_batch<true><<<grid, kRenderBlock, 0, st>>>(descs, segs, nseg, total_vb, counter);
+    else
+        k_render_batch<false><<<grid, kRenderBlock, 0, st>>>(descs, segs, nseg, total_vb, counter);
     return 1;
 }
 
-int render_batch_grid(int device) {
+int render_batch_grid(int device, bool tiles) {
     int per_sm = 0, sms = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_batch, kRenderBlock, 0);
+    if (tiles)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_batch<true>, kRenderBlock, 0);
+    else
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_render_batch<false>, kRenderBlock, 0);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     return per_sm > 0 && sms > 0 ? per_sm * sms : 1;
 }
 
-int64_t render_batch_vblocks(int64_t npix, int log2L) {
-    return ((npix << log2L) + kBatchLanes - 1) / kBatchLanes;
+int64_t render_batch_vblocks(int64_t npix, int log2L, bool tiles) {
+    const int block = tiles ? kBatchLanes : kRenderBlock;
+    return ((npix << log2L) + block - 1) / block;
 }
+
+bool render_batch_tiles(const RenderArgs &a) { return tiled(a); }
+bool render_batch_fills(int64_t lanes) { return lanes >= kTileLanes; }
 
 int launch_trace(const Scene &sc, const float *o, const float *d, int64_t n, float *t, int32_t *tri,
                  unsigned *status, cudaStream_t st) {

@@ -89,7 +89,7 @@ struct Batch {
     cudaEvent_t ev = nullptr;
     RenderArgs *descs_host = nullptr, *descs_dev = nullptr;
     BatchSeg *segs_host = nullptr, *segs_dev = nullptr;
-    unsigned long long *counter = nullptr;
+    unsigned long long *counter = nullptr;  // of the launch in lanes and of that in tiles
     std::vector<std::pair<Req *, int64_t>> pixels;  // relighting pixels carried
     std::vector<Req *> steps;                        // compensation steps carried
 };
@@ -110,7 +110,7 @@ struct dpcs_server {
     uint64_t next_id = 1;
     size_t used = 0, high_water = 0;
     int64_t submitted = 0, completed = 0, failed = 0, iterations = 0, launches = 0;
-    int grid = 1;
+    int grid[2] = {1, 1};  // of the batch kernel in lanes and in tiles
     void *recs = nullptr;  // path records of the compensation steps' tiles (steps run one after another)
     size_t recs_bytes = 0;
     std::vector<void *> retired;  // smaller ones that queued steps may still use
@@ -354,7 +354,7 @@ void plan_fixed_share(dpcs_server *s, const std::vector<Req *> &relight, const s
                       std::vector<int64_t> &give, int64_t &budget, int64_t total_budget, Batch &b);
 void plan_by_deadline(dpcs_server *s, const std::vector<Req *> &relight, const std::vector<Req *> &comp,
                       std::vector<int64_t> &give, int64_t &budget, Batch &b);
-dpcs_status enqueue_iteration(dpcs_server *s, Batch &b, int nseg, int64_t vb);
+dpcs_status enqueue_iteration(dpcs_server *s, Batch &b, const int nseg[2], const int64_t vb[2]);
 
 dpcs_status launch_iteration(dpcs_server *s, Batch &b) {
     std::vector<Req *> comp, relight;
@@ -367,21 +367,8 @@ dpcs_status launch_iteration(dpcs_server *s, Batch &b) {
         }
     }
     if (comp.empty() && relight.empty()) return DPCS_OK;
-    int nseg = 0;
-    int64_t vb = 0;
     const int64_t total_budget = s->cfg.samples_per_iteration;
     int64_t budget = total_budget;
-    auto add_seg = [&](Req *q, int64_t pix0, int64_t npx) {
-        b.descs_host[nseg] = q->args;
-        BatchSeg &g = b.segs_host[nseg];
-        g.vb_begin = vb;
-        g.pix_begin = pix0;
-        g.npix = npx;
-        g.slot = nseg;
-        g.pad = 0;
-        vb += render_batch_vblocks(npx, q->args.log2L);
-        ++nseg;
-    };
     // `active` is in arrival order.  1) (fixed share, quanta-deadline) every
     // relighting request gets a small quantum, so short requests finish
     // within an iteration or two; under the deadline policy the deadlines
@@ -397,12 +384,25 @@ dpcs_status launch_iteration(dpcs_server *s, Batch &b) {
     } else {
         plan_fixed_share(s, relight, comp, give, budget, total_budget, b);
     }
-    for (size_t i = 0; i < relight.size(); ++i) {
-        if (give[i] <= 0) continue;
-        Req *q = relight[i];
-        add_seg(q, q->next_pix, give[i]);
-        b.pixels.push_back({q, give[i]});
-        q->next_pix += give[i];
+    // tiles where the lanes that may run in them fill the chip
+    int64_t lanes = 0;
+    for (size_t i = 0; i < relight.size(); ++i)
+        if (give[i] > 0 && render_batch_tiles(relight[i]->args)) lanes += give[i] << relight[i]->args.log2L;
+    const bool fills = render_batch_fills(lanes);
+    int nseg[2] = {0, 0};  // segments in lanes, then those in tiles
+    int64_t vb[2] = {0, 0};
+    for (int tiles = 0; tiles < 2; ++tiles) {
+        for (size_t i = 0; i < relight.size(); ++i) {
+            Req *q = relight[i];
+            if (give[i] <= 0 || (fills && render_batch_tiles(q->args)) != (tiles == 1)) continue;
+            const int n = nseg[0] + nseg[1];
+            b.descs_host[n] = q->args;
+            b.segs_host[n] = BatchSeg{vb[tiles], q->next_pix, give[i], n, 0};
+            vb[tiles] += render_batch_vblocks(give[i], q->args.log2L, tiles == 1);
+            ++nseg[tiles];
+            b.pixels.push_back({q, give[i]});
+            q->next_pix += give[i];
+        }
     }
     return enqueue_iteration(s, b, nseg, vb);
 }
@@ -498,17 +498,20 @@ void plan_by_deadline(dpcs_server *s, const std::vector<Req *> &relight, const s
     }
 }
 
-dpcs_status enqueue_iteration(dpcs_server *s, Batch &b, int nseg, int64_t vb) {
+dpcs_status enqueue_iteration(dpcs_server *s, Batch &b, const int nseg[2], const int64_t vb[2]) {
     cudaStream_t st = s->stream;
     cudaError_t e = cudaSuccess;
     int n = 0;
-    if (nseg > 0) {
-        e = cudaMemcpyAsync(b.descs_dev, b.descs_host, sizeof(RenderArgs) * nseg, cudaMemcpyHostToDevice, st);
+    if (const int all = nseg[0] + nseg[1]) {
+        e = cudaMemcpyAsync(b.descs_dev, b.descs_host, sizeof(RenderArgs) * all, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(b.segs_dev, b.segs_host, sizeof(BatchSeg) * nseg, cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(b.counter, 0, sizeof(unsigned long long), st);
+            e = cudaMemcpyAsync(b.segs_dev, b.segs_host, sizeof(BatchSeg) * all, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(b.counter, 0, 2 * sizeof(unsigned long long), st);
         if (e != cudaSuccess) return scuda(s, e, "serve: batch upload");
-        n += launch_render_batch(b.descs_dev, b.segs_dev, nseg, vb, b.counter, s->grid, st);
+        for (int tiles = 0; tiles < 2; ++tiles)
+            if (nseg[tiles])
+                n += launch_render_batch(b.descs_dev, b.segs_dev + (tiles ? nseg[0] : 0), nseg[tiles], vb[tiles],
+                                         b.counter + tiles, tiles == 1, s->grid[tiles], st);
     }
     for (Req *q : b.steps) {
         // a fresh Philox key per step (step k uses seed + k); a whole image is
@@ -593,7 +596,7 @@ dpcs_status dpcs_serve_create(dpcs_ctx *ctx, const dpcs_serve_config *cfg, dpcs_
         if (e == cudaSuccess) e = cudaMallocHost((void **)&b.segs_host, sizeof(BatchSeg) * cfg->max_active);
         if (e == cudaSuccess) e = cudaMalloc((void **)&b.descs_dev, sizeof(RenderArgs) * cfg->max_active);
         if (e == cudaSuccess) e = cudaMalloc((void **)&b.segs_dev, sizeof(BatchSeg) * cfg->max_active);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&b.counter, sizeof(unsigned long long));
+        if (e == cudaSuccess) e = cudaMalloc((void **)&b.counter, 2 * sizeof(unsigned long long));
     }
     if (e != cudaSuccess) {
         dpcs_status st = ctx_fail(ctx, DPCS_ERR_CUDA, "serve: create failed");
@@ -603,7 +606,7 @@ dpcs_status dpcs_serve_create(dpcs_ctx *ctx, const dpcs_serve_config *cfg, dpcs_
         delete s;
         return st;
     }
-    s->grid = render_batch_grid(s->device);
+    for (int tiles = 0; tiles < 2; ++tiles) s->grid[tiles] = render_batch_grid(s->device, tiles == 1);
     *out = s;
     return DPCS_OK;
 }

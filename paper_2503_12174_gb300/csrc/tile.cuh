@@ -591,9 +591,7 @@ __device__ __forceinline__ void tile_adjoint(const RenderArgs &a, Core &core, Ti
 constexpr int32_t kTileTriangles = 10240;
 constexpr int32_t kRecordTriangles = 65536;
 constexpr int64_t kTileLanes = 500000;
-__host__ __device__ __forceinline__ int64_t path_lanes(const RenderArgs &a) { return ((int64_t)a.Hc * a.Wc) << a.log2L; }
-// the scenes and path lengths that pay (the server's batch kernel, whose grid stays full)
-__host__ __device__ __forceinline__ bool tiled_paths(const RenderArgs &a) { return a.bounces > 1 && a.T <= kTileTriangles; }
+inline int64_t path_lanes(const RenderArgs &a) { return ((int64_t)a.Hc * a.Wc) << a.log2L; }
 // do these arguments run in the small tiles?
 inline bool small_tiles(const RenderArgs &a) { return path_lanes(a) < kTileLanes; }
 // do the samples fill the rounds of a pixel's lanes (35 samples on 32 lanes do not)?
@@ -604,7 +602,7 @@ inline bool full_rounds(const RenderArgs &a) {
 // renders
 inline bool tiled(const RenderArgs &a) {
     const bool middle = path_lanes(a) >= kTileLanes && path_lanes(a) < 4 * kTileLanes;
-    return tiled_paths(a) && !(a.bounces == 2 && middle && full_rounds(a));
+    return a.bounces > 1 && a.T <= kTileTriangles && !(a.bounces == 2 && middle && full_rounds(a));
 }
 // kernels that record every vertex
 inline bool tiled_records(const RenderArgs &a) {
