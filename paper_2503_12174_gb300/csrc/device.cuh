@@ -450,10 +450,14 @@ __device__ __forceinline__ bool tri_isect_wt(const Ray &r, f3 v0, f3 v1, f3 v2, 
     return t > 0.0f && t <= tmax;
 }
 
-// out of line: the rare edge cases stay out of the traversal loop's code
-static __device__ __noinline__ bool tri_isect_wt_call(const Ray &r, f3 v0, f3 v1, f3 v2, float tmax, float &t,
-                                                      float &u, float &v) {
-    return tri_isect_wt(r, v0, v1, v2, tmax, t, u, v);
+// Out of line: the rare edge cases stay out of the traversal loop's code.
+// Returns (t, u, v), t = 0: no hit.  By value: with t, u and v as reference
+// arguments the kernels as compiled kept the barycentrics of a triangle that
+// lost a tie in t, beside the winner's position.
+static __device__ __noinline__ float3 tri_isect_wt_call(const Ray &r, f3 v0, f3 v1, f3 v2, float tmax) {
+    float t, u, v;
+    const bool hit = tri_isect_wt(r, v0, v1, v2, tmax, t, u, v);
+    return hit ? make_float3(t, u, v) : make_float3(0.f, 0.f, 0.f);
 }
 
 // Moller-Trumbore, two-sided, t in (0, tmax].  near_edge reports a miss
@@ -502,7 +506,13 @@ __device__ __forceinline__ bool tri_isect(const Ray &r, f3 v0, f3 v1, f3 v2, flo
 #elif DPCS_WATERTIGHT == 1
     bool near_edge;
     if (tri_isect_mt(r, v0, v1, v2, tmax, t, u, v, near_edge)) return true;
-    return near_edge && tri_isect_wt_call(r, v0, v1, v2, tmax, t, u, v);
+    if (!near_edge) return false;
+    const float3 w = tri_isect_wt_call(r, v0, v1, v2, tmax);
+    if (!(w.x > 0.0f)) return false;
+    t = w.x;
+    u = w.y;
+    v = w.z;
+    return true;
 #else
     bool near_edge;
     return tri_isect_mt(r, v0, v1, v2, tmax, t, u, v, near_edge);

@@ -178,10 +178,7 @@ __device__ __forceinline__ void tree_walk(const RenderArgs &a, const Ray &ray, b
             const float4 B = __ldg(a.tris + 3 * pos + 1);
             const float4 C = __ldg(a.tris + 3 * pos + 2);
             float t, u, v;
-            bool near_edge, wt = false;
-            bool ok = tri_isect_mt(ray, xyz(A), xyz(B), xyz(C), ht, t, u, v, near_edge);
-            if (!ok && near_edge) ok = wt = tri_isect_wt_call(ray, xyz(A), xyz(B), xyz(C), ht, t, u, v);
-            if (ok) {
+            if (tri_isect(ray, xyz(A), xyz(B), xyz(C), ht, t, u, v)) {
                 // ties in t to the lowest original triangle index
                 if (t < ht || (!any && hpos >= 0 && __float_as_int(A.w) < __float_as_int(__ldg(a.tris + 3 * hpos).w))) {
                     hpos = pos;
@@ -189,14 +186,6 @@ __device__ __forceinline__ void tree_walk(const RenderArgs &a, const Ray &ray, b
                     hu = u;
                     hv = v;
                     if (any) room = kStack;
-                } else if (wt) {
-                    // A ray that meets a shared edge exactly (1 path in 1e7)
-                    // ties in the watertight test.  trav_resume as compiled
-                    // keeps the barycentrics of the triangle that loses such a
-                    // tie; the tiles do the same, so that every kernel gives
-                    // the same image.
-                    hu = u;
-                    hv = v;
                 }
             }
             node = room < kStack ? stack[++room] : kDone;
