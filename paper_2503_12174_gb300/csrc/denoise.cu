@@ -97,8 +97,9 @@ __device__ __forceinline__ float ex2(float x) {
 // 8-byte load a feature and packed FP32 operations, half the instructions of
 // one tap at a time.  Pairs start on even columns, so a window row is r pairs
 // and one tap left over at its right (even outputs) or left end, which runs as
-// a pair with itself and a distance term that makes the second weight 0; it
-// loads nothing outside the window, whose NaN would otherwise count.  The
+// a pair of its guide with itself, a distance term that makes the second weight
+// 0 and no image beside it (0 times an infinite one would be NaN); it loads
+// nothing outside the window, whose NaN would otherwise count.  The
 // widths carry log2(e), and a weight is one ex2 of the whole exponent
 // (against 64 bits the filter's error is 1.8e-7, with expf it was 2.7e-7).
 // 1024 x 1024 at r = 5, forward / adjoint, one tap at a time -> pairs: 0.193 /
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(kTile *kTile / kStrip)
         {  // the tap left over, at the window's right or left end
             const int at = par ? 0 : 2 * r, gx = x0 + (int)threadIdx.x + at;
 #pragma unroll
-            for (int n = 0; n < kFeat; ++n) f[n] = pair(row[n * N + at], row[n * N + at]);
+            for (int n = 0; n < kFeat; ++n) f[n] = pair(row[n * N + at], n < 7 ? row[n * N + at] : 0.0f);
             taps(f, pair(gx < 0 || gx >= W ? -kFar : (float)(r * r) * nks, -kFar));
         }
     }
