@@ -144,7 +144,7 @@ dpcs_status ensure(dpcs_ctx *c, Buf &b, size_t bytes, const char *what) {
 // calls cannot do without), when it would have to be allocated while the
 // stream is being captured, or when the device has no room.  A smaller buffer
 // is kept until the context goes, since a captured graph may hold its address;
-// sizes double, so those come to less than the one in use.
+// sizes at least double, so those come to less than the one in use.
 void *optional_scratch(dpcs_ctx *c, Buf &b, size_t bytes, cudaStream_t st) {
     if (!bytes || c->budget) return nullptr;
     if (b.n >= bytes) return b.p;
@@ -153,8 +153,7 @@ void *optional_scratch(dpcs_ctx *c, Buf &b, size_t bytes, cudaStream_t st) {
         cudaGetLastError();
         return nullptr;
     }
-    size_t n = size_t(1) << 20;
-    while (n < bytes) n <<= 1;
+    const size_t n = bytes > 2 * b.n ? bytes : 2 * b.n;
     void *p = nullptr;
     if (cudaMalloc(&p, n) != cudaSuccess) {
         cudaGetLastError();

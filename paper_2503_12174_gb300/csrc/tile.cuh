@@ -612,10 +612,16 @@ inline size_t tile_block_bytes(const RenderArgs &a, bool replay, int S, int word
     return (spl * S * ((size_t)words * 4 * a.bounces + 1) + 255) & ~size_t(255);
 }
 
+// blocks of B threads that take the tiles of S lanes from their counter
+inline int64_t tile_blocks(const RenderArgs &a, int B, int S) {
+    const int64_t ntile = (path_lanes(a) + S - 1) / S, most = resident_blocks(B);
+    return ntile < most ? ntile : most;
+}
+
 inline size_t tile_scratch_bytes(const RenderArgs &a, bool replay, int words) {
     if (!tiled_records(a) || a.root == kEmptyRoot) return 0;
-    return small_tiles(a) ? (size_t)resident_blocks(64) * tile_block_bytes(a, replay, 64, words)
-                          : (size_t)resident_blocks(128) * tile_block_bytes(a, replay, 256, words);
+    return small_tiles(a) ? (size_t)tile_blocks(a, 64, 64) * tile_block_bytes(a, replay, 64, words)
+                          : (size_t)tile_blocks(a, 128, 256) * tile_block_bytes(a, replay, 256, words);
 }
 
 struct TileGrid {
@@ -626,9 +632,8 @@ struct TileGrid {
 };
 inline TileGrid tile_grid(const RenderArgs &a, const LossArgs &l, int B, int S, int words) {
     TileGrid g;
-    g.ntile = ((((int64_t)a.Hc * a.Wc) << a.log2L) + S - 1) / S;
-    const int64_t cap = resident_blocks(B);
-    g.grid = (unsigned)(g.ntile < cap ? g.ntile : cap);
+    g.ntile = (path_lanes(a) + S - 1) / S;
+    g.grid = (unsigned)tile_blocks(a, B, S);
     g.per_block = tile_block_bytes(a, l.target == nullptr, S, words);
     g.counter = reinterpret_cast<unsigned long long *>(l.acc + kTileCounter);
     return g;
