@@ -97,10 +97,10 @@ typedef struct dpcs_view {
 } dpcs_view;
 
 /* Create a context on CUDA device `device`; scratch and scenes may use at
- * most `hbm_budget_bytes` (0 = no limit).  Without a limit the adjoint calls
- * also take scratch for path records (up to 1 GB) where it is to be
- * had; with one they do without, to the same results.  *out receives the
- * context. */
+ * most `hbm_budget_bytes` (0 = no limit).  Without a limit the adjoint calls,
+ * and the compensation steps of the context's servers, also take scratch for
+ * path records (up to 1 GB) where it is to be had; with one they do without, to
+ * the same results.  *out receives the context. */
 dpcs_status dpcs_create(int device, size_t hbm_budget_bytes, dpcs_ctx **out);
 
 /* Free every scene, scratch buffer and the context itself (synchronises). */
@@ -703,7 +703,7 @@ typedef struct dpcs_request {
 typedef struct dpcs_serve_stats {
     int64_t submitted, completed, failed, waiting, active;
     int64_t iterations, launches;
-    size_t memory_used, memory_high_water;
+    size_t memory_used, memory_high_water;  /* device bytes of active requests, path records of compensations included */
 } dpcs_serve_stats;
 
 /* Create a server on ctx's device.  The host buffers of a request must stay

@@ -1568,6 +1568,8 @@ dpcs_status ctx_render_args(dpcs_ctx *c, dpcs_scene scene, const float *albedo, 
 
 int ctx_device(const dpcs_ctx *c) { return c->device; }
 
+bool ctx_has_budget(const dpcs_ctx *c) { return c->budget != 0; }
+
 void ctx_add_launches(dpcs_ctx *c, int n) {
     if (n > 0) c->launches += (uint64_t)n;
 }

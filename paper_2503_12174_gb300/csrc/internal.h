@@ -221,6 +221,7 @@ dpcs_status ctx_render_args(dpcs_ctx *c, dpcs_scene scene, const float *albedo, 
                             int32_t Wt, const float *Ip, const dpcs_view *view, const dpcs_params *params,
                             int32_t spp, int32_t bounces, uint64_t seed, RenderArgs &a);
 int ctx_device(const dpcs_ctx *c);
+bool ctx_has_budget(const dpcs_ctx *c);
 void ctx_add_launches(dpcs_ctx *c, int n);
 dpcs_status ctx_fail(dpcs_ctx *c, dpcs_status code, const char *msg);
 

@@ -76,6 +76,7 @@ struct Req {
     int64_t npix = 0, next_pix = 0, pix_done = 0;
     int steps_issued = 0, steps_done = 0;
     bool copy_queued = false;
+    bool uses_recs = false;
     cudaEvent_t done_ev = nullptr;
     int64_t remaining_samples() const {
         return r.kind == DPCS_REQ_RELIGHT ? (npix - next_pix) * (int64_t)r.spp
@@ -111,9 +112,11 @@ struct dpcs_server {
     size_t used = 0, high_water = 0;
     int64_t submitted = 0, completed = 0, failed = 0, iterations = 0, launches = 0;
     int grid[2] = {1, 1};  // of the batch kernel in lanes and in tiles
-    void *recs = nullptr;  // path records of the compensation steps' tiles (steps run one after another)
+    // path records of the compensation steps' tiles (steps run one after
+    // another), held while compensation requests are active
+    void *recs = nullptr;
     size_t recs_bytes = 0;
-    std::vector<void *> retired;  // smaller ones that queued steps may still use
+    int recs_users = 0;
 };
 
 namespace {
@@ -145,6 +148,43 @@ dpcs_view request_view(const ServeScene &sc, const dpcs_request &r) {
     v.Hc = r.Hc;
     v.Wc = r.Wc;
     return v;
+}
+
+// one compensation step in a single trace of its paths (k_render_grad):
+// render, L2 loss, adjoint, then PRF adjoint, Adam and Ep for the next step
+bool comp_step_fuses(const Req *q) {
+    const int L = 1 << q->args.log2L;
+    const int spl = (q->args.spp + L - 1) / L;
+    return spl <= kFusedSamples && spl * q->args.bounces <= kFusedRecs;
+}
+
+size_t step_scratch_bytes(const Req *q) { return grad_scratch_bytes(q->args, !comp_step_fuses(q), kRecWordsHost); }
+
+// Records for the tiled steps of a compensation request that comes in, from
+// the request pool in stream order, so that the larger buffer replaces one
+// that queued steps still use.  None (the steps run in lanes) when they have no
+// tile kernel, when the server or its context has a memory budget, which is
+// left for what requests cannot do without, or when there is no room.
+void take_recs(dpcs_server *s, Req *q) {
+    const size_t bytes = step_scratch_bytes(q);
+    if (!bytes || s->cfg.hbm_budget_bytes || ctx_has_budget(s->ctx)) return;
+    q->uses_recs = true;
+    ++s->recs_users;
+    if (s->recs_bytes >= bytes) return;
+    void *p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, bytes, s->pool, s->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (s->recs) cudaFreeAsync(s->recs, s->stream);
+    s->used += bytes - s->recs_bytes;
+    s->high_water = std::max(s->high_water, s->used);
+    s->recs = p;
+    s->recs_bytes = bytes;
+}
+
+void *step_scratch(const dpcs_server *s, const Req *q) {
+    return q->uses_recs && s->recs_bytes >= step_scratch_bytes(q) ? s->recs : nullptr;
 }
 
 dpcs_status admit(dpcs_server *s, Req *q) {
@@ -195,29 +235,10 @@ dpcs_status admit(dpcs_server *s, Req *q) {
     q->args.Ec = q->Ec;
     q->args.counters = nullptr;
     q->npix = (int64_t)npix;
+    if (r.kind == DPCS_REQ_COMPENSATE) take_recs(s, q);
     s->launches += launch_prf(q->Ip, (int64_t)np, sc.params.gamma_p, sc.params.gain_p, q->Ep4, s->stream);
     q->state = DPCS_REQ_ACTIVE;
     return DPCS_OK;
-}
-
-// Records for a tiled compensation step; null (the lanes kernels) when the
-// arguments have no tile kernel, the server has a memory budget, which is left
-// for its requests, or there is no room.
-void *step_scratch(dpcs_server *s, const RenderArgs &a, bool replay) {
-    const size_t bytes = grad_scratch_bytes(a, replay, kRecWordsHost);
-    if (!bytes || s->cfg.hbm_budget_bytes) return nullptr;
-    if (s->recs_bytes >= bytes) return s->recs;
-    size_t n = size_t(1) << 20;
-    while (n < bytes) n <<= 1;
-    void *p = nullptr;
-    if (cudaMalloc(&p, n) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (s->recs) s->retired.push_back(s->recs);
-    s->recs = p;
-    s->recs_bytes = n;
-    return p;
 }
 
 // a step's accumulators cleared, and Eq. 1's adjoint into G (with the loss of
@@ -257,19 +278,11 @@ int enqueue_comp_backward(dpcs_server *s, Req *q) {
     a.gE = q->gE;
     a.dEp = q->dEp4;
     a.dtex = nullptr;  // only Ip is optimised
-    n += launch_replay(a, q->acc, step_scratch(s, a, true), st);
+    n += launch_replay(a, q->acc, step_scratch(s, q), st);
     n += finish_step(q, sc, np, nullptr, st);
     n += launch_adam(q->Ip, q->G, q->M, q->V, np * 3, q->r.lr, 0.9f, 0.999f, 1e-8f, q->steps_issued, 0.0f, 1.0f, st);
     n += launch_prf(q->Ip, np, sc.params.gamma_p, sc.params.gain_p, q->Ep4, st);
     return n;
-}
-
-// one compensation step in a single trace of its paths (k_render_grad):
-// render, L2 loss, adjoint, then PRF adjoint, Adam and Ep for the next step
-bool comp_step_fuses(const Req *q) {
-    const int L = 1 << q->args.log2L;
-    const int spl = (q->args.spp + L - 1) / L;
-    return spl <= kFusedSamples && spl * q->args.bounces <= kFusedRecs;
 }
 
 int enqueue_comp_step_fused(dpcs_server *s, Req *q) {
@@ -282,7 +295,7 @@ int enqueue_comp_step_fused(dpcs_server *s, Req *q) {
     a.dEp = q->dEp4;
     a.dtex = nullptr;  // only Ip is optimised
     const LossArgs l{q->target, 1.0f, 0, q->acc};
-    n += launch_render_grad(a, l, step_scratch(s, a, false), st);
+    n += launch_render_grad(a, l, step_scratch(s, q), st);
     n += finish_step(q, sc, np, q->loss, st);
     n += launch_adam(q->Ip, q->G, q->M, q->V, np * 3, q->r.lr, 0.9f, 0.999f, 1e-8f, q->steps_issued, 0.0f, 1.0f, st);
     n += launch_prf(q->Ip, np, sc.params.gamma_p, sc.params.gain_p, q->Ep4, st);
@@ -294,6 +307,15 @@ void release(dpcs_server *s, Req *q) {
         cudaFreeAsync(q->mem, s->stream);
         q->mem = nullptr;
         s->used -= q->bytes;
+    }
+    if (q->uses_recs) {
+        q->uses_recs = false;
+        if (--s->recs_users == 0 && s->recs) {
+            cudaFreeAsync(s->recs, s->stream);
+            s->used -= s->recs_bytes;
+            s->recs = nullptr;
+            s->recs_bytes = 0;
+        }
     }
     if (q->done_ev) {
         cudaEventDestroy(q->done_ev);
@@ -623,8 +645,6 @@ dpcs_status dpcs_serve_destroy(dpcs_server *s) {
         if (sc.tex4) cudaFree(sc.tex4);
     for (Batch &b : s->batches) free_batch_bufs(b);
     cudaStreamSynchronize(s->stream);
-    if (s->recs) cudaFree(s->recs);
-    for (void *p : s->retired) cudaFree(p);
     cudaStreamDestroy(s->stream);
     cudaMemPoolDestroy(s->pool);
     delete s;
