@@ -562,6 +562,7 @@ __device__ __forceinline__ void ldg8(const float4 *p, float4 &a, float4 &b) {
         : "l"(p));
 }
 
+#if DPCS_SLAB_FMA
 // slab() with the two planes of an axis in one packed FMA (the
 // same roundings; a node lists them side by side)
 __device__ __forceinline__ bool slab2(u64 x, u64 y, u64 z, u64 ix, u64 iy, u64 iz, u64 ox, u64 oy, u64 oz, float err,
@@ -575,6 +576,7 @@ __device__ __forceinline__ bool slab2(u64 x, u64 y, u64 z, u64 ix, u64 iy, u64 i
     tnear = tn;
     return tn <= fmaf(tf, 1.0000004f, err);
 }
+#endif
 
 struct Trav {
     int node, sp, visits;
@@ -593,12 +595,10 @@ __device__ __forceinline__ void trav_begin(Trav &st, int32_t root, float tmax, b
 }
 
 // kPacked: a node in two loads, its slabs in packed FMAs (the same results):
-// 200k-triangle heightfield, 1024 x 1024 x 16 spp, 8.24 -> 8.09 ms.  Not in
-// the server's batch kernel, whose single-bounce requests share it with the
-// tiles: 11.61 ms packed, 11.37 plain (16 mixed requests); nor where the
-// compiler chooses the fusions, which it would choose anew, nor in the
+// 200k-triangle heightfield, 1024 x 1024 x 16 spp, 8.24 -> 8.09 ms.  Not where
+// the compiler chooses the fusions, which it would choose anew, nor in the
 // wavefront passes (not measured).
-#ifdef DPCS_FUSION_BY_COMPILER
+#if defined(DPCS_FUSION_BY_COMPILER) || !DPCS_SLAB_FMA
 constexpr bool kPackedSlabs = false;
 #else
 constexpr bool kPackedSlabs = true;
@@ -636,6 +636,7 @@ __device__ __forceinline__ bool trav_resume(const float4 *__restrict__ nodes, co
             float tl, tr;
             bool hl, hr;
             if constexpr (kPacked) {
+#if DPCS_SLAB_FMA
                 const float4 *nd = nodes + 4 * (size_t)(uint32_t)node;
                 ldg8(nd, n0, n1);
                 ldg8(nd + 2, n2, n3);
@@ -644,6 +645,7 @@ __device__ __forceinline__ bool trav_resume(const float4 *__restrict__ nodes, co
                           oz = pk2(-ray.oinv.z, -ray.oinv.z);
                 hl = slab2(pk2(n0.x, n0.y), pk2(n0.z, n0.w), pk2(n2.x, n2.y), ix, iy, iz, ox, oy, oz, ray.err, st.h.t, tl);
                 hr = slab2(pk2(n1.x, n1.y), pk2(n1.z, n1.w), pk2(n2.z, n2.w), ix, iy, iz, ox, oy, oz, ray.err, st.h.t, tr);
+#endif
             } else {
                 n0 = __ldg(nodes + 4 * node + 0);
                 n1 = __ldg(nodes + 4 * node + 1);

@@ -148,7 +148,6 @@ __global__ void __launch_bounds__(256) k_inputs(const InputArgs q, unsigned bp) 
 // and lane 0 writes Ec and Ic.  Every lane of the warp must call this (the
 // reduction shuffles over the full warp); lanes with valid == false only
 // take part in the shuffles.
-template <bool kPacked>
 __device__ __forceinline__ void render_lanes(const RenderArgs &a, int64_t pix, int sl, bool valid) {
     const int L = 1 << a.log2L;
     f3 sum = mk3(0.f, 0.f, 0.f);
@@ -192,7 +191,7 @@ __device__ __forceinline__ void render_lanes(const RenderArgs &a, int64_t pix, i
                 trav_begin(st, a.root, shadow ? tmax : INFINITY, shadow);
                 pending = true;
             }
-            if (!trav_resume<kPacked>(a.nodes, a.tris, nulls ? kEmptyRoot : a.root, a.T, ray, st, stack, a.status, cnt, min(DPCS_YIELD_MIN, alive), a.visit_cap))
+            if (!trav_resume(a.nodes, a.tris, nulls ? kEmptyRoot : a.root, a.T, ray, st, stack, a.status, cnt, min(DPCS_YIELD_MIN, alive), a.visit_cap))
                 continue;
             pending = false;
             const bool hit = st.h.pos >= 0;
@@ -278,7 +277,7 @@ template <int kMinBlocks>
 __global__ void __launch_bounds__(kRenderBlock, kMinBlocks) k_render(const RenderArgs a) {
     const int64_t gt = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t pix = gt >> a.log2L;
-    render_lanes<true>(a, pix, (int)(gt & ((1 << a.log2L) - 1)), pix < (int64_t)a.Hc * a.Wc);
+    render_lanes(a, pix, (int)(gt & ((1 << a.log2L) - 1)), pix < (int64_t)a.Hc * a.Wc);
 }
 
 // Forward render over block tiles (tile.cuh): the image of render_lanes bit
@@ -340,7 +339,7 @@ __global__ void __launch_bounds__(kRenderBlock, DPCS_BATCH_MINB)
         } else {
             const int64_t lt = (vb - sg.vb_begin) * kRenderBlock + threadIdx.x;  // thread index within the segment
             const int64_t lp = lt >> sa.log2L;
-            render_lanes<true>(sa, sg.pix_begin + lp, (int)(lt & ((1 << sa.log2L) - 1)), lp < sg.npix);
+            render_lanes(sa, sg.pix_begin + lp, (int)(lt & ((1 << sa.log2L) - 1)), lp < sg.npix);
         }
         __syncthreads();
     }

@@ -84,8 +84,8 @@ __device__ __forceinline__ int dir_bin(f3 d) {
 // ---------------------------------------------------------------------------
 // traversal
 // ---------------------------------------------------------------------------
-// One step down the tree: 50 instructions against the 54 of trav_resume's
-// (a chain of nodes with one child hit each).  The stack grows down from
+// One step down the tree: 50 instructions against the 54 of trav_resume's with
+// plain slabs (a chain of nodes with one child hit each).  The stack grows down from
 // stack[kStack]; its last place, which no tree the library builds needs, leaves
 // room = -1, and the caller ends the ray.
 __device__ __forceinline__ void tree_node(const RenderArgs &a, const Ray &ray, float ht, int &node, int &room, int *stack,
@@ -97,12 +97,17 @@ __device__ __forceinline__ void tree_node(const RenderArgs &a, const Ray &ray, f
     float4 n0, n1, n2, n3;
     ldg8(nd, n0, n1);
     ldg8(nd + 2, n2, n3);
+    float tl, tr;
+#if DPCS_SLAB_FMA
     const u64 ix = pk2(ray.inv.x, ray.inv.x), iy = pk2(ray.inv.y, ray.inv.y), iz = pk2(ray.inv.z, ray.inv.z);
     const u64 ox = pk2(-ray.oinv.x, -ray.oinv.x), oy = pk2(-ray.oinv.y, -ray.oinv.y),
               oz = pk2(-ray.oinv.z, -ray.oinv.z);
-    float tl, tr;
     const bool hl = slab2(pk2(n0.x, n0.y), pk2(n0.z, n0.w), pk2(n2.x, n2.y), ix, iy, iz, ox, oy, oz, ray.err, ht, tl);
     const bool hr = slab2(pk2(n1.x, n1.y), pk2(n1.z, n1.w), pk2(n2.z, n2.w), ix, iy, iz, ox, oy, oz, ray.err, ht, tr);
+#else
+    const bool hl = slab(ray, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, ht, tl);
+    const bool hr = slab(ray, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, ht, tr);
+#endif
     const int cl = __float_as_int(n3.x), cr = __float_as_int(n3.y);
     const bool lf = tl <= tr;
     if (hl | hr) {
