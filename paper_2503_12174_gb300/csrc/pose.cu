@@ -394,7 +394,8 @@ __device__ void block_partial(const float acc[6], double *out) {
 }
 
 // Interior term, one item per camera sample (pixel i / spp, sample i % spp),
-// the sample's path as the render traces it.
+// the sample's path as the render traces it (up to the fusions that the
+// compiler chooses in this file).
 template <bool kPbr>
 __global__ void __launch_bounds__(kPoseBlock, DPCS_POSE_MINB) k_pose_interior(const RenderArgs a, const PoseArgs p) {
     float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};

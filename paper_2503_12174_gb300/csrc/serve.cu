@@ -17,7 +17,8 @@
 //      with no quanta; or (quanta-deadline policy) the quanta first, then
 //      the rest in order of deadline;
 //   4. enqueue on the server stream: the batch descriptors, one persistent
-//      k_render_batch launch over the relighting pixels, each compensation
+//      k_render_batch launch over the relighting pixels that run in lanes and
+//      one over those that run in tiles, each compensation
 //      request's step: render, loss and path adjoint in one trace
 //      (k_render_grad, or render + loss + replay when its records would not
 //      fit), then Adam and PRF; the host copies of requests that finish in

@@ -14,9 +14,9 @@
 // their warp, and lanes whose path has ended wait for the others' (13.5 of
 // 32 lanes active).  Phases compact both: a warp gets 32 live rays, neighbours
 // in direction, so their walks down the tree have similar lengths, and 32
-// hits to shade (21 of 32 lanes active, 0.82 G warp instructions instead of
-// 1.19 G; corner 256 x 256 at 64 spp, 3 bounces: 1.367 -> 1.047 ms on GB300;
-// 640 x 360 at 35 spp, whose second round has 3 lanes of 32: 4.12 -> 2.52 ms).
+// hits to shade (22 of 32 lanes active, 0.83 G warp instructions instead of
+// 1.19 G; corner 256 x 256 at 64 spp, 3 bounces: 1.367 -> 1.048 ms on GB300;
+// 640 x 360 at 35 spp, whose second round has 3 lanes of 32: 4.12 -> 2.55 ms).
 // Of that the direction sort gives 5 %.  Tiles of one or three slots a thread
 // were 15 and 9 % slower than of two; letting a slot take its next sample as
 // soon as its path ended mixed bounces in the phases and was 9 % slower.
@@ -126,12 +126,13 @@ __device__ __forceinline__ void tree_node(const RenderArgs &a, const Ray &ray, f
 // A lane takes up to kBurst steps down the tree, then the warp meets and the
 // lanes at a leaf test it.  Without the limit all lanes wait for the one that
 // is longest on its way to a leaf, which curved surfaces, whose boxes overlap,
-// make long: a closed sphere of 1,280 triangles (384 x 384 x 16 spp, 4 bounces)
-// took 3.90 ms against 3.14 of the lanes kernel of its day and takes 3.05, an
-// open half sphere 0.97 -> 0.79 of that kernel's time.  Bursts of 1 / 2 / 3 / 4 /
-// 6: 1.09 / 0.98 / 0.97 / 0.97 / 0.99 of it on the sphere, 0.82 / 0.77 / 0.76 /
-// 0.75 / 0.75 on the corner, which gains nothing from them.  Unrolled, renders
-// are another 2 to 4 % faster and the kernels with a sweep 2 to 5 % slower.
+// make long.  384 x 384 x 16 spp, 4 bounces, in parts of the lanes kernel's time
+// before there were tiles, without a limit and in bursts of 1 / 2 / 3 / 4 / 6:
+// closed sphere of 1,280 triangles 1.24, 1.09 / 0.98 / 0.97 / 0.97 / 0.99; half
+// sphere of 1,600 0.97, 0.87 / 0.80 / 0.80 / 0.80 / 0.83; corner 0.73, 0.82 / 0.77 /
+// 0.76 / 0.75 / 0.75, whose flat walls need no limit.  (With the triangle test's
+// present form bursts of 4 take 0.94, 0.78 and 0.73.)  Unrolled, renders are 2 to
+// 4 % faster, the kernels that record 1 to 5 % slower.
 //
 // As in trav_resume every step, node or leaf, counts towards the visit cap: a
 // ray that would take one more reports it and ends as a miss, so a walk ends
@@ -496,9 +497,12 @@ __device__ __forceinline__ void tile_image(const RenderArgs &a, Core &core, Tile
 
 // The one-trace step (l.target set) or the replay (l.target null: a.gE holds
 // dLoss/dEc) over block tiles.  Persistent: a block takes tiles from a counter
-// and keeps its records (`words` 16-byte chunks a vertex) in its own part of
-// `scratch`, small enough in all to stay in L2: 512 x 512 at 16 spp, gradient
-// of Ip, 2.10 -> 1.50 ms.  sweep(k, slot, gb) sweeps the slot's path of round k.
+// and keeps its records (`chunks` 16-byte chunks a vertex) in its own part of
+// `scratch`.  The gain over the lanes kernels is the compaction's, and that a
+// record is written once to its place where those spill it to local memory: 512
+// x 512 at 16 spp, gradient of Ip, 2.07 -> 1.50 ms.  The records of the blocks
+// in flight (90 MB at three vertices a lane, 360 at most) do not stay in L2:
+// nearly every byte goes to DRAM and most come back.  sweep(k, slot, gb) sweeps the slot's path of round k.
 template <int B, int S, class Core, class Sweep>
 __device__ __forceinline__ void tile_adjoint(const RenderArgs &a, Core &core, Tile<S> &P, const LossArgs &l, char *scratch,
                                              size_t per_block, int64_t ntile, unsigned long long *counter, int chunks,
@@ -561,27 +565,30 @@ __device__ __forceinline__ void tile_adjoint(const RenderArgs &a, Core &core, Ti
 // dispatch
 // ---------------------------------------------------------------------------
 // Where the tiles pay (GB300; in parts of the time that the lanes kernels took
-// before there were tiles, which their packed form takes 0.87 to 0.97 of).
+// before there were tiles, of which today's take 0.85 to 0.98).
 //
 // Paths of one bounce have nothing to compact (plane 512 x 512 at 16 spp 206 /
 // 230 us).  With two there is little, and images of 0.5 to 2 M lanes, whose last
-// wave of large tiles is long, take 0.94 to 1.06 (corner, heightfields, rooms,
-// spheres) where every round of samples is full: lanes there.  (Samples that
-// leave part of the last round's lanes idle cost tiles nothing: 0.77 of the
-// corner with 11 samples on 8 lanes, 1.3 M.)  Longer paths, 2.4 M lanes, 4 bounces: corner walls of
-// 1,026 / 8,226 triangles 0.74 / 0.76, a room of 2,352 / 8,112 0.92 / 0.89, a half
-// sphere 0.80, closed spheres of 1,280 / 5,120 0.97 / 0.94 (lanes 0.87 / 0.89),
-// heightfields of 2,048 / 7,200 0.93 / 0.93 (0.95 / 0.96).  A tree of some MB no
-// longer sits in the L1 that the tiles' shared memory leaves.
+// wave of large tiles is long, took 0.94 to 1.06 (corner, heightfields, rooms,
+// spheres) where every round of samples is full: lanes there, 0.90 to 0.98.
+// (Samples that leave part of the last round's lanes idle cost tiles nothing:
+// 0.74 of the corner with 35 samples on 32 lanes, 1.2 M.)  Longer paths, 2.4 M
+// lanes, 4 bounces: corner walls of 1,026 / 8,226 triangles 0.73 / 0.75, a room of
+// 2,352 / 8,112 0.90 / 0.88, a half sphere of 1,600 / 6,400 0.78 / 0.79, closed
+// spheres of 1,280 / 5,120 0.94 / 0.92, heightfields of 2,048 / 7,200 0.91 / 0.91.
+// A tree of some MB no longer sits in the L1 that the tiles' shared memory
+// leaves: heightfields of 20,000 and 51,200 in lanes 0.93, in tiles 0.96 and more.
 //
 // Kernels that keep vertex records win for longer, since a tile writes them
-// once: one-trace steps, 2.4 M lanes, 4 bounces 0.70 (corner), 0.82 (20,000-
-// triangle heightfield, lanes 0.95), 0.98 (20,480-triangle sphere, 0.91).  Not in
-// small images, where the large trees' steps took 1.04 to 1.08.
+// once: one-trace steps, 4 bounces, lanes / tiles, at 147 k and 2.4 M lanes:
+// corner 0.88 / 0.87 and 0.92 / 0.70, closed spheres of 1,280 / 20,480 triangles
+// 0.84 / 0.87 and 0.86 / 1.00, 0.85 / 0.88 and 0.89 / 0.96, heightfields of 20,000 /
+// 51,200 0.96 / 1.03 and 0.94 / 0.81, 0.91 / 0.90 and 0.94 / 0.83.
 //
-// Small images want more, smaller tiles: tiles of 64 / 256 lanes take 0.82 /
-// 1.11 (corner), 0.88 / 1.33 (sphere), 0.94 / 1.18 (heightfield of 7,200) at
-// 147 k lanes and 0.93 / 0.81, 0.89 / 1.01, 1.03 / 0.96 at 1 M.
+// Small images want more, smaller tiles: steps in tiles of 64 / 256 lanes take
+// 0.87 / 1.08 (corner), 0.87 / 1.30 (sphere), 0.87 / 1.09 (heightfield of 7,200) at
+// 147 k lanes, 0.91 / 0.82, 0.89 / 0.98, 0.95 / 0.87 at 590 k and 0.92 / 0.73, 0.88 /
+// 1.03, 0.98 / 0.89 at 1 M.
 constexpr int32_t kTileTriangles = 10240;
 constexpr int32_t kRecordTriangles = 65536;
 constexpr int64_t kTileLanes = 500000;
@@ -599,9 +606,7 @@ inline bool tiled(const RenderArgs &a) {
     return a.bounces > 1 && a.T <= kTileTriangles && !(a.bounces == 2 && middle && full_rounds(a));
 }
 // kernels that record every vertex
-inline bool tiled_records(const RenderArgs &a) {
-    return a.bounces > 1 && a.T <= (small_tiles(a) ? kTileTriangles : kRecordTriangles);
-}
+inline bool tiled_records(const RenderArgs &a) { return a.bounces > 1 && a.T <= kRecordTriangles; }
 // blocks of b threads that the GPU holds at once: the persistent grid
 inline int resident_blocks(int b) {
     int dev = 0, sms = 0;

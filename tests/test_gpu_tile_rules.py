@@ -33,7 +33,7 @@ CASES = [
     ("corner", 248, 252, 16, 3), ("corner", 250, 250, 16, 3),      # 999,936 and 1,000,000: the replay
     ("sphere", 250, 250, 16, 4), ("sphere", 31, 33, 5, 8),
     (72, 125, 250, 16, 3), (73, 125, 250, 16, 3),                  # 10,082 and 10,368 triangles
-    (101, 124, 252, 16, 3), (101, 125, 250, 16, 3),                # 20,000: records by the lanes
+    (101, 124, 252, 16, 3), (101, 125, 250, 16, 3),                # 20,000: renders in lanes, records in tiles
     ("corner", 125, 250, 17, 2), ("corner", 250, 250, 11, 2), ("corner", 40, 50, 3, 4),  # rounds of samples not full
     (73, 41, 43, 16, 1), (28, 250, 250, 16, 3), (29, 250, 250, 16, 3),  # one bounce; 1,458 and 1,568: the replay
 ]
