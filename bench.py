@@ -56,19 +56,19 @@ L2_FLUSH_BYTES = 256 << 20
 # ncu capture of the same command.  It holds only for the kernel sources it
 # was measured on; once they change, the roofline's traffic is reported as
 # null until a new capture is taken.
-RENDER_TRAFFIC = {"bytes": 12837888, "sources_sha256": "f56d3aaeccd4791c6a6d2ed6e8a153af4e7a39b8b60a3bed4b7664d4b0a89273"}
+RENDER_TRAFFIC = {"bytes": 12257536, "sources_sha256": "4e9f607d0dba4f26e66a3998b7398ccff9d34e38aa9a607548ee700829c3e33c"}
 # Warp instructions one k_render_tile launch of the forward workload issues, and
 # the active lanes per instruction, from the same ncu capture
 # (smsp__inst_executed.sum, smsp__thread_inst_executed_per_inst_executed);
 # reported while the kernel sources keep this hash.
-RENDER_ISSUE = {"warp_instructions": 813127652, "lanes_per_instruction": 21.23,
-                "sources_sha256": "f56d3aaeccd4791c6a6d2ed6e8a153af4e7a39b8b60a3bed4b7664d4b0a89273"}
+RENDER_ISSUE = {"warp_instructions": 831512703, "lanes_per_instruction": 21.58,
+                "sources_sha256": "4e9f607d0dba4f26e66a3998b7398ccff9d34e38aa9a607548ee700829c3e33c"}
 # The same two figures for one k_grad_tile launch of the compensation step
 # with every gradient requested.
-FWD_BWD_TRAFFIC = {"bytes": 1418324480,
-                   "sources_sha256": "f56d3aaeccd4791c6a6d2ed6e8a153af4e7a39b8b60a3bed4b7664d4b0a89273"}
-FWD_BWD_ISSUE = {"warp_instructions": 1046747543, "lanes_per_instruction": 21.94,
-                 "sources_sha256": "f56d3aaeccd4791c6a6d2ed6e8a153af4e7a39b8b60a3bed4b7664d4b0a89273"}
+FWD_BWD_TRAFFIC = {"bytes": 1367145984,
+                   "sources_sha256": "4e9f607d0dba4f26e66a3998b7398ccff9d34e38aa9a607548ee700829c3e33c"}
+FWD_BWD_ISSUE = {"warp_instructions": 1074521911, "lanes_per_instruction": 22.16,
+                 "sources_sha256": "4e9f607d0dba4f26e66a3998b7398ccff9d34e38aa9a607548ee700829c3e33c"}
 # the kernels' sources and the tree builder (its topology sets the node visits)
 KERNEL_SOURCES = ("paper_2503_12174_gb300/csrc/render.cu", "paper_2503_12174_gb300/csrc/tile.cuh",
                   "paper_2503_12174_gb300/csrc/device.cuh", "paper_2503_12174_gb300/csrc/internal.h",
